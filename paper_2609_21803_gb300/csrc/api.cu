@@ -242,6 +242,25 @@ comet_status check_instances(const comet_instance_desc* inst, int32_t n_instance
 
 namespace comet {
 
+// Shape of a pushing launch of n TOs.  A CTA's warps start every trip of the
+// solver together (`in_step`) so that they share instruction fetches, which
+// pays once the SMs are full.  A launch that leaves a quarter of the resident
+// warps idle is bound by its slowest solves instead: there nobody waits for a
+// CTA mate, and long TOs run one to a CTA, which spreads them over all SMs.
+// Measured: 500 TOs at N = 80 7.1 ms one to a CTA, 7.5 four to a CTA out of
+// step, 9.3 in step; 1,400 (9.2 per SM) 11.3 against 12.0 in step; 1,824 (12
+// per SM, the resident limit) 12.6 against 12.4; 4,000 20.4 against 18.6.
+// At N = 16 (one pass of the stage loops) 144 TOs take 2.11 ms four to a
+// CTA and 2.13 one to a CTA.
+struct LaunchShape {
+    int wpb, in_step;
+};
+static LaunchShape launch_shape(int num_sms, int blocks_per_sm, int warps_per_block, int Nmax, int64_t n) {
+    const int64_t resident = (int64_t)num_sms * blocks_per_sm * warps_per_block;
+    if (4 * n > 3 * resident) return {warps_per_block, 1};
+    return {Nmax > 32 ? 1 : warps_per_block, 0};
+}
+
 static int64_t resident_warps(const comet_problem* p, int64_t n) {
     // bimanual: one CTA per TO, the workspace unit is a CTA
     if (p->task == COMET_TASK_BIMANUAL)
@@ -249,8 +268,8 @@ static int64_t resident_warps(const comet_problem* p, int64_t n) {
     // resident warps: every SM filled, never more warps than TOs; the grid is
     // whole CTAs and any warp may pick any TO, so the workspace covers them all
     const int64_t resident = (int64_t)p->num_sms * p->blocks_per_sm * p->warps_per_block;
-    return ((std::min<int64_t>(resident, std::max<int64_t>(n, 1)) + p->warps_per_block - 1) / p->warps_per_block) *
-           p->warps_per_block;
+    const int wpb = launch_shape(p->num_sms, p->blocks_per_sm, p->warps_per_block, p->Nmax, n).wpb;
+    return ((std::min<int64_t>(resident, std::max<int64_t>(n, 1)) + wpb - 1) / wpb) * wpb;
 }
 
 // floats of workspace per unit (a warp for pushing, a CTA for bimanual)
@@ -329,10 +348,13 @@ comet_status launch_eval_device(comet_problem* p, const comet_mode_seq* d_seqs, 
     a.stall_staging = p->stall_staging;
     a.sp = make_params(p->opts, max_iters);
     for (const comet_instance_desc& d : p->inst) a.sp.free_motion |= d.task == COMET_TASK_PUSHER_SLIDER && d.n_modes == 13;
-    if (p->task == COMET_TASK_BIMANUAL)
+    if (p->task == COMET_TASK_BIMANUAL) {
         CUDA_TRY(launch_bimanual(a, (int)warps, s), "bimanual evaluator launch");
-    else
-        CUDA_TRY(launch_eval(a, (int)warps, p->warps_per_block, s), "evaluator launch");
+    } else {
+        const LaunchShape sh = launch_shape(p->num_sms, p->blocks_per_sm, p->warps_per_block, p->Nmax, n_max);
+        a.in_step = sh.in_step;
+        CUDA_TRY(launch_eval(a, (int)warps, sh.wpb, s), "evaluator launch");
+    }
     return COMET_OK;
 }
 
@@ -625,6 +647,8 @@ comet_status comet_eval_modes_timed(comet_problem* p, const comet_timing_opts* t
     const int bps = comet::timing_blocks_per_sm(wpb, p->Nmax);
     if (bps < 1) return fail(COMET_ERR_CUDA, "timing kernel: no resident block");
     const int64_t resident = (int64_t)p->num_sms * bps * wpb;
+    const comet::LaunchShape sh = comet::launch_shape(p->num_sms, bps, wpb, p->Nmax, n);  // as for the fixed step
+    wpb = sh.wpb;
     const int64_t warps = ((std::min<int64_t>(resident, n) + wpb - 1) / wpb) * wpb;
     const int64_t ws_floats = comet::timing_ws_per_warp_floats(p->Nmax) * warps;
     if (p->tws_floats < ws_floats) {
@@ -637,8 +661,16 @@ comet_status comet_eval_modes_timed(comet_problem* p, const comet_timing_opts* t
     cudaStream_t s = p->stream;
     CUDA_TRY(cudaMemsetAsync(p->d_queue, 0, sizeof(unsigned int), s), "queue reset");
     CUDA_TRY(cudaMemsetAsync(p->d_bad, 0, sizeof(int), s), "flag reset");
+    // mixed interval counts: longest first, which also gives a CTA's warps
+    // TOs of about the same length
+    const bool lpt = p->hetero && p->perm_cap >= n && n > 1;
+    if (lpt)
+        CUDA_TRY(comet::launch_lpt_order(mode_seqs, n, nullptr, p->d_inst, (int)p->inst.size(), p->d_lpt, p->d_perm, s),
+                 "longest-first order");
     comet::TimingArgs a;
     memset(&a, 0, sizeof(a));
+    a.e.perm = lpt ? p->d_perm : nullptr;
+    a.e.in_step = sh.in_step;
     a.e.inst = p->d_inst;
     a.e.n_inst = (int)p->inst.size();
     a.e.seqs = mode_seqs;

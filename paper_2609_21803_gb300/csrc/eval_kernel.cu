@@ -62,6 +62,18 @@ __device__ __forceinline__ double warp_max_d(double v) {
     return v;
 }
 
+// The CTA's barrier if `on` (uniform over the launch), as one predicated
+// instruction.
+__device__ __forceinline__ void cta_in_step(int on) {
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        "setp.ne.s32 p, %0, 0;\n"
+        "@p bar.sync 0;\n"
+        "}\n" ::"r"(on)
+        : "memory");
+}
+
 // error-free sum a + b = s + e (Knuth two-sum)
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
     s = a + b;
@@ -1395,6 +1407,19 @@ __device__ void refine_step(Ctx& C, float beta, float rho, bool curvature) {
 // most of the local-memory spills a 128-register cap costs (12 warps per SM
 // at 168 registers were 7 % faster than 16 at 128 on the 4-segment
 // enumeration, with DRAM write-back 7 times lower).
+// The CTA's warps start phase A of every trip at one barrier.  The hot loop
+// is about 90 KB of straight-line code against an instruction cache of about
+// 32 KB per SM quarter (measured: straight-line FMAs issue at full rate up to
+// 24-32 KB, at a third of it from 48 KB on; 12 warps per SM at different
+// places of a 96-128 KB loop reach 0.33-0.38 issues per cycle and quarter,
+// 12 warps in step 0.91, as a fetched line then serves all of them).  In step
+// at the trip's start, the warps stay close enough to share most fetches:
+// 20,736 TOs at N = 80 took 76.6 ms without and 63.5 ms with the barrier, with
+// equal results (no_instruction stalls per issue 3.2 -> 0.75); a second
+// barrier before phase B gained nothing, and 2 or 12 warps per CTA took 12 %
+// longer than 4.  Launches that do not fill the SMs skip it (in_step = 0).
+// A warp that runs out of TOs leaves; a barrier waits only for warps that
+// have not left.
 // kUnr: stages per trip of the stage-parallel loops (phases A, C and D
 // unrolled 1 or 2 times; the autotuner picks it with the launch shape).
 template <bool kRefine, bool kFree, int kUnr = 1>
@@ -1539,6 +1564,7 @@ __global__ void __launch_bounds__(128, 3) eval_kernel(EvalArgs A) {
             bool model_curv = curv, fac = false, done = false;
             float beta_old = beta;
             for (;;) {
+                cta_in_step(A.in_step);  // start phase A together (see the kernel's comment)
                 const Measures m = phase_a<kFree, kUnr>(C, beta, rho, model_curv, true, trip == kUpdate, beta_old);
                 if (trip == kMeasure) {
                     if (!m.finite) {

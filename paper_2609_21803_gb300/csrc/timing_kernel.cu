@@ -87,6 +87,18 @@ __device__ __forceinline__ double twarp_max_d(double v) {
     return v;
 }
 
+// the CTA's barrier if `on` (uniform over the launch), as one predicated
+// instruction
+__device__ __forceinline__ void cta_in_step(int on) {
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        "setp.ne.s32 p, %0, 0;\n"
+        "@p bar.sync 0;\n"
+        "}\n" ::"r"(on)
+        : "memory");
+}
+
 // error-free sum a + b = s + e (Knuth two-sum)
 __device__ __forceinline__ void two_sum_t(float a, float b, float& s, float& e) {
     s = a + b;
@@ -1237,6 +1249,9 @@ __device__ TCert tcertify(const TCtx& C, float beta_f) {
     return ct;
 }
 
+// The CTA's warps start every phase A at one barrier, to share instruction
+// fetches as in the fixed-step evaluator (there: why).  4,096 four-segment
+// TOs under a binding bound: 119 -> 94 ms; 2,048 with room: 129 -> 99 ms.
 __global__ void __launch_bounds__(128, 3) timing_kernel(const TimingArgs A) {
     extern __shared__ float tsmem_raw[];
     const int lane = threadIdx.x & 31;
@@ -1259,7 +1274,7 @@ __global__ void __launch_bounds__(128, 3) timing_kernel(const TimingArgs A) {
         if (lane == 0) t = atomicAdd(E.queue, 1u);
         t = __shfl_sync(kFullT, t, 0);
         if ((int64_t)t >= n_tos) break;
-        const int64_t ti = (int64_t)t;
+        const int64_t ti = E.perm ? (int64_t)E.perm[t] : (int64_t)t;
         const comet_mode_seq sq = E.seqs[ti];
         bool bad = sq.instance < 0 || sq.instance >= E.n_inst;
         const DevInstance* P = bad ? E.inst : E.inst + sq.instance;
@@ -1333,6 +1348,7 @@ __global__ void __launch_bounds__(128, 3) timing_kernel(const TimingArgs A) {
             bool model_curv = curv, fac = false, done = false;
             float beta_old = beta;
             for (;;) {
+                cta_in_step(E.in_step);  // start phase A together (see the kernel's comment)
                 const TMeasures m = tphase_a(C, beta, rho, model_curv, trip == kUpdate, beta_old);
                 if (trip == kMeasure) {
                     if (!m.finite) {
