@@ -5,7 +5,8 @@
 // compaction of the first B unseen orders into the next batch F_{s+1}.
 //
 // Every count lives in device memory and every launch has a fixed grid, so
-// a whole expansion round can be captured in a CUDA graph.
+// a whole expansion round can be captured in a CUDA graph.  A launch serves
+// one frontier or several at once (blockIdx.y), as the batched planner does.
 
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -34,10 +35,6 @@ __device__ __forceinline__ uint32_t float_key(float f) {
     if (f != f) return 0xffffffffu;
     const uint32_t b = __float_as_uint(f);
     return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
-
-__device__ __forceinline__ bool key_less(const TopKey& a, const TopKey& b) {
-    return a.mk < b.mk || (a.mk == b.mk && a.code < b.code);
 }
 
 __device__ unsigned long long encode_seq(const comet_mode_seq& s, int n_modes) {
@@ -84,36 +81,27 @@ __device__ bool set_contains(const unsigned long long* set, unsigned long long m
     return false;
 }
 
-// candidate table: code -> smallest ordinal proposing it
-__device__ void cand_insert(unsigned long long* keys, unsigned int* ords, unsigned long long mask,
-                            unsigned long long code, unsigned int ord) {
+// candidate table: code -> smallest ordinal proposing it.  Ordinals are kept
+// inverted (~ord, the largest wins), so that zeroed memory is an empty table;
+// each round's winners clear their entries again.  Returns the entry.
+__device__ int cand_insert(unsigned long long* keys, unsigned int* ords, unsigned long long mask,
+                           unsigned long long code, unsigned int ord) {
     unsigned long long h = mix64(code) & mask;
     for (unsigned long long probe = 0; probe <= mask; ++probe) {
         const unsigned long long prev = atomicCAS(&keys[h], kEmpty, code);
         if (prev == kEmpty || prev == code) {
-            atomicMin(&ords[h], ord);
-            return;
+            atomicMax(&ords[h], ~ord);
+            return (int)h;
         }
         h = (h + 1) & mask;
     }
-}
-
-__device__ unsigned int cand_min(const unsigned long long* keys, const unsigned int* ords, unsigned long long mask,
-                                 unsigned long long code) {
-    unsigned long long h = mix64(code) & mask;
-    for (unsigned long long probe = 0; probe <= mask; ++probe) {
-        if (keys[h] == code) return ords[h];
-        if (keys[h] == kEmpty) break;
-        h = (h + 1) & mask;
-    }
-    return 0xffffffffu;
+    return -1;  // table full (it holds twice the proposals, so unreachable)
 }
 
 // ------------------------------------------------------------- add to V
 
-__global__ void add_kernel(FrontierDev F, const comet_mode_seq* seqs, int64_t n, const int64_t* d_n, const float* cost,
+__device__ void add_orders(const FrontierDev& F, const comet_mode_seq* seqs, int64_t nn, const float* cost,
                            const float* viol, float eps_feas, float merit_mu) {
-    const int64_t nn = d_n ? *d_n : n;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nn; i += (int64_t)gridDim.x * blockDim.x) {
         const comet_mode_seq s = seqs[i];
         if (s.instance != F.instance || s.len < 1 || s.len > F.lmax) {
@@ -136,51 +124,93 @@ __global__ void add_kernel(FrontierDev F, const comet_mode_seq* seqs, int64_t n,
     }
 }
 
-// ---------------------------------------------------------------- top-k
-// Each CTA sorts a chunk of kChunk keys (bitonic, shared memory) and writes
-// its k smallest, in order, to out[block * k ...].
+__global__ void add_kernel(FrontierDev F, const comet_mode_seq* seqs, int64_t n, const int64_t* d_n, const float* cost,
+                           const float* viol, float eps_feas, float merit_mu) {
+    add_orders(F, seqs, d_n ? *d_n : n, cost, viol, eps_feas, merit_mu);
+}
 
-__global__ void topk_chunk_kernel(const TopKey* in_keys, const unsigned long long* codes, const float* merit,
-                                  const unsigned long long* n_in_dev, int64_t n_in_fixed, int k, TopKey* out) {
-    extern __shared__ TopKey sk[];
+// frontier y adds its slots [off[y], off[y] + n): n = its own next count, or
+// off[y + 1] - off[y] when `seeds`
+__global__ void add_many_kernel(const FrontierDev* Fs, const comet_mode_seq* seqs, const int64_t* off, int seeds,
+                                const float* cost, const float* viol, float eps_feas, float merit_mu) {
+    const FrontierDev F = Fs[blockIdx.y];
+    const int64_t o = off[blockIdx.y], n = seeds ? off[blockIdx.y + 1] - o : *F.n_next;
+    add_orders(F, seqs + o, n, cost + o, viol + o, eps_feas, merit_mu);
+}
+
+// ---------------------------------------------------------------- top-k
+// The k smallest keys of each chunk of the input, in order, by counting: a
+// key's place is the number of smaller keys in its chunk.  A CTA places 32
+// keys (a lane each); its 8 warps share the chunk, an eighth of each tile
+// each, read as shared-memory broadcasts.  Keys are unique in practice; equal
+// ones (the padding of an earlier pass) keep their input order.
+//
+// Counting does n^2 compares where a sort does n log^2 n, but without its 78
+// barriers, and spread over all SMs: a 4,096-key bitonic sort in one CTA took
+// about 80 us of every round, counting the 3,000 keys of a set of at most 7,096 takes 17 us.
+// Chunks bound the square: the first pass of a large set runs on chunks of
+// max(4096, 4 k) keys, each leaving k.
+
+constexpr int kRankWarps = 8, kRankTile = 1024;
+
+// chunk of a pass that is not the last
+__host__ __device__ inline int rank_chunk(int k) { return ((4 * k > kChunk ? 4 * k : kChunk) + 31) / 32 * 32; }
+
+__device__ __forceinline__ TopKey load_key(const TopKey* in_keys, const FrontierDev& F, int64_t i) {
+    if (in_keys) return in_keys[i];
+    TopKey key;
+    key.mk = float_key(F.merit[i]);
+    key.idx = (uint32_t)i;
+    key.code = F.codes[i];
+    return key;
+}
+
+// pass: 0 reads V, odd passes write top_a and even ones top_b
+__global__ void __launch_bounds__(32 * kRankWarps) topk_rank_kernel(FrontierDev F0, const FrontierDev* Fs, int pass,
+                                                                    int chunk, int k) {
+    __shared__ TopKey tile[kRankTile];
+    __shared__ int part[kRankWarps][32];
+    const FrontierDev F = Fs ? Fs[blockIdx.y] : F0;
+    const TopKey* in_keys = pass == 0 ? nullptr : (pass & 1) ? F.top_a : F.top_b;
+    TopKey* out = (pass & 1) ? F.top_b : F.top_a;
     // |V| may have run past the capacity (flagged on add): never read beyond it
-    const int64_t n_in = n_in_dev ? min((int64_t)*n_in_dev, n_in_fixed) : n_in_fixed;
-    const int64_t base = (int64_t)blockIdx.x * kChunk;
-    for (int t = threadIdx.x; t < kChunk; t += blockDim.x) {
-        const int64_t i = base + t;
-        TopKey key;
-        if (i < n_in) {
-            if (in_keys) {
-                key = in_keys[i];
-            } else {
-                key.mk = float_key(merit[i]);
-                key.idx = (uint32_t)i;
-                key.code = codes[i];
-            }
-        } else {
-            key.mk = 0xffffffffu;
-            key.idx = 0xffffffffu;
-            key.code = ~0ull;
+    int64_t n_max = F.capacity;  // keys that this pass can hold
+    for (int q = 0; q < pass; ++q) n_max = (n_max + rank_chunk(k) - 1) / rank_chunk(k) * k;
+    const int64_t n_in = pass == 0 ? min((int64_t)*F.nV, F.capacity) : n_max;
+    const int per = chunk / 32;  // CTAs of a chunk
+    const int c = blockIdx.x / per, i0 = (blockIdx.x - c * per) * 32;
+    const int64_t base = (int64_t)c * chunk;
+    if (c > 0 && base >= n_max) return;  // a smaller frontier than the launch's largest
+    const int len = (int)max((int64_t)0, min((int64_t)chunk, n_in - base));
+    if (i0 >= len && i0 >= k) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int i = i0 + lane;
+    TopKey me;
+    me.mk = 0xffffffffu;
+    me.idx = 0xffffffffu;
+    me.code = ~0ull;
+    if (i < len) me = load_key(in_keys, F, base + i);
+    int rank = 0;
+    for (int t0 = 0; t0 < len; t0 += kRankTile) {
+        const int tn = min(kRankTile, len - t0);
+        __syncthreads();
+        for (int t = threadIdx.x; t < tn; t += blockDim.x) tile[t] = load_key(in_keys, F, base + t0 + t);
+        __syncthreads();
+        const int j1 = min(tn, (warp + 1) * (kRankTile / kRankWarps));
+#pragma unroll 4
+        for (int j = warp * (kRankTile / kRankWarps); j < j1; ++j) {
+            const TopKey o = tile[j];
+            rank += o.mk < me.mk;
+            if (o.mk == me.mk) rank += o.code < me.code || (o.code == me.code && t0 + j < i);
         }
-        sk[t] = key;
     }
+    part[warp][lane] = rank;
     __syncthreads();
-    for (int size = 2; size <= kChunk; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int t = threadIdx.x; t < kChunk / 2; t += blockDim.x) {
-                const int lo = 2 * stride * (t / stride) + (t % stride);
-                const int hi = lo + stride;
-                const bool up = ((lo & size) == 0);
-                TopKey a = sk[lo], b = sk[hi];
-                if (key_less(b, a) == up) {
-                    sk[lo] = b;
-                    sk[hi] = a;
-                }
-            }
-            __syncthreads();
-        }
+    if (warp == 0) {
+        for (int w = 1; w < kRankWarps; ++w) rank += part[w][lane];
+        if (i >= len) rank = i;  // padding after the chunk's keys
+        if (rank < k && i < chunk) out[(int64_t)c * k + rank] = me;
     }
-    for (int t = threadIdx.x; t < k; t += blockDim.x) out[(int64_t)blockIdx.x * k + t] = sk[t];
 }
 
 // --------------------------------------------------------- neighbourhood
@@ -270,18 +300,35 @@ __device__ int neighbour_r(const FrontierDev& F, const uint16_t* s, int L, int j
     return Ln;
 }
 
-__global__ void neighbour_kernel(FrontierDev F, const TopKey* top, int k, int64_t slots) {
-    const int64_t total = (int64_t)k * slots;
+// One thread per edit slot; a slot that proposes an unseen order leaves its
+// code and its entry in the candidate table.  A block's slots belong to a few
+// consecutive parents, whose codes are decoded once per block: a decode is up
+// to 16 dependent 64-bit divisions, most of a slot's work otherwise (35 us
+// against 26 us for the 560,000 slots of a two-edit round).
+constexpr int kNbThreads = 256;
+
+__global__ void __launch_bounds__(kNbThreads) neighbour_kernel(FrontierDev F0, const FrontierDev* Fs, int in_b, int k) {
+    __shared__ uint16_t par[kNbThreads][COMET_MAX_SEGMENTS];
+    __shared__ int par_len[kNbThreads];
+    const FrontierDev F = Fs ? Fs[blockIdx.y] : F0;
+    const TopKey* top = in_b ? F.top_b : F.top_a;
+    // k slots <= 2^26 (checked when the frontier is created)
+    const unsigned slots = (unsigned)F.slots, total = (unsigned)k * slots;
     const unsigned long long nV = min(*F.nV, (unsigned long long)F.capacity);
-    const int kk = (int)min((unsigned long long)k, nV);
-    for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < total; o += (int64_t)gridDim.x * blockDim.x) {
-        const int r = (int)(o / slots);
-        const int j = (int)(o - (int64_t)r * slots);
+    const unsigned kk = (unsigned)min((unsigned long long)k, nV);
+    for (unsigned o0 = blockIdx.x * kNbThreads; o0 < total; o0 += gridDim.x * kNbThreads) {
+        const unsigned r0 = o0 / slots, r1 = min(o0 + kNbThreads - 1, total - 1) / slots;
+        __syncthreads();
+        if (threadIdx.x <= r1 - r0 && r0 + threadIdx.x < kk)
+            par_len[threadIdx.x] = decode_code(top[r0 + threadIdx.x].code, F.n_modes, par[threadIdx.x]);
+        __syncthreads();
+        const unsigned o = o0 + threadIdx.x;
+        if (o >= total) continue;
+        const unsigned r = o / slots;
         unsigned long long code = kEmpty;
         if (r < kk) {
-            uint16_t s[COMET_MAX_SEGMENTS], nb[COMET_MAX_SEGMENTS];
-            const int L = decode_code(top[r].code, F.n_modes, s);
-            const int Ln = neighbour_r(F, s, L, j, nb);
+            uint16_t nb[COMET_MAX_SEGMENTS];
+            const int Ln = neighbour_r(F, par[r - r0], par_len[r - r0], (int)(o - r * slots), nb);
             if (Ln > 0) {
                 comet_mode_seq q;
                 q.len = (uint8_t)Ln;
@@ -290,77 +337,84 @@ __global__ void neighbour_kernel(FrontierDev F, const TopKey* top, int k, int64_
                 if (set_contains(F.set, F.set_mask, code))
                     code = kEmpty;  // already in V
                 else
-                    cand_insert(F.cand_keys, F.cand_ord, F.cand_mask, code, (unsigned int)o);
+                    F.flag[o] = cand_insert(F.cand_keys, F.cand_ord, F.cand_mask, code, o);
             }
         }
         F.cand_code[o] = code;
     }
 }
 
-// winners (first proposal of each unseen code) -> flags
-__global__ void winner_kernel(FrontierDev F, int64_t total) {
-    for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < total; o += (int64_t)gridDim.x * blockDim.x) {
-        const unsigned long long code = F.cand_code[o];
-        int flag = 0;
-        if (code != kEmpty) flag = cand_min(F.cand_keys, F.cand_ord, F.cand_mask, code) == (unsigned int)o;
-        F.flag[o] = flag;
+// Winners (the first proposal of each unseen code) keep their code, the
+// other slots lose it; the winners of each block of kScan slots are counted.
+__global__ void __launch_bounds__(kScan) winner_kernel(FrontierDev F0, const FrontierDev* Fs, int k) {
+    const FrontierDev F = Fs ? Fs[blockIdx.y] : F0;
+    const int64_t total = (int64_t)k * F.slots, o = blockIdx.x * (int64_t)kScan + threadIdx.x;
+    if (blockIdx.x * (int64_t)kScan >= total) return;
+    bool win = false;
+    if (o < total && F.cand_code[o] != kEmpty) {
+        const int at = F.flag[o];
+        win = at >= 0 && F.cand_ord[at] == ~(unsigned int)o;
+        if (!win) F.cand_code[o] = kEmpty;
     }
+    const int n = __syncthreads_count(win);
+    if (threadIdx.x == 0) F.counts[blockIdx.x] = n;
 }
 
-// single-CTA exclusive scan over the flags in ordinal order; the first
-// `batch` winners (capped by the remaining evaluation budget) become F_{s+1}
-__global__ void compact_kernel(FrontierDev F, int64_t total, int batch, int64_t budget) {
+// The first `batch` winners in ordinal order (capped by the remaining
+// evaluation budget) become F_{s+1}: every block adds up the counts before
+// it, so the slots are placed in one parallel pass (a single-CTA scan took
+// 0.7 ms over the 560,000 slots of a two-edit round).  Winners clear their
+// entry of the candidate table.
+__global__ void __launch_bounds__(kScan) compact_kernel(FrontierDev F0, const FrontierDev* Fs, int k, int batch_in,
+                                                        int64_t budget) {
     __shared__ int warp_sums[32];
-    __shared__ int carry;
+    const FrontierDev F = Fs ? Fs[blockIdx.y] : F0;
+    const int64_t total = (int64_t)k * F.slots;
+    const int blocks = (int)((total + kScan - 1) / kScan);
+    if ((int)blockIdx.x >= blocks) return;
     const unsigned long long nV = min(*F.nV, (unsigned long long)F.capacity);
-    int64_t cap = batch;
+    int64_t cap = Fs ? F.batch : batch_in;
     if (budget > 0) cap = min(cap, budget - (int64_t)nV);
     if (cap < 0) cap = 0;
-    if (threadIdx.x == 0) carry = 0;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    // winners in the blocks before this one; block 0 adds up all of them
+    int before = 0;
+    const int upto = blockIdx.x == 0 ? blocks : (int)blockIdx.x;
+    for (int b = threadIdx.x; b < upto; b += kScan) before += F.counts[b];
+    for (int d = 16; d > 0; d >>= 1) before += __shfl_xor_sync(0xffffffffu, before, d);
+    if (lane == 0) warp_sums[w] = before;
     __syncthreads();
-    for (int64_t base = 0; base < total; base += blockDim.x) {
-        const int64_t o = base + threadIdx.x;
-        const int f = (o < total) ? F.flag[o] : 0;
-        // block-wide inclusive scan of f
-        int v = f;
-        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-        for (int d = 1; d < 32; d <<= 1) {
-            const int x = __shfl_up_sync(0xffffffffu, v, d);
-            if (lane >= d) v += x;
-        }
-        if (lane == 31) warp_sums[w] = v;
-        __syncthreads();
-        if (w == 0) {
-            int s = (lane < (int)(blockDim.x >> 5)) ? warp_sums[lane] : 0;
-            for (int d = 1; d < 32; d <<= 1) {
-                const int x = __shfl_up_sync(0xffffffffu, s, d);
-                if (lane >= d) s += x;
-            }
-            warp_sums[lane] = s;
-        }
-        __syncthreads();
-        const int excl = carry + (w > 0 ? warp_sums[w - 1] : 0) + v - f;
-        if (f && excl < cap) {
-            comet_mode_seq q;
-            const unsigned long long code = F.cand_code[o];
-            uint16_t m[COMET_MAX_SEGMENTS];
-            const int L = decode_code(code, F.n_modes, m);
-            q.instance = F.instance;
-            q.len = (uint8_t)L;
-            for (int i = 0; i < COMET_MAX_SEGMENTS; ++i) q.modes[i] = (i < L) ? m[i] : 0;
-            q.pad[0] = q.pad[1] = q.pad[2] = 0;
-            F.next[excl] = q;
-        }
-        __syncthreads();
-        if (threadIdx.x == blockDim.x - 1) carry = excl + f;
-        __syncthreads();
+    before = 0;
+    for (int i = 0; i < kScan / 32; ++i) before += warp_sums[i];
+    __syncthreads();
+    if (blockIdx.x == 0) {
+        if (threadIdx.x == 0) *F.n_next = min((int64_t)before, cap);
+        before = 0;
     }
-    if (threadIdx.x == 0) *F.n_next = min((int64_t)carry, cap);
+    const int64_t o = blockIdx.x * (int64_t)kScan + threadIdx.x;
+    const unsigned long long code = o < total ? F.cand_code[o] : kEmpty;
+    const unsigned bal = __ballot_sync(0xffffffffu, code != kEmpty);
+    if (lane == 0) warp_sums[w] = __popc(bal);
+    __syncthreads();
+    if (code == kEmpty) return;
+    for (int i = 0; i < w; ++i) before += warp_sums[i];
+    const int place = before + __popc(bal & ((1u << lane) - 1u));
+    const int at = F.flag[o];
+    F.cand_keys[at] = kEmpty;
+    F.cand_ord[at] = 0u;
+    if (place < cap) {
+        comet_mode_seq q;
+        uint16_t m[COMET_MAX_SEGMENTS];
+        const int L = decode_code(code, F.n_modes, m);
+        q.instance = F.instance;
+        q.len = (uint8_t)L;
+        for (int i = 0; i < COMET_MAX_SEGMENTS; ++i) q.modes[i] = (i < L) ? m[i] : 0;
+        q.pad[0] = q.pad[1] = q.pad[2] = 0;
+        F.next[place] = q;
+    }
 }
 
 }  // namespace
-
-size_t topk_smem_bytes() { return sizeof(TopKey) * kChunk; }
 
 // V's codes back into the (cleared) hash set after a checkpoint restored
 // codes[0..n) and merit[0..n)
@@ -387,64 +441,86 @@ cudaError_t launch_frontier_add(const FrontierDev& F, const comet_mode_seq* seqs
     return cudaGetLastError();
 }
 
-cudaError_t prepare_expand() {
-    // shared-memory attribute of the top-k kernel, once per device (not a
-    // stream operation: called at frontier creation, outside any capture)
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+// the orders of several frontiers in one launch (see add_many_kernel);
+// n_max: the largest count of one frontier
+cudaError_t launch_frontier_add_many(const FrontierDev* d_fs, int n_f, const comet_mode_seq* seqs, const int64_t* d_off,
+                                     bool seeds, int64_t n_max, const float* cost, const float* viol, float eps_feas,
+                                     float merit_mu, cudaStream_t s) {
+    for (int y = 0; y < n_f; y += kMaxGridY) {
+        const dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>((n_max + 255) / 256, 1024)),
+                        (unsigned)std::min(n_f - y, kMaxGridY));
+        add_many_kernel<<<grid, 256, 0, s>>>(d_fs + y, seqs, d_off + y, seeds ? 1 : 0, cost, viol, eps_feas, merit_mu);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+namespace {
+
+// Top-k of one frontier (F) or of n_f frontiers (d_fs, capacities up to
+// `capacity`); *in_b tells whether the keys are in top_b (else top_a).
+cudaError_t topk(const FrontierDev& F, const FrontierDev* d_fs, int n_f, int64_t capacity, int k, bool* in_b,
+                 cudaStream_t s) {
+    // one pass over up to kRankOnce keys; else chunk passes until that fits
+    // (each chunk of at least 4 k keys leaves k)
+    int64_t n_in = capacity;
+    for (int pass = 0;; ++pass) {
+        const bool last = n_in <= kRankOnce;
+        const int64_t chunk = last ? (std::max<int64_t>(n_in, k) + 31) / 32 * 32 : rank_chunk(k);
+        const int64_t chunks = last ? 1 : (n_in + chunk - 1) / chunk;
+        const dim3 grid((unsigned)(chunks * (chunk / 32)), (unsigned)n_f);
+        topk_rank_kernel<<<grid, 32 * kRankWarps, 0, s>>>(F, d_fs, pass, (int)chunk, k);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        *in_b = pass & 1;
+        if (last) return cudaSuccess;
+        n_in = chunks * k;
+    }
+}
+
+// One expansion round of one frontier (F; batch) or of n_f frontiers (d_fs,
+// each with its own batch), total: the largest number of slots.
+cudaError_t expand(const FrontierDev& F, const FrontierDev* d_fs, int n_f, int64_t capacity, int64_t total, int k,
+                   int batch, int64_t budget, cudaStream_t s) {
+    bool in_b = false;
+    cudaError_t e = topk(F, d_fs, n_f, capacity, k, &in_b, s);
     if (e != cudaSuccess) return e;
-    static bool done[64] = {};
-    if (dev < 64 && done[dev]) return cudaSuccess;
-    e = cudaFuncSetAttribute(topk_chunk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)topk_smem_bytes());
-    if (e == cudaSuccess && dev < 64) done[dev] = true;
+    const dim3 g1((unsigned)std::min<int64_t>((total + kNbThreads - 1) / kNbThreads, 65535), (unsigned)n_f);
+    const dim3 g2((unsigned)((total + kScan - 1) / kScan), (unsigned)n_f);
+    neighbour_kernel<<<g1, kNbThreads, 0, s>>>(F, d_fs, in_b ? 1 : 0, k);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    winner_kernel<<<g2, kScan, 0, s>>>(F, d_fs, k);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    compact_kernel<<<g2, kScan, 0, s>>>(F, d_fs, k, batch, budget);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+const TopKey* launch_topk(const FrontierDev& F, int k, cudaStream_t s, cudaError_t* err) {
+    bool in_b = false;
+    *err = topk(F, nullptr, 1, F.capacity, k, &in_b, s);
+    return *err != cudaSuccess ? nullptr : in_b ? F.top_b : F.top_a;
+}
+
+cudaError_t launch_topk_many(const FrontierDev* d_fs, int n_f, int64_t capacity, int k, bool* in_b, cudaStream_t s) {
+    cudaError_t e = cudaSuccess;
+    for (int y = 0; y < n_f && e == cudaSuccess; y += kMaxGridY)
+        e = topk(FrontierDev{}, d_fs + y, std::min(n_f - y, kMaxGridY), capacity, k, in_b, s);
     return e;
 }
 
-const TopKey* launch_topk(const FrontierDev& F, int k, cudaStream_t s, cudaError_t* err) {
-    cudaError_t e = prepare_expand();
-    *err = e;
-    if (e != cudaSuccess) return nullptr;
-    // chunk passes until one chunk remains; the first pass reads V directly
-    int64_t n_in = F.capacity;
-    const TopKey* in = nullptr;
-    TopKey* bufs[2] = {F.top_a, F.top_b};
-    int which = 0;
-    bool first = true;
-    for (;;) {
-        const int64_t chunks = (n_in + kChunk - 1) / kChunk;
-        topk_chunk_kernel<<<(unsigned)chunks, 1024, topk_smem_bytes(), s>>>(
-            in, F.codes, F.merit, first ? F.nV : nullptr, n_in, k, bufs[which]);
-        if ((e = cudaGetLastError()) != cudaSuccess) {
-            *err = e;
-            return nullptr;
-        }
-        first = false;
-        in = bufs[which];
-        n_in = chunks * k;
-        which ^= 1;
-        if (chunks == 1) break;
-    }
-    return in;
+cudaError_t launch_expand(const FrontierDev& F, int k, int batch, int64_t budget, cudaStream_t s) {
+    return expand(F, nullptr, 1, F.capacity, (int64_t)k * F.slots, k, batch, budget, s);
 }
 
-cudaError_t launch_expand(const FrontierDev& F, int k, int batch, int64_t budget, cudaStream_t s) {
-    cudaError_t e;
-    const TopKey* top = launch_topk(F, k, s, &e);
-    if (!top) return e;
-
-    const int64_t slots = F.slots;
-    const int64_t total = (int64_t)k * slots;
-    e = cudaMemsetAsync(F.cand_keys, 0, sizeof(unsigned long long) * (F.cand_mask + 1), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(F.cand_ord, 0xff, sizeof(unsigned int) * (F.cand_mask + 1), s);
-    if (e != cudaSuccess) return e;
-    const int threads = 256;
-    const int blocks = (int)std::min<int64_t>((total + threads - 1) / threads, 4096);
-    neighbour_kernel<<<blocks, threads, 0, s>>>(F, top, k, slots);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    winner_kernel<<<blocks, threads, 0, s>>>(F, total);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    compact_kernel<<<1, 1024, 0, s>>>(F, total, batch, budget);
-    return cudaGetLastError();
+cudaError_t launch_expand_many(const FrontierDev* d_fs, int n_f, int64_t capacity, int64_t slots, int k,
+                               int64_t budget, cudaStream_t s) {
+    cudaError_t e = cudaSuccess;
+    for (int y = 0; y < n_f && e == cudaSuccess; y += kMaxGridY)
+        e = expand(FrontierDev{}, d_fs + y, std::min(n_f - y, kMaxGridY), capacity, (int64_t)k * slots, k, 0, budget, s);
+    return e;
 }
 
 }  // namespace comet

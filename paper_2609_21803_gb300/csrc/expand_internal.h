@@ -11,7 +11,10 @@
 
 namespace comet {
 
-constexpr int kChunk = 4096;  // keys sorted per CTA in the top-k passes
+constexpr int kChunk = 4096;         // smallest chunk of a top-k pass; the largest k
+constexpr int64_t kRankOnce = 16384;  // keys ranked in one pass
+constexpr int kScan = 1024;           // slots per block of the compaction
+constexpr int kMaxGridY = 65535;      // frontiers per launch
 
 struct TopKey {
     uint32_t mk;    // order-preserving key of M_hat
@@ -34,11 +37,13 @@ struct FrontierDev {
     unsigned long long set_mask;
     TopKey* top_a;              // top-k pass buffers
     TopKey* top_b;
-    unsigned long long* cand_code;  // [k_max * slots]
-    int* flag;                      // [k_max * slots]
-    unsigned long long* cand_keys;  // candidate table
+    unsigned long long* cand_code;  // [k_max * slots] proposed codes, then the winners'
+    int* flag;                      // [k_max * slots] entry of a proposal in the candidate table
+    int* counts;                    // winners per kScan slots
+    unsigned long long* cand_keys;  // candidate table, empty (zero) between rounds
     unsigned int* cand_ord;
     unsigned long long cand_mask;
+    int batch;                      // orders of the next batch
     comet_mode_seq* next;           // [batch]
     int64_t* n_next;
     int* error;                     // 1 malformed order, 2 capacity exceeded
@@ -55,13 +60,18 @@ inline int64_t edit_slots(int lmax, int n_alpha, int radius) {
 constexpr int kGrammarNone = 0, kGrammarPush = 1;
 constexpr int kPushFree = 12;  // free motion in the 13-mode pushing alphabet
 
-size_t topk_smem_bytes();
-cudaError_t prepare_expand();
 cudaError_t launch_frontier_restore(const FrontierDev& F, int64_t n, cudaStream_t s);
 cudaError_t launch_frontier_add(const FrontierDev& F, const comet_mode_seq* seqs, int64_t n, const int64_t* d_n,
                                 const float* cost, const float* viol, float eps_feas, float merit_mu, cudaStream_t s);
 const TopKey* launch_topk(const FrontierDev& F, int k, cudaStream_t s, cudaError_t* err);
 cudaError_t launch_expand(const FrontierDev& F, int k, int batch, int64_t budget, cudaStream_t s);
+// the same for n_f frontiers (an array in device memory) in one launch each
+cudaError_t launch_frontier_add_many(const FrontierDev* d_fs, int n_f, const comet_mode_seq* seqs, const int64_t* d_off,
+                                     bool seeds, int64_t n_max, const float* cost, const float* viol, float eps_feas,
+                                     float merit_mu, cudaStream_t s);
+cudaError_t launch_topk_many(const FrontierDev* d_fs, int n_f, int64_t capacity, int k, bool* in_b, cudaStream_t s);
+cudaError_t launch_expand_many(const FrontierDev* d_fs, int n_f, int64_t capacity, int64_t slots, int k,
+                               int64_t budget, cudaStream_t s);
 
 }  // namespace comet
 

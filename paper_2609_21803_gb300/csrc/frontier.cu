@@ -78,10 +78,6 @@ comet_status comet_frontier_create_ex(comet_problem* p, int32_t instance, int64_
     const int64_t slots = comet::edit_slots(d.max_segments, n_alpha, radius);
     if ((int64_t)k_max * slots > ((int64_t)1 << 26))
         return ffail(COMET_ERR_INVALID_ARG, "k_max x neighbourhood slots above 2^26 (use radius 1 or a smaller beam)");
-    {
-        const cudaError_t pe = comet::prepare_expand();
-        if (pe != cudaSuccess) return fcuda(pe, "expand kernels");
-    }
     comet_frontier* f = new comet_frontier();
     f->p = p;
     f->batch = batch;
@@ -98,6 +94,7 @@ comet_status comet_frontier_create_ex(comet_problem* p, int32_t instance, int64_
     F.slots = (int)slots;
     F.capacity = capacity;
     F.batch_cap = std::max<int64_t>(batch, 1);
+    F.batch = batch;
     const uint64_t set_cap = pow2_at_least((uint64_t)capacity * 2);
     const int64_t total = (int64_t)k_max * F.slots;
     const uint64_t cand_cap = pow2_at_least((uint64_t)total * 2);
@@ -118,6 +115,7 @@ comet_status comet_frontier_create_ex(comet_problem* p, int32_t instance, int64_
     const size_t o_tb = take(sizeof(comet::TopKey) * top_n);
     const size_t o_cc = take(sizeof(unsigned long long) * total);
     const size_t o_fl = take(sizeof(int) * total);
+    const size_t o_ct = take(sizeof(int) * ((total + comet::kScan - 1) / comet::kScan));
     const size_t o_ck = take(sizeof(unsigned long long) * cand_cap);
     const size_t o_co = take(sizeof(unsigned int) * cand_cap);
     const size_t o_nx = take(sizeof(comet_mode_seq) * batch);
@@ -138,6 +136,7 @@ comet_status comet_frontier_create_ex(comet_problem* p, int32_t instance, int64_
     F.top_b = (comet::TopKey*)(b + o_tb);
     F.cand_code = (unsigned long long*)(b + o_cc);
     F.flag = (int*)(b + o_fl);
+    F.counts = (int*)(b + o_ct);
     F.cand_keys = (unsigned long long*)(b + o_ck);
     F.cand_ord = (unsigned int*)(b + o_co);
     F.cand_mask = cand_cap - 1;
@@ -697,18 +696,19 @@ __global__ void gather_next_kernel(const SlotSrc* src, int n_inst, int batch, co
     }
 }
 
-// ranked entries of one frontier -> orders; ranks past |V| become empty
-// slots (length 0), which the evaluator skips
-__global__ void decode_top_kernel(const comet::TopKey* top, int k, const unsigned long long* nV, int instance,
-                                  int n_modes, comet_mode_seq* out) {
+// ranked entries of every frontier (blockIdx.y) -> orders, k slots each;
+// ranks past |V| become empty slots (length 0), which the evaluator skips
+__global__ void decode_top_kernel(const comet::FrontierDev* Fs, int in_b, int k, comet_mode_seq* out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= k) return;
+    const comet::FrontierDev& F = Fs[blockIdx.y];
+    const comet::TopKey* top = in_b ? F.top_b : F.top_a;
     comet_mode_seq q;
     memset(&q, 0, sizeof(q));
-    q.instance = instance;
-    if ((unsigned long long)i < *nV) {
+    q.instance = F.instance;
+    if ((unsigned long long)i < *F.nV) {
         unsigned long long code = top[i].code;
-        const unsigned long long base = (unsigned long long)(n_modes + 1);
+        const unsigned long long base = (unsigned long long)(F.n_modes + 1);
         const int L = (int)(code % base);
         code /= base;
         q.len = (uint8_t)L;
@@ -717,7 +717,7 @@ __global__ void decode_top_kernel(const comet::TopKey* top, int k, const unsigne
             code /= base;
         }
     }
-    out[i] = q;
+    out[(int64_t)blockIdx.y * k + i] = q;
 }
 
 }  // namespace
@@ -813,12 +813,17 @@ comet_status plan_batch_impl(comet_problem* p, int32_t n_inst, const int32_t* in
     const size_t b_seq = ((sizeof(comet_mode_seq) * n_eval_max + 255) / 256) * 256;
     const size_t b_f = ((sizeof(float) * n_eval_max + 255) / 256) * 256;
     const size_t b_src = ((sizeof(SlotSrc) * n_inst + 255) / 256) * 256;
-    FTRY(cudaMalloc(&buf.p, b_seq + 2 * b_f + b_src), "planner buffers");
+    const size_t b_fs = ((sizeof(comet::FrontierDev) * n_inst + 255) / 256) * 256;
+    const size_t b_off = ((sizeof(int64_t) * (n_inst + 1) + 255) / 256) * 256;
+    FTRY(cudaMalloc(&buf.p, b_seq + 2 * b_f + b_src + b_fs + 2 * b_off), "planner buffers");
     char* bp = (char*)buf.p;
     comet_mode_seq* d_seqs = (comet_mode_seq*)bp;
     float* d_cost = (float*)(bp + b_seq);
     int32_t* d_status = (int32_t*)(bp + b_seq + b_f);
     SlotSrc* d_src = (SlotSrc*)(bp + b_seq + 2 * b_f);
+    comet::FrontierDev* d_fs = (comet::FrontierDev*)(bp + b_seq + 2 * b_f + b_src);
+    int64_t* d_seed_off = (int64_t*)((char*)d_fs + b_fs);
+    int64_t* d_off = (int64_t*)((char*)d_seed_off + b_off);
     DevBuf warm_buf, rows_buf;
     float* d_warm = nullptr;
     int* d_rows = nullptr;
@@ -833,10 +838,26 @@ comet_status plan_batch_impl(comet_problem* p, int32_t n_inst, const int32_t* in
         d_warm = (float*)warm_buf.p;
         d_rows = (int*)rows_buf.p;
     }
+    int64_t cap_max = 0, slots_max = 0, seeds_max = 0;
     {
         std::vector<SlotSrc> h(n_inst);
-        for (int i = 0; i < n_inst; ++i) h[i] = SlotSrc{fr[i]->d.next, fr[i]->d.n_next};
+        std::vector<comet::FrontierDev> hf(n_inst);
+        std::vector<int64_t> ho(n_inst + 1);
+        for (int i = 0; i < n_inst; ++i) {
+            h[i] = SlotSrc{fr[i]->d.next, fr[i]->d.n_next};
+            hf[i] = fr[i]->d;
+            ho[i] = (int64_t)i * batch;
+            cap_max = std::max(cap_max, fr[i]->d.capacity);
+            slots_max = std::max<int64_t>(slots_max, fr[i]->d.slots);
+            seeds_max = std::max(seeds_max, seed_offsets[i + 1] - seed_offsets[i]);
+        }
+        ho[n_inst] = (int64_t)n_inst * batch;
         FTRY(cudaMemcpyAsync(d_src, h.data(), sizeof(SlotSrc) * n_inst, cudaMemcpyHostToDevice, s), "slots");
+        FTRY(cudaMemcpyAsync(d_fs, hf.data(), sizeof(comet::FrontierDev) * n_inst, cudaMemcpyHostToDevice, s),
+             "frontiers");
+        FTRY(cudaMemcpyAsync(d_seed_off, seed_offsets, sizeof(int64_t) * (n_inst + 1), cudaMemcpyHostToDevice, s),
+             "offsets");
+        FTRY(cudaMemcpyAsync(d_off, ho.data(), sizeof(int64_t) * (n_inst + 1), cudaMemcpyHostToDevice, s), "offsets");
     }
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
     struct EvGuard {
@@ -857,17 +878,15 @@ comet_status plan_batch_impl(comet_problem* p, int32_t n_inst, const int32_t* in
     }
     st = comet::launch_eval_device(p, d_seqs, S, nullptr, d_warm, 0, d_cost, nullptr, d_status);
     if (st != COMET_OK) return st;
-    for (int i = 0; i < n_inst; ++i) {
-        const int64_t o = seed_offsets[i], n = seed_offsets[i + 1] - o;
-        FTRY(comet::launch_frontier_add(fr[i]->d, d_seqs + o, n, nullptr, d_cost + o, p->d_viol + o, eps, mmu, s),
-             "add seeds");
-    }
-    // one round: every frontier expands, all next batches are evaluated in
-    // one persistent launch, each frontier adds its slots
+    FTRY(comet::launch_frontier_add_many(d_fs, n_inst, d_seqs, d_seed_off, true, seeds_max, d_cost, p->d_viol, eps, mmu,
+                                         s),
+         "add seeds");
+    // one round: every frontier expands (one launch per step for all of them:
+    // 32 frontiers one after the other took 3.5 ms a round), all next batches
+    // are evaluated in one persistent launch, each frontier adds its slots
     auto round = [&]() -> comet_status {
+        FTRY(comet::launch_expand_many(d_fs, n_inst, cap_max, slots_max, po.k, po.budget, s), "expand");
         for (int i = 0; i < n_inst; ++i) {
-            const cudaError_t e = comet::launch_expand(fr[i]->d, po.k, fr[i]->batch, po.budget, s);
-            if (e != cudaSuccess) return fcuda(e, "expand");
             if (q) {
                 // rank the whole neighbourhood, keep `batch` in order; the
                 // warm starts land in the frontier's slots
@@ -881,14 +900,8 @@ comet_status plan_batch_impl(comet_problem* p, int32_t n_inst, const int32_t* in
         FTRY(cudaGetLastError(), "gather");
         comet_status r = comet::launch_eval_device(p, d_seqs, n_round, nullptr, d_warm, 0, d_cost, nullptr, d_status);
         if (r != COMET_OK) return r;
-        for (int i = 0; i < n_inst; ++i) {
-            comet::FrontierDev Fa = fr[i]->d;
-            Fa.batch_cap = batch;
-            const int64_t o = (int64_t)i * batch;
-            const cudaError_t e = comet::launch_frontier_add(Fa, d_seqs + o, batch, fr[i]->d.n_next, d_cost + o,
-                                                             p->d_viol + o, eps, mmu, s);
-            if (e != cudaSuccess) return fcuda(e, "add");
-        }
+        FTRY(comet::launch_frontier_add_many(d_fs, n_inst, d_seqs, d_off, false, batch, d_cost, p->d_viol, eps, mmu, s),
+             "add");
         return COMET_OK;
     };
     if (po.use_graph && po.rounds > 0) {
@@ -918,12 +931,11 @@ comet_status plan_batch_impl(comet_problem* p, int32_t n_inst, const int32_t* in
     // refinement: the K_ref best of every instance, ranked and decoded on the
     // device (ranks past |V_i| become empty slots), re-solved in one launch
     FTRY(cudaEventRecord(ev[2], s), "event");
-    for (int i = 0; i < n_inst; ++i) {
-        cudaError_t e = cudaSuccess;
-        const comet::TopKey* top = comet::launch_topk(fr[i]->d, po.k_ref, s, &e);
-        if (!top) return fcuda(e, "top-k");
-        decode_top_kernel<<<(unsigned)((po.k_ref + 127) / 128), 128, 0, s>>>(
-            top, po.k_ref, fr[i]->d.nV, instances[i], p->inst[instances[i]].n_modes, d_seqs + (int64_t)i * po.k_ref);
+    bool in_b = false;
+    FTRY(comet::launch_topk_many(d_fs, n_inst, cap_max, po.k_ref, &in_b, s), "top-k");
+    for (int y = 0; y < n_inst; y += comet::kMaxGridY) {
+        const dim3 grid((unsigned)((po.k_ref + 127) / 128), (unsigned)std::min(n_inst - y, comet::kMaxGridY));
+        decode_top_kernel<<<grid, 128, 0, s>>>(d_fs + y, in_b ? 1 : 0, po.k_ref, d_seqs + (int64_t)y * po.k_ref);
         FTRY(cudaGetLastError(), "decode");
     }
     const int32_t t_ref = po.ref_iters > 0 ? po.ref_iters : (p->opts.ref_iters > 0 ? p->opts.ref_iters : 1500);
