@@ -171,9 +171,10 @@ __device__ __forceinline__ bool weight_of(const LayerTab& t, int64_t i, int& l, 
     for (int j = 0; j < kLayers; ++j) {
         const int64_t o = i - t.w_off[j];
         if (o >= 0 && o < (int64_t)t.dout[j] * t.din[j]) {
+            // a layer has at most (12 x 512 + 16) x 256 weights: 32 bits
             l = j;
-            r = (int)(o / t.din[j]);
-            c = (int)(o - (int64_t)r * t.din[j]);
+            r = (int)((unsigned)o / (unsigned)t.din[j]);
+            c = (int)((unsigned)o - (unsigned)r * (unsigned)t.din[j]);
             return true;
         }
     }
@@ -231,39 +232,54 @@ __global__ void adamw_kernel(float* p, const float* g, float* m, float* v, int64
 }
 
 // features of order i (see comet_proposal.h); rows i >= n (device count)
-// and orders of another instance range give zero rows
+// and orders of another instance range give zero rows.  A thread writes 8
+// consecutive features (in_dim is a multiple of 64) as one 16-byte store
+// where X allows it (vec).
 __global__ void features_kernel(const comet_mode_seq* seqs, int64_t n_rows, const int64_t* d_n, const float* fi,
-                                int n_inst, int l_max, int n_modes, int in_dim, uint16_t* X, uint16_t* Xt,
-                                int64_t ld_t, int bim) {
+                                int n_inst, int l_max, int n_modes, int in_dim, uint16_t* X, int bim, int vec) {
     const int slot_w = bim ? kBimSlot : n_modes + 1;
     const int64_t nn = d_n ? min(*d_n, n_rows) : n_rows;
-    const int64_t total = n_rows * in_dim;
+    const int chunks = in_dim / 8;
+    const int64_t total = n_rows * chunks;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = t / in_dim;
-        const int c = (int)(t - i * in_dim);
-        float x = 0.f;
+        const int64_t i = t / chunks;
+        const int c0 = (int)(t - i * chunks) * 8;
+        uint32_t pk[4] = {0u, 0u, 0u, 0u};
         if (i < nn) {
-            const comet_mode_seq s = seqs[i];
-            if (s.instance >= 0 && s.instance < n_inst && s.len >= 1 && s.len <= l_max) {
-                if (c < kInstFeat) {
-                    x = fi[s.instance * kInstFeat + c];
-                } else if (c < kInstFeat + slot_w * l_max) {
-                    const int slot = (c - kInstFeat) / slot_w, e = (c - kInstFeat) % slot_w;
-                    if (bim) {
-                        // mode m = 169 g + 13 h_L + h_R: one-hots of g, h_L, h_R
-                        const int m = slot < s.len ? (int)s.modes[slot] : -1;
-                        x = (m < 0) ? (e == kBimSlot - 1 ? 1.f : 0.f)
-                                    : ((e == m / 169 || e == 3 + (m / 13) % 13 || e == 16 + m % 13) ? 1.f : 0.f);
-                    } else {
-                        const int want = slot < s.len ? (int)s.modes[slot] : n_modes;
-                        x = (e == want) ? 1.f : 0.f;
+            const comet_mode_seq* s = seqs + i;
+            const int inst = s->instance, len = s->len;
+            if (inst >= 0 && inst < n_inst && len >= 1 && len <= l_max) {
+                int slot = c0 < kInstFeat ? 0 : (c0 - kInstFeat) / slot_w;
+                int e = c0 < kInstFeat ? c0 - kInstFeat : (c0 - kInstFeat) - slot * slot_w;
+                int m = slot < len ? (int)s->modes[slot] : -1;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    float x = 0.f;
+                    if (e < 0) {
+                        x = fi[inst * kInstFeat + c0 + j];
+                    } else if (slot < l_max) {
+                        if (bim)
+                            // mode m = 169 g + 13 h_L + h_R: one-hots of g, h_L, h_R
+                            x = (m < 0) ? (e == kBimSlot - 1 ? 1.f : 0.f)
+                                        : ((e == m / 169 || e == 3 + (m / 13) % 13 || e == 16 + m % 13) ? 1.f : 0.f);
+                        else
+                            x = (e == (m < 0 ? n_modes : m)) ? 1.f : 0.f;
+                    }
+                    pk[j / 2] |= (uint32_t)bf16_bits(x) << (16 * (j & 1));
+                    if (++e == slot_w) {
+                        e = 0;
+                        ++slot;
+                        m = slot < len ? (int)s->modes[slot] : -1;
                     }
                 }
             }
         }
-        const uint16_t b = bf16_bits(x);
-        X[i * in_dim + c] = b;
-        if (Xt) Xt[(int64_t)c * ld_t + i] = b;
+        uint16_t* out = X + i * in_dim + c0;
+        if (vec) {
+            *reinterpret_cast<uint4*>(out) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+        } else {
+            for (int j = 0; j < 8; ++j) out[j] = (uint16_t)(pk[j / 2] >> (16 * (j & 1)));
+        }
     }
 }
 
@@ -300,80 +316,42 @@ __global__ void targets_kernel(const comet_mode_seq* seqs, int64_t n, const floa
     }
 }
 
-// mini-batch gather: row b of the batch is sample hash(seed, step, b) mod S
+// mini-batch gather: row b of the batch is sample hash(seed, step, b) mod S.
+// A warp per row (one modulo each), 16 bytes per lane: rows are whole 16-byte
+// units (in_dim a multiple of 64, out_dim of 16).
 __global__ void gather_kernel(const uint16_t* dX, const float* dT, const float* dOm, int64_t S, int batch,
                               const int64_t* d_step, unsigned long long seed, int in_dim, int out_dim, uint16_t* X,
-                              uint16_t* Xt, int64_t ld_t, float* T, float* Om) {
+                              float* T, float* Om) {
     const unsigned long long step = (unsigned long long)(*d_step);
-    const int64_t per = (int64_t)in_dim + out_dim;
-    const int64_t total = (int64_t)batch * per;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t b = t / per;
-        const int c = (int)(t - b * per);
+    const int lane = threadIdx.x & 31, nx = in_dim / 8, ny = out_dim / 4;
+    for (int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); b < batch; b += gridDim.x * (blockDim.x >> 5)) {
         const unsigned long long h = mix64(seed ^ mix64(step * 0x100000001b3ull + (unsigned long long)b));
         const int64_t j = (int64_t)(h % (unsigned long long)S);
-        if (c < in_dim) {
-            const uint16_t v = dX[j * in_dim + c];
-            X[b * in_dim + c] = v;
-            Xt[(int64_t)c * ld_t + b] = v;
-        } else {
-            const int o = c - in_dim;
-            T[b * out_dim + o] = dT[j * out_dim + o];
-            Om[b * out_dim + o] = dOm[j * out_dim + o];
+        const uint4* x = reinterpret_cast<const uint4*>(dX + j * in_dim);
+        const float4 *t = reinterpret_cast<const float4*>(dT + j * out_dim),
+                     *w = reinterpret_cast<const float4*>(dOm + j * out_dim);
+        uint4* xo = reinterpret_cast<uint4*>(X + (int64_t)b * in_dim);
+        float4 *to = reinterpret_cast<float4*>(T + (int64_t)b * out_dim),
+               *wo = reinterpret_cast<float4*>(Om + (int64_t)b * out_dim);
+        for (int c = lane; c < nx; c += 32) xo[c] = x[c];
+#pragma unroll 4
+        for (int c = lane; c < ny; c += 32) {
+            to[c] = t[c];
+            wo[c] = w[c];
         }
     }
 }
 
-// dL/dY = (2/B) Omega (Y - T) -> G (bf16) and its transpose; the loss sum
-// is accumulated into *loss and the step counter advanced
-__global__ void loss_grad_kernel(const float* Y, const float* T, const float* Om, int64_t M, int out_dim, uint16_t* G,
-                                 uint16_t* Gt, int64_t ld_t, float* loss, int64_t* d_step) {
-    __shared__ float red[32];
-    const float inv_b = 1.f / (float)M;
-    float acc = 0.f;
-    const int64_t total = M * out_dim;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = t / out_dim;
-        const int c = (int)(t - r * out_dim);
-        const float d = Y[t] - T[t], w = Om[t];
-        acc += w * d * d;
-        const uint16_t g = bf16_bits(2.f * w * d * inv_b);
-        G[t] = g;
-        Gt[(int64_t)c * ld_t + r] = g;
-    }
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        float v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.f;
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (threadIdx.x == 0) atomicAdd(loss, v * inv_b);
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) *d_step += 1;
+int grid_for(int64_t work, int threads = 256) {
+    return (int)std::max<int64_t>(1, std::min<int64_t>((work + threads - 1) / threads, 152 * 16));
 }
 
-// db[n] = sum_m G[m][n], from the transposed copy (one block per n)
-__global__ void bias_grad_kernel(const uint16_t* Gt, int64_t ld_t, int64_t M, float* db) {
-    __shared__ float red[32];
-    const uint16_t* row = Gt + (int64_t)blockIdx.x * ld_t;
-    float acc = 0.f;
-    for (int64_t m = threadIdx.x; m < M; m += blockDim.x) acc += bf16_value(row[m]);
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        float v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.f;
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (threadIdx.x == 0) db[blockIdx.x] = v;
-    }
-}
-
-// merit = exp(y_0) and the warm start of order i from the predicted
-// controls: Euler rollout of the pusher-slider model from the start pose
-// (s_0 = 0, s reset to 0 after a face change), or the cold-start poses
-__global__ void predict_post_kernel(const float* Y, int out_dim, const comet_mode_seq* seqs, const int* row_of,
-                                    int64_t n_rows, const int64_t* d_n, const comet::DevInstance* inst, int n_inst,
-                                    int n_max, int warm_mode, float* merit, float* warm, int64_t stride, int bim) {
+// The same with an Euler rollout of the pusher-slider model from the start
+// pose (warm_mode 0, pushing; s_0 = 0, s reset to 0 after a face change): a
+// chain over the knots, so a thread takes a whole order.
+__global__ void predict_rollout_kernel(const float* Y, int out_dim, const comet_mode_seq* seqs, const int* row_of,
+                                       int64_t n_rows, const int64_t* d_n, const comet::DevInstance* inst, int n_inst,
+                                       int n_max, float* merit, float* warm, int64_t stride) {
     const int64_t nn = d_n ? min(*d_n, n_rows) : n_rows;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nn; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t r = row_of ? (int64_t)row_of[i] : i;
@@ -388,27 +366,8 @@ __global__ void predict_post_kernel(const float* Y, int out_dim, const comet_mod
         }
         const comet::DevInstance& P = inst[s.instance];
         const int L = s.len, N = P.K * L, Nm1 = n_max + 1;
-        if (bim) {
-            // bimanual: the cold start's poses (hand offsets 0) and the
-            // predicted controls, forces back from units of m g
-            const float mg = P.mass * kGrav;
-            for (int k = 0; k <= n_max; ++k) {
-                const float al = (float)k / (float)N;
-                for (int c = 0; c < 5; ++c)
-                    w[c * Nm1 + k] = (k <= N && c < 3) ? (1.f - al) * P.start[c] + al * P.goal[c] : 0.f;
-            }
-            for (int c = 0; c < 12; ++c)
-                for (int k = 0; k < n_max; ++k)
-                    w[5 * Nm1 + c * n_max + k] = (k < N) ? y[1 + c * n_max + k] * (bim_force(c) ? mg : 1.f) : 0.f;
-            continue;
-        }
         float x[4] = {P.start[0], P.start[1], P.start[2], 0.f};
         for (int k = 0; k <= N; ++k) {
-            if (warm_mode == 1 && k > 0) {
-                const float al = (float)k / (float)N;
-                for (int c = 0; c < 3; ++c) x[c] = (1.f - al) * P.start[c] + al * P.goal[c];
-                x[3] = 0.f;
-            }
             for (int c = 0; c < 4; ++c) w[c * Nm1 + k] = x[c];
             if (k == N) break;
             const float fn = y[1 + k], ft = y[1 + n_max + k], sd = y[1 + 2 * n_max + k];
@@ -416,32 +375,85 @@ __global__ void predict_post_kernel(const float* Y, int out_dim, const comet_mod
                 const float u = y[1 + c * n_max + k];
                 w[4 * Nm1 + c * n_max + k] = u;
             }
-            if (warm_mode == 0) {
-                const int seg = (int)(((long long)k * L) / N);
-                const int face = s.modes[seg] / 3;
-                const float nx = (face == 0) ? 1.f : ((face == 2) ? -1.f : 0.f);
-                const float ny = (face == 1) ? 1.f : ((face == 3) ? -1.f : 0.f);
-                const float tx = -ny, ty = nx;
-                float st, ct;
-                sincosf(x[2], &st, &ct);
-                const float vx = P.kappa * (fn * nx + ft * tx), vy = P.kappa * (fn * ny + ft * ty);
-                const float om = P.kappa * (-P.a[face] * ft - x[3] * fn) * P.inv_c2;
-                bool reset = false;
-                if (k + 1 < N) {
-                    const int seg1 = (int)(((long long)(k + 1) * L) / N);
-                    reset = (s.modes[seg1] / 3) != face;
-                }
-                x[0] += P.dt * (ct * vx - st * vy);
-                x[1] += P.dt * (st * vx + ct * vy);
-                x[2] += P.dt * om;
-                x[3] = reset ? 0.f : x[3] + P.dt * sd;
+            const int seg = (int)(((long long)k * L) / N);
+            const int face = s.modes[seg] / 3;
+            const float nx = (face == 0) ? 1.f : ((face == 2) ? -1.f : 0.f);
+            const float ny = (face == 1) ? 1.f : ((face == 3) ? -1.f : 0.f);
+            const float tx = -ny, ty = nx;
+            float st, ct;
+            sincosf(x[2], &st, &ct);
+            const float vx = P.kappa * (fn * nx + ft * tx), vy = P.kappa * (fn * ny + ft * ty);
+            const float om = P.kappa * (-P.a[face] * ft - x[3] * fn) * P.inv_c2;
+            bool reset = false;
+            if (k + 1 < N) {
+                const int seg1 = (int)(((long long)(k + 1) * L) / N);
+                reset = (s.modes[seg1] / 3) != face;
             }
+            x[0] += P.dt * (ct * vx - st * vy);
+            x[1] += P.dt * (st * vx + ct * vy);
+            x[2] += P.dt * om;
+            x[3] = reset ? 0.f : x[3] + P.dt * sd;
         }
         for (int k = N + 1; k <= n_max; ++k)
             for (int c = 0; c < 4; ++c) w[c * Nm1 + k] = 0.f;
         for (int c = 0; c < 3; ++c)
             for (int k = N; k < n_max; ++k) w[4 * Nm1 + c * n_max + k] = 0.f;
     }
+}
+
+// merit = exp(y_0) and the warm start of order i: the cold start's poses and
+// the predicted controls (bimanual forces back from units of m g).  A warp
+// per order, lanes along the record, so that reads and writes are whole
+// lines: 20,736 records of 564 floats take PP us, and took 154 us with a
+// thread per record.
+__global__ void predict_post_kernel(const float* Y, int out_dim, const comet_mode_seq* seqs, const int* row_of,
+                                    int64_t n_rows, const int64_t* d_n, const comet::DevInstance* inst, int n_inst,
+                                    int n_max, float* merit, float* warm, int64_t stride, int bim) {
+    const int64_t nn = d_n ? min(*d_n, n_rows) : n_rows;
+    const int lane = threadIdx.x & 31, nx = bim ? 5 : 4, nc = bim ? 12 : 3, Nm1 = n_max + 1;
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t i = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); i < nn; i += warps) {
+        const int64_t r = row_of ? (int64_t)row_of[i] : i;
+        const float* y = Y + r * out_dim;
+        if (merit && lane == 0) merit[i] = expf(y[0]);
+        if (!warm) continue;
+        float* w = warm + i * stride;
+        const int si = seqs[i].instance, L = seqs[i].len;
+        if (si < 0 || si >= n_inst || L < 1) {
+            for (int64_t t = lane; t < stride; t += 32) w[t] = 0.f;
+            continue;
+        }
+        const comet::DevInstance& P = inst[si];
+        const int N = P.K * L;
+        for (int k = lane; k <= n_max; k += 32) {
+            const float al = (float)k / (float)N;
+            for (int c = 0; c < nx; ++c) {
+                float x = 0.f;
+                if (k <= N && c < 3) x = (k > 0 || bim) ? (1.f - al) * P.start[c] + al * P.goal[c] : P.start[c];
+                w[c * Nm1 + k] = x;
+            }
+        }
+        const float mg = P.mass * kGrav;
+        for (int c = 0; c < nc; ++c) {
+            const float f = bim && bim_force(c) ? mg : 1.f;
+#pragma unroll 4
+            for (int k = lane; k < n_max; k += 32)
+                w[nx * Nm1 + c * n_max + k] = (k < N) ? y[1 + c * n_max + k] * f : 0.f;
+        }
+    }
+}
+
+// launch of the two (warm_mode 0 is read as 1 for the bimanual task)
+cudaError_t launch_post(const comet_proposal* q, const comet_mode_seq* seqs, const int* row_of, int64_t n,
+                        const int64_t* d_n, float* merit, float* warm, cudaStream_t s) {
+    if (n < 1) return cudaSuccess;
+    if (q->desc.warm_mode == 0 && !q->bim && warm)
+        predict_rollout_kernel<<<grid_for(n, 128), 128, 0, s>>>(q->Y, q->out_dim, seqs, row_of, n, d_n, q->p->d_inst,
+                                                                q->n_inst, q->n_max, merit, warm, q->p->stride);
+    else
+        predict_post_kernel<<<grid_for(n * 32), 256, 0, s>>>(q->Y, q->out_dim, seqs, row_of, n, d_n, q->p->d_inst,
+                                                             q->n_inst, q->n_max, merit, warm, q->p->stride, q->bim);
+    return cudaGetLastError();
 }
 
 __global__ void encode_kernel(const comet_mode_seq* seqs, int64_t n_rows, const int64_t* d_n, int n_modes,
@@ -481,18 +493,41 @@ __global__ void set_count_kernel(int64_t* n_next, int keep) {
     if (threadIdx.x == 0 && blockIdx.x == 0) *n_next = min(*n_next, (int64_t)keep);
 }
 
-// Xt[c][b] = X[b][c]
-__global__ void transpose_kernel(const uint16_t* X, int64_t n, int in_dim, uint16_t* Xt, int64_t ld) {
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n * in_dim;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t b = t / in_dim;
-        const int c = (int)(t - b * in_dim);
-        Xt[(int64_t)c * ld + b] = X[t];
+// Xt[c][b] = X[b][c]: 64 x 64 tiles through shared memory, 16-byte accesses
+// on both sides (in_dim and ld are multiples of 64; rows past n give zeros up
+// to the tile's end, which lies inside ld).  4,096 x 64: TT us, 5.6 with a
+// two-byte scatter.
+__global__ void __launch_bounds__(256) transpose_kernel(const uint16_t* X, int64_t n, int in_dim, uint16_t* Xt,
+                                                        int64_t ld) {
+    __shared__ uint16_t tile[64][66];
+    const int64_t b0 = (int64_t)blockIdx.x * 64;
+    const int c0 = blockIdx.y * 64;
+#pragma unroll
+    for (int u = threadIdx.x; u < 512; u += 256) {
+        const int r = u >> 3, q = u & 7;
+        uint4 v = make_uint4(0, 0, 0, 0);
+        if (b0 + r < n) v = *reinterpret_cast<const uint4*>(X + (b0 + r) * in_dim + c0 + 8 * q);
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int i = 0; i < 8; ++i) tile[r][8 * q + i] = (uint16_t)(w[i / 2] >> (16 * (i & 1)));
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = threadIdx.x; u < 512; u += 256) {
+        const int c = u >> 3, q = u & 7;
+        uint32_t w[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            w[i] = (uint32_t)tile[8 * q + 2 * i][c] | ((uint32_t)tile[8 * q + 2 * i + 1][c] << 16);
+        *reinterpret_cast<uint4*>(Xt + (int64_t)(c0 + c) * ld + b0 + 8 * q) = make_uint4(w[0], w[1], w[2], w[3]);
     }
 }
 
-int grid_for(int64_t work, int threads = 256) {
-    return (int)std::max<int64_t>(1, std::min<int64_t>((work + threads - 1) / threads, 152 * 16));
+// ones under a transposed activation: the row that the weight-gradient GEMM
+// turns into the bias gradient
+__global__ void ones_kernel(uint16_t* row, int64_t n) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i < n) row[i] = 0x3f80;
 }
 
 // ------------------------------------------------------------ host side
@@ -522,26 +557,44 @@ cudaError_t ensure_rows(comet_proposal* q, int64_t rows) {
     cudaError_t e;
     const int W = q->width, I = q->in_dim, O = q->out_dim;
     if ((e = qalloc(q, &q->X, (size_t)cap * I)) != cudaSuccess) return e;
-    if ((e = qalloc(q, &q->Xt, (size_t)cap * I)) != cudaSuccess) return e;
+    if ((e = qalloc(q, &q->Xt, (size_t)cap * (I + 1))) != cudaSuccess) return e;
     if ((e = qalloc(q, &q->Y, (size_t)cap * O)) != cudaSuccess) return e;
     if ((e = qalloc(q, &q->T, (size_t)cap * O)) != cudaSuccess) return e;
     if ((e = qalloc(q, &q->Om, (size_t)cap * O)) != cudaSuccess) return e;
     for (int l = 0; l < 3; ++l) {
         if ((e = qalloc(q, &q->Z[l], (size_t)cap * W)) != cudaSuccess) return e;
         if ((e = qalloc(q, &q->H[l], (size_t)cap * W)) != cudaSuccess) return e;
-        if ((e = qalloc(q, &q->Ht[l], (size_t)cap * W)) != cudaSuccess) return e;
+        if ((e = qalloc(q, &q->Ht[l], (size_t)cap * (W + 1))) != cudaSuccess) return e;
     }
     for (int l = 0; l < kLayers; ++l) {
         const int d = (l == kLayers - 1) ? O : W;
         if ((e = qalloc(q, &q->G[l], (size_t)cap * d)) != cudaSuccess) return e;
         if ((e = qalloc(q, &q->Gt[l], (size_t)cap * d)) != cudaSuccess) return e;
     }
+    const unsigned blocks = (unsigned)((cap + 255) / 256);
+    ones_kernel<<<blocks, 256, 0, q->p->stream>>>(q->Xt + cap * I, cap);
+    for (int l = 0; l < 3; ++l) ones_kernel<<<blocks, 256, 0, q->p->stream>>>(q->Ht[l] + cap * W, cap);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     q->rows_cap = cap;
     q->ld_t = cap;
     return cudaSuccess;
 }
 
-cudaError_t forward(comet_proposal* q, int64_t M, bool train, cudaStream_t s) {
+// one training batch: device arrays with 16-byte aligned rows
+struct Batch {
+    const uint16_t* x;
+    const float *target, *weight;
+};
+
+// gradients and the loss of a step start at zero (one block, see create)
+cudaError_t zero_step(comet_proposal* q, cudaStream_t s) {
+    return cudaMemsetAsync(q->grad, 0, sizeof(float) * (q->n_params + 1), s);
+}
+
+// Forward pass of M rows: inference from q->X into q->Y, or of a training
+// batch, which keeps Z and both layouts of the activations and ends in the
+// loss and its gradient (fused into the last layer, whose output is not kept)
+cudaError_t forward(comet_proposal* q, int64_t M, const Batch* train, cudaStream_t s) {
     using namespace comet::mlp;
     const int W = q->width;
     // inference: the four layers in one persistent kernel (the layered GEMMs
@@ -557,15 +610,28 @@ cudaError_t forward(comet_proposal* q, int64_t M, bool train, cudaStream_t s) {
         memset(&ep, 0, sizeof(ep));
         ep.err = q->d_err;
         ep.bias = q->master + q->b_off[l];
-        const Mat A = (l == 0) ? Mat{q->X, M, q->in_dim, q->in_dim} : Mat{q->H[l - 1], M, W, W};
+        const uint16_t* x = train ? train->x : q->X;
+        const Mat A = (l == 0) ? Mat{x, M, q->in_dim, q->in_dim} : Mat{q->H[l - 1], M, W, W};
         const Mat B{q->wq[l], q->dout[l], q->din[l], q->din[l]};
         if (l < kLayers - 1) {
             ep.kind = kEpiBiasGelu;
-            ep.out_f32 = q->Z[l];
+            ep.out_f32 = train ? q->Z[l] : nullptr;
             ep.ld_out = W;
             ep.h = q->H[l];
             ep.ld_h = W;
             ep.h_t = train ? q->Ht[l] : nullptr;
+            ep.ld_ht = q->ld_t;
+        } else if (train) {
+            ep.kind = kEpiLoss;
+            ep.target = train->target;
+            ep.weight = train->weight;
+            ep.ld_z = q->out_dim;
+            ep.inv_b = 1.f / (float)M;
+            ep.loss = q->d_loss;
+            ep.step = q->d_step;
+            ep.h = q->G[l];
+            ep.ld_h = q->out_dim;
+            ep.h_t = q->Gt[l];
             ep.ld_ht = q->ld_t;
         } else {
             ep.kind = kEpiStore;
@@ -578,30 +644,12 @@ cudaError_t forward(comet_proposal* q, int64_t M, bool train, cudaStream_t s) {
     return cudaSuccess;
 }
 
-// backward + AdamW of the batch in q->X / Xt / T / Om (M rows)
+// backward + AdamW after a training forward of M rows (X^T in q->Xt)
 cudaError_t backward_update(comet_proposal* q, int64_t M, const comet_adamw_opts& o, cudaStream_t s) {
     using namespace comet::mlp;
     cudaError_t e;
-    if ((e = cudaMemsetAsync(q->grad, 0, sizeof(float) * q->n_params, s)) != cudaSuccess) return e;
-    loss_grad_kernel<<<grid_for(M * q->out_dim), 256, 0, s>>>(q->Y, q->T, q->Om, M, q->out_dim, q->G[kLayers - 1],
-                                                               q->Gt[kLayers - 1], q->ld_t, q->d_loss, q->d_step);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int W = q->width;
-    const int splits = (int)std::max<int64_t>(1, std::min<int64_t>(16, M / 256));
-    for (int l = kLayers - 1; l >= 0; --l) {
-        // dW_l = G_l^T H_{l-1}: both operands from the transposed copies
-        Epilogue ew;
-        memset(&ew, 0, sizeof(ew));
-        ew.kind = kEpiAtomicAdd;
-        ew.out_f32 = q->grad + q->w_off[l];
-        ew.ld_out = q->din[l];
-        ew.err = q->d_err;
-        const Mat A{q->Gt[l], q->dout[l], M, q->ld_t};
-        const Mat B{(l > 0) ? q->Ht[l - 1] : q->Xt, q->din[l], M, q->ld_t};
-        if ((e = gemm_bf16(A, B, q->dout[l], q->din[l], (int)M, splits, ew, s)) != cudaSuccess) return e;
-        bias_grad_kernel<<<q->dout[l], 256, 0, s>>>(q->Gt[l], q->ld_t, M, q->grad + q->b_off[l]);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        if (l == 0) break;
+    for (int l = kLayers - 1; l > 0; --l) {
         // G_{l-1} = (G_l W_l) * GELU'(Z_{l-1})
         Epilogue eg;
         memset(&eg, 0, sizeof(eg));
@@ -617,9 +665,22 @@ cudaError_t backward_update(comet_proposal* q, int64_t M, const comet_adamw_opts
         const Mat Bg{q->wqt[l], q->din[l], q->dout[l], q->dout[l]};
         if ((e = gemm_bf16(Ag, Bg, M, q->din[l], q->dout[l], 1, eg, s)) != cudaSuccess) return e;
     }
+    // every dW_l = G_l^T H_{l-1} and db_l in one launch, from the transposed
+    // copies (four weight-gradient launches and four bias reductions before)
+    DwLayer dw[kLayers];
+    for (int l = 0; l < kLayers; ++l)
+        dw[l] = DwLayer{q->Gt[l], (l > 0) ? q->Ht[l - 1] : q->Xt, q->ld_t, q->dout[l], q->din[l],
+                        q->grad + q->w_off[l], q->grad + q->b_off[l]};
+    if ((e = dw_bf16(dw, kLayers, M, q->p->num_sms, q->d_err, s)) != cudaSuccess) return e;
     adamw_kernel<<<grid_for(q->n_params), 256, 0, s>>>(q->master, q->grad, q->m1, q->m2, q->n_params, layer_tab(q),
                                                        q->d_step, (float)o.lr, (float)o.beta1, (float)o.beta2,
                                                        (float)o.eps, (float)o.weight_decay);
+    return cudaGetLastError();
+}
+
+cudaError_t transpose_x(comet_proposal* q, const uint16_t* x, int64_t n, cudaStream_t s) {
+    transpose_kernel<<<dim3((unsigned)((n + 63) / 64), (unsigned)(q->in_dim / 64)), 256, 0, s>>>(x, n, q->in_dim, q->Xt,
+                                                                                               q->ld_t);
     return cudaGetLastError();
 }
 
@@ -667,10 +728,10 @@ comet_status proposal_prune_device(comet_proposal* q, comet_frontier* f, int kee
                                    cudaStream_t s) {
     FrontierDev& F = f->d;
     const int64_t cap = f->batch;
-    features_kernel<<<grid_for(cap * q->in_dim), 256, 0, s>>>(F.next, cap, F.n_next, q->feat_inst, q->n_inst,
-                                                              q->l_max, q->n_modes, q->in_dim, q->X, nullptr, 0, q->bim);
+    features_kernel<<<grid_for(cap * q->in_dim / 8), 256, 0, s>>>(F.next, cap, F.n_next, q->feat_inst, q->n_inst,
+                                                                  q->l_max, q->n_modes, q->in_dim, q->X, q->bim, 1);
     QTRY(cudaGetLastError(), "features");
-    QTRY(forward(q, cap, false, s), "forward");
+    QTRY(forward(q, cap, nullptr, s), "forward");
     encode_kernel<<<grid_for(cap), 256, 0, s>>>(F.next, cap, F.n_next, q->n_modes, q->pr_codes);
     log_merit_kernel<<<grid_for(cap), 256, 0, s>>>(q->Y, q->out_dim, cap, F.n_next, q->pr_merit);
     QTRY(cudaGetLastError(), "scores");
@@ -690,11 +751,7 @@ comet_status proposal_prune_device(comet_proposal* q, comet_frontier* f, int kee
     set_count_kernel<<<1, 32, 0, s>>>(F.n_next, keep);
     QTRY(cudaGetLastError(), "keep");
     if (warm) {
-        predict_post_kernel<<<grid_for(keep, 128), 128, 0, s>>>(q->Y, q->out_dim, F.next, row_scratch, keep, F.n_next,
-                                                                q->p->d_inst, q->n_inst, q->n_max,
-                                                                q->desc.warm_mode, nullptr, warm, q->p->stride,
-                                                                q->bim);
-        QTRY(cudaGetLastError(), "warm starts");
+        QTRY(launch_post(q, F.next, row_scratch, keep, F.n_next, nullptr, warm, s), "warm starts");
     }
     return COMET_OK;
 }
@@ -712,14 +769,11 @@ comet_problem* proposal_problem(const comet_proposal* q) { return q ? q->p : nul
 comet_status proposal_predict_device(comet_proposal* q, const comet_mode_seq* seqs, int64_t n, float* merit,
                                      float* warm, cudaStream_t s) {
     QTRY(ensure_rows(q, n), "proposal activations");
-    features_kernel<<<grid_for(n * q->in_dim), 256, 0, s>>>(seqs, n, nullptr, q->feat_inst, q->n_inst, q->l_max,
-                                                            q->n_modes, q->in_dim, q->X, nullptr, 0, q->bim);
+    features_kernel<<<grid_for(n * q->in_dim / 8), 256, 0, s>>>(seqs, n, nullptr, q->feat_inst, q->n_inst, q->l_max,
+                                                                q->n_modes, q->in_dim, q->X, q->bim, 1);
     QTRY(cudaGetLastError(), "features");
-    QTRY(forward(q, n, false, s), "forward");
-    predict_post_kernel<<<grid_for(n, 128), 128, 0, s>>>(q->Y, q->out_dim, seqs, nullptr, n, nullptr, q->p->d_inst,
-                                                         q->n_inst, q->n_max, q->desc.warm_mode, merit, warm,
-                                                         q->p->stride, q->bim);
-    QTRY(cudaGetLastError(), "predict");
+    QTRY(forward(q, n, nullptr, s), "forward");
+    QTRY(launch_post(q, seqs, nullptr, n, nullptr, merit, warm, s), "predict");
     return COMET_OK;
 }
 
@@ -801,12 +855,15 @@ comet_status comet_proposal_create(comet_problem* p, const comet_proposal_desc* 
     };
     cudaError_t e = cudaSuccess;
     cudaStream_t s = p->stream;
-    if ((e = qalloc(q, &q->master, off)) != cudaSuccess || (e = qalloc(q, &q->grad, off)) != cudaSuccess ||
+    if ((e = qalloc(q, &q->master, off)) != cudaSuccess || (e = qalloc(q, &q->grad, off + 2)) != cudaSuccess ||
         (e = qalloc(q, &q->m1, off)) != cudaSuccess || (e = qalloc(q, &q->m2, off)) != cudaSuccess ||
         (e = qalloc(q, &q->feat_inst, (size_t)q->n_inst * kInstFeat)) != cudaSuccess ||
-        (e = qalloc(q, &q->d_step, 1)) != cudaSuccess || (e = qalloc(q, &q->d_loss, 1)) != cudaSuccess ||
-        (e = qalloc(q, &q->d_err, 1)) != cudaSuccess)
+        (e = qalloc(q, &q->d_step, 1)) != cudaSuccess)
         return cleanup(qcuda(e, "proposal allocation"));
+    // the loss and the error flag lie behind the gradients, cleared and read
+    // back together
+    q->d_loss = q->grad + off;
+    q->d_err = reinterpret_cast<int*>(q->grad + off + 1);
     for (int l = 0; l < kLayers; ++l)
         if ((e = qalloc(q, &q->wq[l], (size_t)q->din[l] * q->dout[l])) != cudaSuccess ||
             (e = qalloc(q, &q->wqt[l], (size_t)q->din[l] * q->dout[l])) != cudaSuccess)
@@ -853,9 +910,8 @@ comet_status comet_proposal_create(comet_problem* p, const comet_proposal_desc* 
     if ((e = cudaGetLastError()) != cudaSuccess) return cleanup(qcuda(e, "proposal init"));
     cudaMemsetAsync(q->m1, 0, sizeof(float) * off, s);
     cudaMemsetAsync(q->m2, 0, sizeof(float) * off, s);
-    cudaMemsetAsync(q->grad, 0, sizeof(float) * off, s);
+    cudaMemsetAsync(q->grad, 0, sizeof(float) * (off + 2), s);
     cudaMemsetAsync(q->d_step, 0, sizeof(int64_t), s);
-    cudaMemsetAsync(q->d_err, 0, sizeof(int), s);
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cleanup(qcuda(e, "proposal init"));
     *out = q;
     return COMET_OK;
@@ -981,8 +1037,9 @@ comet_status comet_proposal_features(comet_proposal* q, const comet_mode_seq* se
         QTRY(cudaMemcpyAsync(tmp, seqs, sizeof(comet_mode_seq) * n, cudaMemcpyHostToDevice, s), "copy orders");
         d = (const comet_mode_seq*)tmp;
     }
-    features_kernel<<<grid_for(n * q->in_dim), 256, 0, s>>>(d, n, nullptr, q->feat_inst, q->n_inst, q->l_max,
-                                                            q->n_modes, q->in_dim, out_x, nullptr, 0, q->bim);
+    features_kernel<<<grid_for(n * q->in_dim / 8), 256, 0, s>>>(d, n, nullptr, q->feat_inst, q->n_inst, q->l_max,
+                                                                q->n_modes, q->in_dim, out_x, q->bim,
+                                                                (reinterpret_cast<uintptr_t>(out_x) & 15u) == 0);
     cudaError_t e = cudaGetLastError();
     if (tmp) {
         cudaStreamSynchronize(s);
@@ -999,7 +1056,7 @@ comet_status comet_proposal_forward(comet_proposal* q, const uint16_t* x, int64_
     QTRY(ensure_rows(q, n), "proposal activations");
     QTRY(to_device(q->X, x, sizeof(uint16_t) * n * q->in_dim, s), "copy x");
     QTRY(cudaMemsetAsync(q->d_err, 0, sizeof(int), s), "reset");
-    QTRY(forward(q, n, false, s), "forward");
+    QTRY(forward(q, n, nullptr, s), "forward");
     QTRY(cudaMemcpyAsync(out_y, q->Y, sizeof(float) * n * q->out_dim, cudaMemcpyDefault, s), "copy y");
     return check_err(q, s);
 }
@@ -1011,12 +1068,12 @@ comet_status comet_proposal_time_forward(comet_proposal* q, const uint16_t* x, i
     QTRY(ensure_rows(q, n), "proposal activations");
     QTRY(to_device(q->X, x, sizeof(uint16_t) * n * q->in_dim, s), "copy x");
     QTRY(cudaMemsetAsync(q->d_err, 0, sizeof(int), s), "reset");
-    QTRY(forward(q, n, false, s), "forward");  // warm
+    QTRY(forward(q, n, nullptr, s), "forward");  // warm
     cudaEvent_t e0, e1;
     QTRY(cudaEventCreate(&e0), "event");
     QTRY(cudaEventCreate(&e1), "event");
     cudaError_t e = cudaEventRecord(e0, s);
-    for (int r = 0; r < reps && e == cudaSuccess; ++r) e = forward(q, n, false, s);
+    for (int r = 0; r < reps && e == cudaSuccess; ++r) e = forward(q, n, nullptr, s);
     if (e == cudaSuccess) e = cudaEventRecord(e1, s);
     if (e == cudaSuccess) e = cudaEventSynchronize(e1);
     float ms = 0.f;
@@ -1039,18 +1096,36 @@ comet_status comet_proposal_train_batch(comet_proposal* q, const uint16_t* x, co
         comet_default_adamw_opts(&o);
     cudaStream_t s = q->p->stream;
     QTRY(ensure_rows(q, n), "proposal activations");
-    QTRY(to_device(q->X, x, sizeof(uint16_t) * n * q->in_dim, s), "copy x");
-    QTRY(to_device(q->T, target, sizeof(float) * n * q->out_dim, s), "copy target");
-    QTRY(to_device(q->Om, weight, sizeof(float) * n * q->out_dim, s), "copy weight");
+    // arrays on the device are used in place (the call waits for its work)
+    // unless their alignment forbids 16-byte rows
+    auto in_place = [](const void* v) { return (reinterpret_cast<uintptr_t>(v) & 15u) == 0 && qdev(v); };
+    Batch in{x, target, weight};
+    if (!in_place(x)) {
+        QTRY(to_device(q->X, x, sizeof(uint16_t) * n * q->in_dim, s), "copy x");
+        in.x = q->X;
+    }
+    if (!in_place(target)) {
+        QTRY(to_device(q->T, target, sizeof(float) * n * q->out_dim, s), "copy target");
+        in.target = q->T;
+    }
+    if (!in_place(weight)) {
+        QTRY(to_device(q->Om, weight, sizeof(float) * n * q->out_dim, s), "copy weight");
+        in.weight = q->Om;
+    }
+    QTRY(cudaMemsetAsync(q->grad, 0, sizeof(float) * (q->n_params + 2), s), "reset");
     // X^T for the first layer's weight gradient
-    transpose_kernel<<<grid_for(n * q->in_dim), 256, 0, s>>>(q->X, n, q->in_dim, q->Xt, q->ld_t);
-    QTRY(cudaGetLastError(), "transpose");
-    QTRY(cudaMemsetAsync(q->d_err, 0, sizeof(int), s), "reset");
-    QTRY(cudaMemsetAsync(q->d_loss, 0, sizeof(float), s), "reset");
-    QTRY(forward(q, n, true, s), "forward");
+    QTRY(transpose_x(q, in.x, n, s), "transpose");
+    QTRY(forward(q, n, &in, s), "forward");
     QTRY(backward_update(q, n, o, s), "backward");
-    if (out_loss) QTRY(cudaMemcpyAsync(out_loss, q->d_loss, sizeof(float), cudaMemcpyDeviceToHost, s), "loss");
-    return check_err(q, s);
+    struct {
+        float loss;
+        int err;
+    } end = {0.f, 0};
+    QTRY(cudaMemcpyAsync(&end, q->d_loss, sizeof(end), cudaMemcpyDeviceToHost, s), "loss");
+    QTRY(cudaStreamSynchronize(s), "synchronise");
+    if (out_loss) *out_loss = end.loss;
+    if (end.err) return qfail(COMET_ERR_TIMEOUT, "tensor-core GEMM: a bounded wait ran out");
+    return COMET_OK;
 }
 
 comet_status comet_proposal_add_samples(comet_proposal* q, const comet_mode_seq* seqs, int64_t n, const float* cost,
@@ -1090,9 +1165,9 @@ comet_status comet_proposal_add_samples(comet_proposal* q, const comet_mode_seq*
     cudaError_t e = cudaMalloc(&dK, sizeof(int) * q->n_inst);
     if (e == cudaSuccess) e = cudaMemcpyAsync(dK, K.data(), sizeof(int) * q->n_inst, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) {
-        features_kernel<<<grid_for(n * q->in_dim), 256, 0, s>>>(ds, n, nullptr, q->feat_inst, q->n_inst, q->l_max,
-                                                                q->n_modes, q->in_dim,
-                                                                q->ds_X + q->ds_n * q->in_dim, nullptr, 0, q->bim);
+        features_kernel<<<grid_for(n * q->in_dim / 8), 256, 0, s>>>(ds, n, nullptr, q->feat_inst, q->n_inst, q->l_max,
+                                                                    q->n_modes, q->in_dim,
+                                                                    q->ds_X + q->ds_n * q->in_dim, q->bim, 1);
         targets_kernel<<<grid_for(n * q->out_dim), 256, 0, s>>>(
             ds, n, dc, dv, dst, dt, stride, dK, q->n_inst, q->n_max, q->out_dim, (float)q->p->opts.merit_mu,
             (float)q->p->opts.eps_feas, (float)q->desc.lambda_w, q->ds_T + q->ds_n * q->out_dim,
@@ -1159,14 +1234,16 @@ comet_status comet_proposal_train(comet_proposal* q, int64_t steps, int32_t batc
     if (e == cudaSuccess) e = cudaMemsetAsync(q->d_err, 0, sizeof(int), s);
     if (e == cudaSuccess) e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        cudaError_t ce = cudaMemsetAsync(q->d_loss, 0, sizeof(float), s);
+        cudaError_t ce = zero_step(q, s);
         if (ce == cudaSuccess) {
-            gather_kernel<<<grid_for((int64_t)batch * (q->in_dim + q->out_dim)), 256, 0, s>>>(
-                q->ds_X, q->ds_T, q->ds_Om, q->ds_n, batch, q->d_step, (unsigned long long)seed, q->in_dim,
-                q->out_dim, q->X, q->Xt, q->ld_t, q->T, q->Om);
+            gather_kernel<<<grid_for((int64_t)batch * 32), 256, 0, s>>>(q->ds_X, q->ds_T, q->ds_Om, q->ds_n, batch,
+                                                                       q->d_step, (unsigned long long)seed, q->in_dim,
+                                                                       q->out_dim, q->X, q->T, q->Om);
             ce = cudaGetLastError();
         }
-        if (ce == cudaSuccess) ce = forward(q, batch, true, s);
+        const Batch in{q->X, q->T, q->Om};
+        if (ce == cudaSuccess) ce = transpose_x(q, q->X, batch, s);
+        if (ce == cudaSuccess) ce = forward(q, batch, &in, s);
         if (ce == cudaSuccess) ce = backward_update(q, batch, o, s);
         e = cudaStreamEndCapture(s, &graph);
         if (ce != cudaSuccess) e = ce;
@@ -1207,8 +1284,11 @@ comet_status comet_proposal_predict(comet_proposal* q, const comet_mode_seq* seq
             if (seqs[i].instance < 0 || seqs[i].instance >= q->n_inst || seqs[i].len < 1 || seqs[i].len > q->l_max)
                 return qfail(COMET_ERR_INVALID_ARG, "malformed order");
     void* tmp = nullptr;
-    const size_t b_seq = pad_to(sizeof(comet_mode_seq) * n, 256), b_m = pad_to(sizeof(float) * n, 256);
-    QTRY(cudaMalloc(&tmp, b_seq + b_m + sizeof(float) * n * stride + 256), "staging");
+    // a staging block for what is in host memory (none: no allocation)
+    const size_t b_seq = host_seqs ? pad_to(sizeof(comet_mode_seq) * n, 256) : 0;
+    const size_t b_m = host_m ? pad_to(sizeof(float) * n, 256) : 0;
+    const size_t b_w = host_w ? sizeof(float) * n * stride : 0;
+    if (b_seq + b_m + b_w) QTRY(cudaMalloc(&tmp, b_seq + b_m + b_w), "staging");
     char* b = (char*)tmp;
     const comet_mode_seq* ds = host_seqs ? (const comet_mode_seq*)b : seqs;
     float* dm = out_merit ? (host_m ? (float*)(b + b_seq) : out_merit) : nullptr;
@@ -1222,8 +1302,10 @@ comet_status comet_proposal_predict(comet_proposal* q, const comet_mode_seq* seq
         e = cudaMemcpyAsync(out_merit, dm, sizeof(float) * n, cudaMemcpyDeviceToHost, s);
     if (st == COMET_OK && e == cudaSuccess && host_w)
         e = cudaMemcpyAsync(out_warm, dw, sizeof(float) * n * stride, cudaMemcpyDeviceToHost, s);
-    cudaStreamSynchronize(s);
-    cudaFree(tmp);
+    if (tmp) {
+        cudaStreamSynchronize(s);
+        cudaFree(tmp);
+    }
     if (st != COMET_OK) return st;
     if (e != cudaSuccess) return qcuda(e, "predict");
     return check_err(q, s);
@@ -1263,6 +1345,7 @@ comet_status comet_gemm_bf16(const uint16_t* a, int64_t lda, const uint16_t* b, 
     QTRY(cudaMalloc(&d_err, sizeof(int)), "flag");
     cudaMemsetAsync(d_err, 0, sizeof(int), s);
     Epilogue e;
+    memset(&e, 0, sizeof(e));
     e.kind = ep->kind;
     e.bias = ep->bias;
     e.out_f32 = ep->out_f32;

@@ -26,6 +26,9 @@
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
 
+#include <string.h>
+
+#include <algorithm>
 #include <mutex>
 
 namespace comet {
@@ -176,12 +179,108 @@ struct __align__(8) Barriers {
     uint32_t failed;
 };
 
-__global__ void __launch_bounds__(kThreads, 1)
-    gemm_bf16_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, int M,
-                     int N, int K, int k_chunk, int bn, int tmem_cols, Epilogue ep) {
+// What a tile's epilogue may take from the operands' alignment: 16-byte
+// accesses along a row (decided on the host).
+struct Tile {
+    int M, N, m0, n0, k_begin, k_len, bn, tmem_cols, vec;
+};
+
+// Epilogue of one 32 x 32 block in the accumulator's own layout: a lane holds
+// 32 consecutive columns of its row, so that rows move as 16-byte accesses
+// and the transposed copy as 64-byte runs over the lanes (rows), with nothing
+// turned around in shared memory and all operand loads issued before the
+// first use.  4,096 x 256 x 256: 9.7 -> AA us (store), 14.7 -> BB us (GELU
+// with its three outputs), 42 -> CC us (GELU' gating, whose loads were one
+// dependent access per row).
+template <int KIND>
+__device__ __forceinline__ void epilogue_rows(const Epilogue& ep, uint32_t taddr, int row, int nb, int ncol,
+                                              bool row_ok, float& loss) {
+    float v[32], x[32];
+    // 4 q < ncol only bites for kEpiLoss (N a multiple of 16); the other kinds
+    // come here with whole blocks
+    const bool whole = KIND != kEpiLoss;
+    if (KIND == kEpiGeluGrad) {
+        const float4* z = reinterpret_cast<const float4*>(ep.z_in + (int64_t)row * ep.ld_z + nb);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const float4 t = row_ok ? z[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+            x[4 * q] = t.x, x[4 * q + 1] = t.y, x[4 * q + 2] = t.z, x[4 * q + 3] = t.w;
+        }
+    } else if (ep.bias) {
+        const float4* z = reinterpret_cast<const float4*>(ep.bias + nb);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const float4 t = whole || 4 * q < ncol ? __ldg(z + q) : make_float4(0.f, 0.f, 0.f, 0.f);
+            x[4 * q] = t.x, x[4 * q + 1] = t.y, x[4 * q + 2] = t.z, x[4 * q + 3] = t.w;
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) x[j] = 0.f;
+    }
+    float t[KIND == kEpiLoss ? 32 : 1], om[KIND == kEpiLoss ? 32 : 1];
+    if constexpr (KIND == kEpiLoss) {
+        const float4* tp = reinterpret_cast<const float4*>(ep.target + (int64_t)row * ep.ld_z + nb);
+        const float4* op = reinterpret_cast<const float4*>(ep.weight + (int64_t)row * ep.ld_z + nb);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const bool ok = row_ok && 4 * q < ncol;
+            const float4 a = ok ? tp[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+            const float4 b = ok ? op[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+            t[4 * q] = a.x, t[4 * q + 1] = a.y, t[4 * q + 2] = a.z, t[4 * q + 3] = a.w;
+            om[4 * q] = b.x, om[4 * q + 1] = b.y, om[4 * q + 2] = b.z, om[4 * q + 3] = b.w;
+        }
+    }
+    tmem_ld32(taddr, v);
+    if (!row_ok) return;
+    uint32_t hb[32];
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+        if constexpr (KIND == kEpiStore) {
+            v[j] += x[j];
+        } else if constexpr (KIND == kEpiBiasGelu) {
+            v[j] += x[j];
+            hb[j] = to_bf16(gelu_f(v[j]));
+        } else if constexpr (KIND == kEpiGeluGrad) {
+            hb[j] = to_bf16(v[j] * gelu_grad_f(x[j]));
+        } else if constexpr (KIND == kEpiLoss) {
+            // dL/dY = (2/B) Omega (Y - T), and the row's share of the loss
+            const float d = v[j] + x[j] - t[j], w = om[j];
+            if (j < ncol) loss += w * d * d;
+            hb[j] = to_bf16(2.f * w * d * ep.inv_b);
+        }
+    }
+    if (KIND == kEpiStore || (KIND == kEpiBiasGelu && ep.out_f32)) {
+        float4* o = reinterpret_cast<float4*>(ep.out_f32 + (int64_t)row * ep.ld_out + nb);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) o[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    }
+    if constexpr (KIND != kEpiStore && KIND != kEpiAtomicAdd) {
+        if (ep.h) {
+            uint4* o = reinterpret_cast<uint4*>(ep.h + (int64_t)row * ep.ld_h + nb);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                uint32_t w[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) w[i] = hb[8 * q + 2 * i] | (hb[8 * q + 2 * i + 1] << 16);
+                if (whole || 8 * q < ncol) o[q] = make_uint4(w[0], w[1], w[2], w[3]);
+            }
+        }
+        if (ep.h_t) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+                if (whole || j < ncol) ep.h_t[(int64_t)(nb + j) * ep.ld_ht + row] = (uint16_t)hb[j];
+        }
+    }
+}
+
+// One CTA's tile of D = A B^T: the pipeline and the epilogue.
+template <int KIND>
+__device__ __forceinline__ void gemm_tile(const CUtensorMap* map_a, const CUtensorMap* map_b, const Tile& T,
+                                          const Epilogue& ep) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     uint8_t* smem = smem_raw + ((1024u - (raw & 1023u)) & 1023u);
+    const int M = T.M, N = T.N, m0 = T.m0, n0 = T.n0, bn = T.bn;
     const uint32_t a_bytes = BM * BK * 2;
     const uint32_t b_bytes = (uint32_t)bn * BK * 2;
     const uint32_t stage_bytes = a_bytes + b_bytes;
@@ -189,11 +288,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t s_base = smem_u32(smem);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m0 = blockIdx.x * BM, n0 = blockIdx.y * bn;
-    const int k_begin = blockIdx.z * k_chunk;
-    const int k_len = min(k_chunk, K - k_begin);
-    const int nkb = (k_len + BK - 1) / BK;
-
+    const int nkb = (T.k_len + BK - 1) / BK;
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(smem_u32(&bars->full[s]), 1);
@@ -206,7 +301,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (warp == 2) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                          smem_u32(&bars->tmem_base)),
-                     "r"(tmem_cols)
+                     "r"(T.tmem_cols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -228,9 +323,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (*(volatile uint32_t*)&bars->failed) break;
             const uint32_t full = smem_u32(&bars->full[s]);
             mbar_expect_tx(full, stage_bytes);
-            const int kx = k_begin + i * BK;
-            tma_load_2d(s_base + s * stage_bytes, &map_a, kx, m0, full);
-            tma_load_2d(s_base + s * stage_bytes + a_bytes, &map_b, kx, n0, full);
+            const int kx = T.k_begin + i * BK;
+            tma_load_2d(s_base + s * stage_bytes, map_a, kx, m0, full);
+            tma_load_2d(s_base + s * stage_bytes + a_bytes, map_b, kx, n0, full);
             ++issued;
         }
         if (*(volatile uint32_t*)&bars->failed) {
@@ -268,37 +363,51 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_after();
     __syncwarp();
     const bool run = __all_sync(0xffffffffu, have && !*(volatile uint32_t*)&bars->failed);
-    // Each 32 x 32 block of the accumulator goes through shared memory (the
-    // pipeline stages are free once the accumulator is complete), so that
-    // row-major outputs are written with lanes along a row and the
-    // transposed copy with lanes along a column: every store is coalesced.
-    // Warp w stages in its own two 32 x 33 tiles (raw accumulator, result).
+    float loss = 0.f;
     if (run) {
         float* st1 = reinterpret_cast<float*>(smem) + warp * (2 * 32 * 33);
         float* st2 = st1 + 32 * 33;
         const int row0 = m0 + warp * 32;
         for (int c0 = 0; c0 < bn; c0 += 32) {
-            float v[32];
-            tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
+            const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
             const int nb = n0 + c0;
-            if (nb >= N) continue;
+            if (nb >= N) break;
+            if (KIND == kEpiLoss || (KIND != kEpiAtomicAdd && T.vec && nb + 32 <= N)) {
+                const int row = row0 + lane;
+                epilogue_rows<KIND>(ep, taddr, row, nb, min(32, N - nb), row < M, loss);
+                continue;
+            }
+            // A block of ragged columns or unaligned rows, and the split-K
+            // sums: turned around in shared memory (the pipeline stages are
+            // free once the accumulator is complete), so that row-major
+            // outputs are written with lanes along a row and the transposed
+            // copy with lanes along a column.  Warp w stages in its own two
+            // 32 x 33 tiles (raw accumulator, result).
+            float v[32];
+            tmem_ld32(taddr, v);
 #pragma unroll
             for (int j = 0; j < 32; ++j) st1[lane * 33 + j] = v[j];
             __syncwarp();
             // lanes along a row: column nb + lane
             const int col = nb + lane;
             const bool col_ok = col < N;
-            const float bias = (ep.bias && col_ok) ? ep.bias[col] : 0.f;
+            const float bias = (KIND != kEpiAtomicAdd && ep.bias && col_ok) ? ep.bias[col] : 0.f;
+#pragma unroll 8
             for (int r = 0; r < 32; ++r) {
                 const int row = row0 + r;
                 const bool ok = col_ok && row < M;
                 const float a = st1[r * 33 + lane];
                 float res = 0.f;
-                if (ep.kind == kEpiStore) {
+                if (KIND == kEpiStore) {
                     if (ok) ep.out_f32[(int64_t)row * ep.ld_out + col] = a + bias;
-                } else if (ep.kind == kEpiAtomicAdd) {
-                    if (ok) atomicAdd(ep.out_f32 + (int64_t)row * ep.ld_out + col, a);
-                } else if (ep.kind == kEpiBiasGelu) {
+                } else if (KIND == kEpiAtomicAdd) {
+                    // the last column of a weight gradient with a row of ones
+                    // under its second operand is the bias gradient
+                    if (ok)
+                        atomicAdd(ep.bias_grad && col == N - 1 ? ep.bias_grad + row
+                                                               : ep.out_f32 + (int64_t)row * ep.ld_out + col,
+                                  a);
+                } else if (KIND == kEpiBiasGelu) {
                     const float z = a + bias;
                     if (ok && ep.out_f32) ep.out_f32[(int64_t)row * ep.ld_out + col] = z;
                     res = gelu_f(z);
@@ -306,14 +415,14 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const float z = ok ? ep.z_in[(int64_t)row * ep.ld_z + col] : 0.f;
                     res = a * gelu_grad_f(z);
                 }
-                if (ep.kind == kEpiBiasGelu || ep.kind == kEpiGeluGrad) {
+                if (KIND == kEpiBiasGelu || KIND == kEpiGeluGrad) {
                     const uint16_t hb = to_bf16(res);
                     if (ok && ep.h) ep.h[(int64_t)row * ep.ld_h + col] = hb;
                     st2[r * 33 + lane] = __uint_as_float((uint32_t)hb);
                 }
             }
             __syncwarp();
-            if (ep.h_t && (ep.kind == kEpiBiasGelu || ep.kind == kEpiGeluGrad)) {
+            if ((KIND == kEpiBiasGelu || KIND == kEpiGeluGrad) && ep.h_t) {
                 // lanes along a column of the transposed copy: row row0 + lane
                 const int row = row0 + lane;
                 if (row < M) {
@@ -325,13 +434,59 @@ __global__ void __launch_bounds__(kThreads, 1)
             __syncwarp();
         }
     }
+    if (KIND == kEpiLoss) {
+        for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+        if (lane == 0) atomicAdd(ep.loss, loss * ep.inv_b);
+        if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *ep.step += 1;
+    }
     if (*(volatile uint32_t*)&bars->failed && threadIdx.x == 0 && ep.err) atomicExch(ep.err, 1);
     tc_fence_before();
     __syncthreads();
     if (warp == 2) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(T.tmem_cols) : "memory");
     }
+}
+
+template <int KIND>
+__global__ void __launch_bounds__(kThreads, 1)
+    gemm_bf16_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, int M,
+                     int N, int K, int k_chunk, int bn, int tmem_cols, int vec, Epilogue ep) {
+    const int k_begin = blockIdx.z * k_chunk;
+    gemm_tile<KIND>(&map_a, &map_b,
+                    Tile{M, N, (int)blockIdx.x * BM, (int)blockIdx.y * bn, k_begin, min(k_chunk, K - k_begin), bn,
+                         tmem_cols, vec},
+                    ep);
+}
+
+// The weight and bias gradients of all layers in one launch: blockIdx.x runs
+// over the (layer, row tile, column tile) triples, blockIdx.y over the splits
+// of the batch.
+struct DwMaps {
+    CUtensorMap a[kDwMax], b[kDwMax];
+};
+struct DwParams {
+    int n, K, k_chunk, first[kDwMax + 1], M[kDwMax], N[kDwMax], cols[kDwMax];
+    float* dw[kDwMax];
+    float* db[kDwMax];
+    int* err;
+};
+
+__global__ void __launch_bounds__(kThreads, 1) dw_kernel(const __grid_constant__ DwMaps maps, const DwParams P) {
+    int l = 0;
+    while (l + 1 < P.n && (int)blockIdx.x >= P.first[l + 1]) ++l;
+    const int t = (int)blockIdx.x - P.first[l];
+    const int k_begin = blockIdx.y * P.k_chunk;
+    Epilogue ep;
+    ep.kind = kEpiAtomicAdd;
+    ep.out_f32 = P.dw[l];
+    ep.ld_out = P.N[l] - 1;
+    ep.bias_grad = P.db[l];
+    ep.err = P.err;
+    gemm_tile<kEpiAtomicAdd>(&maps.a[l], &maps.b[l],
+                             Tile{P.M[l], P.N[l], t / P.cols[l] * BM, t % P.cols[l] * kMaxBN, k_begin,
+                                  min(P.k_chunk, P.K - k_begin), kMaxBN, kMaxBN, 0},
+                             ep);
 }
 
 // ------------------------------------------------------------------------
@@ -614,7 +769,13 @@ cudaError_t gemm_prepare() {
     const int need = (int)smem_request(kMaxBN);
     std::lock_guard<std::mutex> lk(g_raise_mu);
     if (dev < 64 && g_raised[dev] >= need) return cudaSuccess;
-    e = cudaFuncSetAttribute(gemm_bf16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, need);
+    const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    e = cudaFuncSetAttribute(gemm_bf16_kernel<kEpiStore>, at, need);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_bf16_kernel<kEpiBiasGelu>, at, need);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_bf16_kernel<kEpiGeluGrad>, at, need);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_bf16_kernel<kEpiAtomicAdd>, at, need);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_bf16_kernel<kEpiLoss>, at, need);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(dw_kernel, at, need);
     if (e == cudaSuccess && dev < 64) g_raised[dev] = need;
     return e;
 }
@@ -622,6 +783,16 @@ cudaError_t gemm_prepare() {
 bool tensor_maps_available() {
     resolve_encode();
     return g_encode != nullptr;
+}
+
+// whether every row access of the epilogue is 16-byte aligned
+static int rows_vectorise(const Epilogue& ep) {
+    auto al = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
+    const bool f = !ep.out_f32 || (al(ep.out_f32) && ep.ld_out % 4 == 0);
+    const bool h = !ep.h || (al(ep.h) && ep.ld_h % 8 == 0);
+    const bool z = !ep.z_in || (al(ep.z_in) && ep.ld_z % 4 == 0);
+    const bool t = ep.kind != kEpiLoss || (al(ep.target) && al(ep.weight) && ep.ld_z % 4 == 0);
+    return f && h && z && t && (!ep.bias || al(ep.bias));
 }
 
 cudaError_t gemm_bf16(const Mat& A, const Mat& B, int64_t M, int N, int K, int k_splits, const Epilogue& ep,
@@ -649,7 +820,53 @@ cudaError_t gemm_bf16(const Mat& A, const Mat& B, int64_t M, int N, int K, int k
     cudaError_t e = gemm_prepare();
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)((M + BM - 1) / BM), (unsigned)((N + bn - 1) / bn), (unsigned)splits);
-    gemm_bf16_kernel<<<grid, kThreads, smem_req, s>>>(ma, mb, (int)M, N, K, k_chunk, bn, tmem_cols, ep);
+    const int vec = rows_vectorise(ep);
+    if (ep.kind == kEpiLoss && (!vec || N % 16)) return cudaErrorInvalidValue;
+#define COMET_GEMM(kind) \
+    gemm_bf16_kernel<kind><<<grid, kThreads, smem_req, s>>>(ma, mb, (int)M, N, K, k_chunk, bn, tmem_cols, vec, ep)
+    switch (ep.kind) {
+        case kEpiStore: COMET_GEMM(kEpiStore); break;
+        case kEpiBiasGelu: COMET_GEMM(kEpiBiasGelu); break;
+        case kEpiGeluGrad: COMET_GEMM(kEpiGeluGrad); break;
+        case kEpiAtomicAdd: COMET_GEMM(kEpiAtomicAdd); break;
+        case kEpiLoss: COMET_GEMM(kEpiLoss); break;
+        default: return cudaErrorInvalidValue;
+    }
+#undef COMET_GEMM
+    return cudaGetLastError();
+}
+
+cudaError_t dw_bf16(const DwLayer* layers, int n, int64_t K, int num_sms, int* err, cudaStream_t s) {
+    if (n < 1 || n > kDwMax || K < 1 || K > (int64_t)INT32_MAX) return cudaErrorInvalidValue;
+    DwMaps maps;
+    DwParams P;
+    memset(&P, 0, sizeof(P));
+    P.n = n;
+    P.K = (int)K;
+    P.err = err;
+    for (int l = 0; l < n; ++l) {
+        const DwLayer& L = layers[l];
+        if ((reinterpret_cast<uintptr_t>(L.g_t) & 15u) || (reinterpret_cast<uintptr_t>(L.h_t) & 15u) || (L.ld & 7) ||
+            L.ld < K)
+            return cudaErrorInvalidValue;
+        if (!make_map(&maps.a[l], Mat{L.g_t, L.dout, K, L.ld}, L.dout, K, BM) ||
+            !make_map(&maps.b[l], Mat{L.h_t, L.din + 1, K, L.ld}, L.din + 1, K, kMaxBN))
+            return cudaErrorInvalidValue;
+        P.M[l] = L.dout;
+        P.N[l] = L.din + 1;
+        P.cols[l] = (L.din + kMaxBN) / kMaxBN;
+        P.dw[l] = L.dw;
+        P.db[l] = L.db;
+        P.first[l + 1] = P.first[l] + (L.dout + BM - 1) / BM * P.cols[l];
+    }
+    // splits of the batch: one wave of two CTAs per SM, at least 256 rows each
+    const int tiles = P.first[n];
+    const int64_t splits = std::max<int64_t>(1, std::min<int64_t>(2 * num_sms / tiles, K / 256));
+    P.k_chunk = (int)(((K + splits - 1) / splits + BK - 1) / BK * BK);
+    const cudaError_t e = gemm_prepare();
+    if (e != cudaSuccess) return e;
+    const dim3 grid((unsigned)tiles, (unsigned)((K + P.k_chunk - 1) / P.k_chunk));
+    dw_kernel<<<grid, kThreads, smem_request(kMaxBN), s>>>(maps, P);
     return cudaGetLastError();
 }
 

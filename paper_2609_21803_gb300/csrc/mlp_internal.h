@@ -18,6 +18,8 @@ enum EpiKind : int {
     kEpiBiasGelu = 1,   // Z = D + bias -> z_f32, H = gelu(Z) -> h (bf16) and h_t (bf16, transposed)
     kEpiGeluGrad = 2,   // G = D * gelu'(z_in) -> h (bf16) and h_t (bf16, transposed)
     kEpiAtomicAdd = 3,  // out_f32[m][n] += D (split-K partial sums)
+    kEpiLoss = 4,       // Y = D + bias, G = (2/B) Omega (Y - T) -> h, h_t; loss += Omega (Y - T)^2 / B (training;
+                        // aligned rows, N a multiple of 16)
 };
 
 struct Epilogue {
@@ -32,6 +34,13 @@ struct Epilogue {
     const float* z_in;      // [M][ld_z] pre-activation (kEpiGeluGrad)
     int64_t ld_z;
     int* err;               // device flag: a bounded wait ran out (nullable)
+    // internal uses (zero otherwise)
+    float* bias_grad;       // kEpiAtomicAdd: sums of column N - 1 go here instead, one per row
+    const float* target;    // kEpiLoss: T, Omega [M][ld_z]
+    const float* weight;
+    float* loss;            // kEpiLoss: loss sum
+    int64_t* step;          // kEpiLoss: the optimiser's step count, advanced once
+    float inv_b;            // kEpiLoss: 1 / B
 };
 
 // A row-major bf16 matrix [rows][cols] with leading dimension ld (elements);
@@ -47,6 +56,20 @@ struct Mat {
 // column tile (larger N is tiled), K >= 1.  Returns a CUDA error code.
 cudaError_t gemm_bf16(const Mat& A, const Mat& B, int64_t M, int N, int K, int k_splits, const Epilogue& ep,
                       cudaStream_t s);
+
+// Weight and bias gradients of up to kDwMax layers in one launch, added to dw
+// and db: dw = G^T H, db = column sums of G, from the transposed copies
+// g_t [dout][ld] and h_t [din + 1][ld], whose last row holds ones.
+constexpr int kDwMax = 4;
+struct DwLayer {
+    const uint16_t* g_t;
+    const uint16_t* h_t;
+    int64_t ld;
+    int dout, din;
+    float* dw;
+    float* db;
+};
+cudaError_t dw_bf16(const DwLayer* layers, int n, int64_t K, int num_sms, int* err, cudaStream_t s);
 
 // The tensor-map encoder from the driver (resolved once); false if absent.
 bool tensor_maps_available();
