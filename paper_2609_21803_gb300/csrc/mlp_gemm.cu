@@ -189,8 +189,8 @@ struct Tile {
 // 32 consecutive columns of its row, so that rows move as 16-byte accesses
 // and the transposed copy as 64-byte runs over the lanes (rows), with nothing
 // turned around in shared memory and all operand loads issued before the
-// first use.  4,096 x 256 x 256: 9.7 -> AA us (store), 14.7 -> BB us (GELU
-// with its three outputs), 42 -> CC us (GELU' gating, whose loads were one
+// first use.  A training step of 4,096 rows, per launch: 14.7 -> 9.0 us (GELU
+// with its three outputs), 42 -> 9.5 us (GELU' gating, whose loads were one
 // dependent access per row).
 template <int KIND>
 __device__ __forceinline__ void epilogue_rows(const Epilogue& ep, uint32_t taddr, int row, int nb, int ncol,
@@ -490,26 +490,38 @@ __global__ void __launch_bounds__(kThreads, 1) dw_kernel(const __grid_constant__
 }
 
 // ------------------------------------------------------------------------
-// Fused forward pass of the 4-layer MLP (in_dim <= 128, width 256, out_dim
-// <= 256): one persistent CTA per SM walks 128-row tiles; the four layers
-// are chained through one 256-column TMEM accumulator and a 64 KB
-// activation tile in shared memory, so a tile never leaves the SM between
-// layers.  Warps 0..15: epilogue (warp w reads TMEM lanes 32 (w mod 4).. and
-// columns 64 (w / 4)..), writing bias + GELU as BF16 into the activation
+// Fused forward pass of the 4-layer MLP (in_dim <= 256, width 256, any
+// out_dim): persistent CTAs walk units of a 128-row tile and a share of the
+// output's 256-column blocks; the layers are chained through two 256-column
+// TMEM accumulators and a 64 KB activation tile in shared memory, so a tile
+// never leaves the SM between layers.  Warps 0..15: epilogue (warp w reads
+// TMEM lanes 32 (w mod 4)..); warp 16, one lane: TMA producer (the X tile,
+// and the weights as 64-column K slices of 256 rows through a ring); warp 17,
+// one lane: MMA issuer.
+//
+// A hidden layer's epilogue writes bias + GELU as BF16 into the activation
 // tile in the 128-byte-swizzled K-major layout the next tcgen05.mma reads
-// (16-byte chunk c of row r at chunk c ^ (r mod 8)); warp 16, one lane: TMA
-// producer (the X tile, and the weights as 64-column K slices of 256 rows
-// through a 3-stage ring); warp 17, one lane: MMA issuer.
+// (16-byte chunk c of row r at chunk c ^ (r mod 8)), one 64-column K slice
+// after the other over all 16 warps (16 columns each); the next layer's MMAs
+// start on a slice as soon as it is ready, into the other accumulator, so
+// that a layer costs its epilogue and one slice's MMA instead of the sum of
+// both.  An output block's MMAs run under the previous block's stores.  What
+// bounds a tile is the epilogue's FP32 arithmetic (GELU on pairs of values by
+// f32x2 instructions, results unchanged).  20,736 rows 64 -> 256: 40 us with
+// one accumulator, scalar GELU and layers in sequence, 29 us now.  The box
+// flip's 192 -> 1,088 (8,192 rows) took 51 us as four GEMM launches, 24 us
+// now; with fewer tiles than SMs the output blocks are split over CTAs, each
+// repeating the hidden layers (cheaper than idle SMs).
 
 constexpr int kFEpiWarps = 16;
 constexpr int kFThreads = (kFEpiWarps + 2) * 32;
-constexpr int kFEpilogue = kFEpiWarps * 32;  // threads of the epilogue warps
-constexpr int kFRing = 3;
+constexpr int kFRing = 3;                    // weight slices in flight (2 when in_dim > 192)
 constexpr uint32_t kWStage = 256 * BK * 2;   // 32 KB: one K slice of a weight
 constexpr uint32_t kXBlock = BM * BK * 2;    // 16 KB: one K slice of a tile
 
 struct __align__(8) FusedBars {
-    uint64_t x_full, x_free, acc_full, h_ready;
+    uint64_t x_full, x_free, drain;
+    uint64_t acc_full[2], acc_free[2], h_ready[4];
     uint64_t w_full[kFRing], w_empty[kFRing];
     uint32_t tmem_base, failed;
 };
@@ -518,38 +530,100 @@ struct FusedParams {
     const float* bias[4];
     float* y;
     int64_t ld_y;
-    int M, in_dim, out_dim;
+    int M, in_dim, out_dim, ring, nsplit;
     int* err;
 };
+
+// Bounded wait that also ends when another role of the CTA has given up.
+__device__ __forceinline__ bool fused_wait(uint32_t bar, uint32_t parity, volatile uint32_t* failed) {
+    if (mbar_try_wait(bar, parity)) return true;
+    const long long t0 = clock64();
+    for (;;) {
+        if (mbar_try_wait(bar, parity)) return true;
+        if (*failed) return false;
+        if (clock64() - t0 > kWaitCycles) return false;
+    }
+}
+
+// 16 consecutive FP32 columns of this thread's TMEM lane (no wait)
+__device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t r[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+}
+
+// two FP32 values in one register pair
+__device__ __forceinline__ uint64_t f2(float a, float b) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void f2_get(uint64_t v, float& a, float& b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// BF16 pair of gelu_f(v + bias) for two values, the same operations as
+// gelu_f in the same order
+__device__ __forceinline__ uint32_t gelu_pair(uint64_t v, uint64_t bias) {
+    const uint64_t x = f2_add(v, bias);
+    const uint64_t u = f2_mul(f2_mul(f2(kGeluB, kGeluB), x), x);
+    float a, b;
+    f2_get(f2_mul(f2(kGeluA, kGeluA), f2_fma(u, x, x)), a, b);
+    const uint64_t t = f2_add(f2(1.f, 1.f), f2(tanh_hw(a), tanh_hw(b)));
+    f2_get(f2_mul(f2_mul(f2(0.5f, 0.5f), x), t), a, b);
+    uint32_t pk;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(pk) : "f"(b), "f"(a));
+    return pk;
+}
 
 __global__ void __launch_bounds__(kFThreads, 1)
     mlp_fused_forward_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w0,
                              const __grid_constant__ CUtensorMap map_w1, const __grid_constant__ CUtensorMap map_w2,
-                             const __grid_constant__ CUtensorMap map_w3, FusedParams fp) {
+                             const __grid_constant__ CUtensorMap map_w3, const FusedParams fp) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     uint8_t* smem = smem_raw + ((1024u - (raw & 1023u)) & 1023u);
-    const int n_xkb = fp.in_dim / BK;                       // 1 or 2 K slices of X
-    uint8_t* xs = smem;                                     // n_xkb x 16 KB
-    uint8_t* hs = xs + 2 * kXBlock;                         // 4 x 16 KB activations
-    uint8_t* ws = hs + 4 * kXBlock;                         // kFRing x 32 KB weights
-    float* bs = reinterpret_cast<float*>(ws + kFRing * kWStage);  // 4 x 256 biases
-    FusedBars* bars = reinterpret_cast<FusedBars*>(bs + 4 * 256);
+    const int n_xkb = fp.in_dim / BK;                             // 1..4 K slices of X
+    const int ring = fp.ring;
+    uint8_t* xs = smem;                                           // n_xkb x 16 KB
+    uint8_t* hs = xs + n_xkb * kXBlock;                           // 4 x 16 KB activations
+    uint8_t* ws = hs + 4 * kXBlock;                               // ring x 32 KB weights
+    float* bs = reinterpret_cast<float*>(ws + ring * kWStage);    // 3 x 256 biases
+    FusedBars* bars = reinterpret_cast<FusedBars*>(bs + 3 * 256);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n_tiles = (fp.M + BM - 1) / BM;
-    const int kb_layer[4] = {n_xkb, 4, 4, 4};
+    const int n_ob = (fp.out_dim + 255) / 256;                    // output blocks
+    const int n_units = (fp.M + BM - 1) / BM * fp.nsplit;
     const CUtensorMap* wmap[4] = {&map_w0, &map_w1, &map_w2, &map_w3};
 
-    for (int t = threadIdx.x; t < 4 * 256; t += kFThreads) {
-        const int l = t >> 8, c = t & 255;
-        bs[t] = (l < 3 || c < fp.out_dim) ? fp.bias[l][c] : 0.f;
-    }
+    for (int t = threadIdx.x; t < 3 * 256; t += kFThreads) bs[t] = fp.bias[t >> 8][t & 255];
     if (threadIdx.x == 0) {
         mbar_init(smem_u32(&bars->x_full), 1);
         mbar_init(smem_u32(&bars->x_free), 1);
-        mbar_init(smem_u32(&bars->acc_full), 1);
-        mbar_init(smem_u32(&bars->h_ready), kFEpilogue);
-        for (int s = 0; s < kFRing; ++s) {
+        mbar_init(smem_u32(&bars->drain), 1);
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(smem_u32(&bars->acc_full[i]), 1);
+            mbar_init(smem_u32(&bars->acc_free[i]), kFEpiWarps);
+        }
+        for (int i = 0; i < 4; ++i) mbar_init(smem_u32(&bars->h_ready[i]), kFEpiWarps);
+        for (int s = 0; s < ring; ++s) {
             mbar_init(smem_u32(&bars->w_full[s]), 1);
             mbar_init(smem_u32(&bars->w_empty[s]), 1);
         }
@@ -559,7 +633,7 @@ __global__ void __launch_bounds__(kFThreads, 1)
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                          smem_u32(&bars->tmem_base)),
-                     "r"(256)
+                     "r"(512)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -569,158 +643,211 @@ __global__ void __launch_bounds__(kFThreads, 1)
     const uint32_t tmem = bars->tmem_base;
     volatile uint32_t* failed = &bars->failed;
 
+    // A unit's steps: the hidden layers 0..2, then its output blocks split,
+    // split + nsplit, ...; step number g (over all units) uses accumulator
+    // g & 1, whose barriers complete once per use
     if (warp == kFEpiWarps) {
         if (lane == 0) {
             // ---- producer
-            uint32_t g = 0;  // weight slices issued
+            uint32_t n_w = 0;  // weight slices issued
             int it = 0;
-            for (int tile = blockIdx.x; tile < n_tiles && !*failed; tile += gridDim.x, ++it) {
-                if (it > 0 && !mbar_wait(smem_u32(&bars->x_free), (uint32_t)(it - 1) & 1u)) {
-                    atomicExch(&bars->failed, 1u);
-                    break;
-                }
+            bool ok = true;
+            auto slice = [&](int l, int kb, int row) {
+                const int s = (int)(n_w % ring);
+                const uint32_t use = n_w / ring;
+                if (n_w >= (uint32_t)ring && !fused_wait(smem_u32(&bars->w_empty[s]), (use & 1u) ^ 1u, failed))
+                    return false;
+                const uint32_t fb = smem_u32(&bars->w_full[s]);
+                mbar_expect_tx(fb, kWStage);
+                tma_load_2d(smem_u32(ws) + s * kWStage, wmap[l], kb * BK, row, fb);
+                ++n_w;
+                return true;
+            };
+            for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x, ++it) {
+                const int tile = u / fp.nsplit, split = u % fp.nsplit;
+                ok = it == 0 || fused_wait(smem_u32(&bars->x_free), (uint32_t)(it - 1) & 1u, failed);
+                if (!ok) break;
                 const uint32_t xb = smem_u32(&bars->x_full);
                 mbar_expect_tx(xb, (uint32_t)n_xkb * kXBlock);
                 for (int kb = 0; kb < n_xkb; ++kb)
                     tma_load_2d(smem_u32(xs) + kb * kXBlock, &map_x, kb * BK, tile * BM, xb);
-                for (int l = 0; l < 4 && !*failed; ++l)
-                    for (int kb = 0; kb < kb_layer[l]; ++kb, ++g) {
-                        const int s = (int)(g % kFRing);
-                        const uint32_t use = g / kFRing;
-                        if (g >= (uint32_t)kFRing && !mbar_wait(smem_u32(&bars->w_empty[s]), (use & 1u) ^ 1u)) {
-                            atomicExch(&bars->failed, 1u);
-                            break;
-                        }
-                        const uint32_t fb = smem_u32(&bars->w_full[s]);
-                        mbar_expect_tx(fb, kWStage);
-                        tma_load_2d(smem_u32(ws) + s * kWStage, wmap[l], kb * BK, 0, fb);
-                    }
+                for (int l = 0; l < 3 && ok; ++l)
+                    for (int kb = 0; kb < (l == 0 ? n_xkb : 4) && ok; ++kb) ok = slice(l, kb, 0);
+                for (int b = split; b < n_ob && ok; b += fp.nsplit)
+                    for (int kb = 0; kb < 4 && ok; ++kb) ok = slice(3, kb, 256 * b);
+            }
+            if (!ok) {
+                // wait (bounded) for the copies in flight before the CTA can
+                // release its shared memory
+                *failed = 1u;
+                for (uint32_t i = n_w > (uint32_t)ring ? n_w - ring : 0; i < n_w; ++i)
+                    mbar_wait(smem_u32(&bars->w_full[i % ring]), (i / ring) & 1u);
+                if (it > 0) mbar_wait(smem_u32(&bars->x_full), (uint32_t)(it - 1) & 1u);
             }
         }
     } else if (warp == kFEpiWarps + 1) {
         if (lane == 0) {
             // ---- MMA issuer
-            const uint32_t idesc = instr_desc(BM, 256);
-            uint32_t g = 0, L = 0;
+            uint32_t n_w = 0, g = 0, hc = 0;  // weight slices used, steps, hidden layers
             int it = 0;
             bool ok = true;
-            for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x, ++it) {
-                if (!mbar_wait(smem_u32(&bars->x_full), (uint32_t)it & 1u)) {
-                    ok = false;
-                    break;
-                }
-                for (int l = 0; l < 4 && ok; ++l, ++L) {
-                    // the accumulator is free and the activations of the
-                    // previous layer are in place
-                    if (L > 0 && !mbar_wait(smem_u32(&bars->h_ready), (L - 1) & 1u)) {
-                        ok = false;
-                        break;
-                    }
+            // step of n_kb K slices with A at `a`; h_wait: the slices of A are
+            // the hidden layer before (number hc - 1), taken as they get ready
+            auto step = [&](uint32_t a, int n_kb, int n_cols, bool h_wait) {
+                const uint32_t acc = g & 1u, idesc = instr_desc(BM, n_cols);
+                if (g >= 2 && !fused_wait(smem_u32(&bars->acc_free[acc]), ((g >> 1) - 1u) & 1u, failed)) return false;
+                for (int kb = 0; kb < n_kb; ++kb, ++n_w) {
+                    const int s = (int)(n_w % ring);
+                    if (h_wait && !fused_wait(smem_u32(&bars->h_ready[kb]), (hc - 1u) & 1u, failed)) return false;
+                    if (!fused_wait(smem_u32(&bars->w_full[s]), (n_w / ring) & 1u, failed)) return false;
                     tc_fence_after();
-                    for (int kb = 0; kb < kb_layer[l] && ok; ++kb, ++g) {
-                        const int s = (int)(g % kFRing);
-                        if (!mbar_wait(smem_u32(&bars->w_full[s]), (g / kFRing) & 1u)) {
-                            ok = false;
-                            break;
-                        }
-                        tc_fence_after();
-                        const uint32_t a = (l == 0 ? smem_u32(xs) : smem_u32(hs)) + kb * kXBlock;
-                        const uint32_t b = smem_u32(ws) + s * kWStage;
+                    const uint32_t ak = a + kb * kXBlock, b = smem_u32(ws) + s * kWStage;
 #pragma unroll
-                        for (int kk = 0; kk < BK / 16; ++kk)
-                            mma_bf16(tmem, smem_desc(a + kk * 32), smem_desc(b + kk * 32), idesc,
-                                     (kb > 0 || kk > 0) ? 1u : 0u);
-                        mma_commit(smem_u32(&bars->w_empty[s]));
-                    }
-                    mma_commit(smem_u32(&bars->acc_full));
-                    if (l == 0) mma_commit(smem_u32(&bars->x_free));
+                    for (int kk = 0; kk < BK / 16; ++kk)
+                        mma_bf16(tmem + acc * 256, smem_desc(ak + kk * 32), smem_desc(b + kk * 32), idesc,
+                                 (kb > 0 || kk > 0) ? 1u : 0u);
+                    mma_commit(smem_u32(&bars->w_empty[s]));
                 }
+                mma_commit(smem_u32(&bars->acc_full[acc]));
+                ++g;
+                return true;
+            };
+            for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x, ++it) {
+                const int split = u % fp.nsplit;
+                ok = fused_wait(smem_u32(&bars->x_full), (uint32_t)it & 1u, failed);
+                if (ok) ok = step(smem_u32(xs), n_xkb, 256, false);
+                if (!ok) break;
+                mma_commit(smem_u32(&bars->x_free));
+                ++hc;
+                for (int l = 1; l < 3 && ok; ++l, ++hc) ok = step(smem_u32(hs), 4, 256, true);
+                for (int b = split; b < n_ob && ok; b += fp.nsplit)
+                    ok = step(smem_u32(hs), 4, min(256, fp.out_dim - 256 * b), b == split);
             }
             if (!ok) {
-                // unblock the epilogue warps: they see the flag and stop (in
-                // the normal case every accumulator phase is committed exactly
-                // once, so that each epilogue wait sees its own phase)
-                atomicExch(&bars->failed, 1u);
-                mma_commit(smem_u32(&bars->acc_full));
+                // the tensor cores are done with shared memory and TMEM
+                // (bounded) before the CTA releases them
+                *failed = 1u;
+                mma_commit(smem_u32(&bars->drain));
+                mbar_wait(smem_u32(&bars->drain), 0);
             }
         }
     } else {
-        // ---- epilogue warps: row r = 32 (warp mod 4) + lane of the tile,
-        // a band of 256 / (kFEpiWarps / 4) columns
-        constexpr int kBand = 256 / (kFEpiWarps / 4);
+        // ---- epilogue warps: row r = 32 (warp mod 4) + lane of the tile
         const int quarter = warp & 3, part = warp >> 2;
         const int r = quarter * 32 + lane;
-        uint32_t L = 0;
-        for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-            bool stop = false;
-            for (int l = 0; l < 4; ++l, ++L) {
-                const bool have = mbar_wait(smem_u32(&bars->acc_full), L & 1u);
-                if (!have) atomicExch(&bars->failed, 1u);
-                if (__any_sync(0xffffffffu, !have || *failed)) {
-                    stop = true;
-                    break;
+        const uint32_t lanes = (uint32_t)(quarter * 32) << 16;
+        uint32_t g = 0;
+        bool ok = true;
+        auto wait_acc = [&]() {
+            const bool have = fused_wait(smem_u32(&bars->acc_full[g & 1u]), (g >> 1) & 1u, failed);
+            tc_fence_after();
+            return (bool)__all_sync(0xffffffffu, have);
+        };
+        // the accumulator's values are in registers
+        auto free_acc = [&]() {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&bars->acc_free[g & 1u]));
+        };
+        for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x) {
+            const int tile = u / fp.nsplit, split = u % fp.nsplit;
+            for (int l = 0; l < 3 && ok; ++l) {
+                ok = wait_acc();
+                if (!ok) break;
+                uint32_t v[4][16];
+                const uint32_t acc = tmem + lanes + (g & 1u) * 256 + 16 * part;
+#pragma unroll
+                for (int s = 0; s < 4; ++s) tmem_ld16_nowait(acc + 64 * s, v[s]);
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                free_acc();
+                const float* bias = bs + 256 * l + 16 * part;
+#pragma unroll
+                for (int s = 0; s < 4; ++s) {
+                    // 16 BF16 = two 16-byte chunks of row r of K slice s,
+                    // placed by the 128-byte swizzle
+                    uint32_t pk[8];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float4 bv = *reinterpret_cast<const float4*>(bias + 64 * s + 4 * q);
+                        pk[2 * q] = gelu_pair(f2(__uint_as_float(v[s][4 * q]), __uint_as_float(v[s][4 * q + 1])),
+                                              f2(bv.x, bv.y));
+                        pk[2 * q + 1] = gelu_pair(
+                            f2(__uint_as_float(v[s][4 * q + 2]), __uint_as_float(v[s][4 * q + 3])), f2(bv.z, bv.w));
+                    }
+                    uint8_t* blk = hs + s * kXBlock + r * 128;
+#pragma unroll
+                    for (int q = 0; q < 2; ++q)
+                        *reinterpret_cast<uint4*>(blk + ((2 * part + q) ^ (r & 7)) * 16) =
+                            make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
+                    // make the writes visible to the tensor cores, release the slice
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&bars->h_ready[s]));
                 }
-                tc_fence_after();
-                const int ncol = (l == 3) ? fp.out_dim : 256;
-                for (int c0 = kBand * part; c0 < kBand * part + kBand; c0 += 32) {
+                ++g;
+            }
+            for (int b = split; b < n_ob && ok; b += fp.nsplit) {
+                ok = wait_acc();
+                if (!ok) break;
+                const int ncol = min(256, fp.out_dim - 256 * b);
+                const int row0 = tile * BM + quarter * 32 + (lane & ~7), j8 = lane & 7;
+#pragma unroll 1
+                for (int c0 = 64 * part; c0 < 64 * part + 64; c0 += 32) {
+                    if (c0 >= ncol) break;
+                    const bool col_ok = c0 + 4 * j8 < ncol;  // out_dim is a multiple of 16
+                    const int64_t col = 256 * (int64_t)b + c0 + 4 * j8;
+                    float4 bv = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (col_ok) bv = __ldg(reinterpret_cast<const float4*>(fp.bias[3] + col));
                     float v[32];
-                    tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c0, v);
-                    if (c0 >= ncol) continue;
-                    const float* bias = bs + 256 * l;
-                    if (l < 3) {
-                        // 32 BF16 = 64 bytes = four 16-byte chunks of row r of
-                        // K slice c0 / 64, placed by the 128-byte swizzle
-                        uint32_t pk[16];
+                    tmem_ld32(tmem + lanes + (g & 1u) * 256 + (uint32_t)c0, v);
+                    // 8 lanes turn their 8 x 8 groups of four columns around
+                    // (three exchanges), so that a store writes whole 128-byte
+                    // lines: lane j then holds columns 4 j .. 4 j + 3 of the
+                    // 8 rows
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            const float a0 = gelu_f(v[2 * j] + bias[c0 + 2 * j]);
-                            const float a1 = gelu_f(v[2 * j + 1] + bias[c0 + 2 * j + 1]);
-                            pk[j] = (uint32_t)to_bf16(a0) | ((uint32_t)to_bf16(a1) << 16);
-                        }
-                        uint8_t* blk = hs + (c0 / 64) * kXBlock + r * 128;
-                        const int ch0 = ((c0 % 64) * 2) / 16;
+                    for (int d = 1; d < 8; d <<= 1) {
+                        const bool up = j8 & d;
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const int pc = (ch0 + q) ^ (r & 7);
-                            *reinterpret_cast<uint4*>(blk + pc * 16) =
-                                make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
-                        }
-                    } else {
-                        // turn the 32 x 32 block around in this warp's 4 KB of
-                        // the (now free) activation tile, XOR-swizzled, so that
-                        // each store writes 32 consecutive floats of one row
-                        float* tb = reinterpret_cast<float*>(hs) + warp * 1024;
+                        for (int p = 0; p < 8; ++p) {
+                            if (p & d) continue;
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) tb[lane * 32 + (j ^ lane)] = v[j] + bias[c0 + j];
-                        __syncwarp();
-                        const int row0 = tile * BM + quarter * 32, col = c0 + lane;
-                        for (int rr = 0; rr < 32; ++rr) {
-                            const int rw = row0 + rr;
-                            if (rw < fp.M && col < ncol) fp.y[(int64_t)rw * fp.ld_y + col] = tb[rr * 32 + (lane ^ rr)];
+                            for (int i = 0; i < 4; ++i) {
+                                float &lo = v[4 * p + i], &hi = v[4 * (p | d) + i];
+                                const float got = __shfl_xor_sync(0xffffffffu, up ? lo : hi, d);
+                                if (up) lo = got; else hi = got;
+                            }
                         }
-                        __syncwarp();
+                    }
+                    if (col_ok) {
+                        float* y = fp.y + (int64_t)row0 * fp.ld_y + col;
+#pragma unroll
+                        for (int p = 0; p < 8; ++p)
+                            if (row0 + p < fp.M)
+                                *reinterpret_cast<float4*>(y + (int64_t)p * fp.ld_y) =
+                                    make_float4(v[4 * p] + bv.x, v[4 * p + 1] + bv.y, v[4 * p + 2] + bv.z,
+                                                v[4 * p + 3] + bv.w);
                     }
                 }
-                // TMEM read and activations written: make the shared-memory
-                // writes visible to the tensor cores, then release the layer
-                tc_fence_before();
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                mbar_arrive(smem_u32(&bars->h_ready));
+                free_acc();
+                ++g;
             }
-            if (stop) break;
         }
+        if (!ok) *failed = 1u;
     }
     if (*failed && threadIdx.x == 0 && fp.err) atomicExch(fp.err, 1);
     tc_fence_before();
     __syncthreads();
     if (warp == 0) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
     }
 }
 
-size_t fused_smem_bytes() {
-    return 1024 + 6 * (size_t)kXBlock + kFRing * (size_t)kWStage + 4 * 256 * sizeof(float) + sizeof(FusedBars) + 64;
+int fused_ring(int in_dim) { return in_dim > 192 ? 2 : kFRing; }
+
+size_t fused_smem_bytes(int in_dim) {
+    return 1024 + (in_dim / BK + 4) * (size_t)kXBlock + fused_ring(in_dim) * (size_t)kWStage + 3 * 256 * sizeof(float) +
+           sizeof(FusedBars) + 64;
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
@@ -870,15 +997,20 @@ cudaError_t dw_bf16(const DwLayer* layers, int n, int64_t K, int num_sms, int* e
     return cudaGetLastError();
 }
 
+bool fused_forward_fits(int in_dim, int width, int out_dim) {
+    return width == 256 && in_dim >= 64 && in_dim <= 256 && in_dim % 64 == 0 && out_dim >= 16 && out_dim % 16 == 0;
+}
+
 cudaError_t mlp_forward_fused(const uint16_t* x, int64_t M, int in_dim, const uint16_t* const w[4], int out_dim,
                               const float* const bias[4], float* y, int64_t ld_y, int* err, int num_sms,
                               cudaStream_t s) {
     if (M <= 0) return cudaSuccess;
-    if ((in_dim != 64 && in_dim != 128) || out_dim < 16 || out_dim > 256 || out_dim % 16 || M > (int64_t)INT32_MAX)
-        return cudaErrorInvalidValue;
+    if (!fused_forward_fits(in_dim, 256, out_dim) || M > (int64_t)INT32_MAX - BM) return cudaErrorInvalidValue;
     for (int l = 0; l < 4; ++l)
         if (reinterpret_cast<uintptr_t>(w[l]) & 15u) return cudaErrorInvalidValue;
-    if (reinterpret_cast<uintptr_t>(x) & 15u) return cudaErrorInvalidValue;
+    if ((reinterpret_cast<uintptr_t>(x) & 15u) || (reinterpret_cast<uintptr_t>(y) & 15u) || ld_y % 4 ||
+        (reinterpret_cast<uintptr_t>(bias[3]) & 15u))
+        return cudaErrorInvalidValue;
     CUtensorMap mx, mw[4];
     const Mat X{x, M, in_dim, in_dim};
     const int din[4] = {in_dim, 256, 256, 256}, dout[4] = {256, 256, 256, out_dim};
@@ -887,7 +1019,6 @@ cudaError_t mlp_forward_fused(const uint16_t* x, int64_t M, int in_dim, const ui
         const Mat W{w[l], dout[l], din[l], din[l]};
         if (!make_map(&mw[l], W, dout[l], din[l], 256)) return cudaErrorInvalidValue;
     }
-    const size_t smem = fused_smem_bytes();
     cudaError_t e = fused_prepare();
     if (e != cudaSuccess) return e;
     FusedParams fp;
@@ -898,9 +1029,14 @@ cudaError_t mlp_forward_fused(const uint16_t* x, int64_t M, int in_dim, const ui
     fp.in_dim = in_dim;
     fp.out_dim = out_dim;
     fp.err = err;
-    const int tiles = (int)((M + BM - 1) / BM);
-    const int grid = tiles < num_sms ? tiles : num_sms;
-    mlp_fused_forward_kernel<<<grid, kFThreads, smem, s>>>(mx, mw[0], mw[1], mw[2], mw[3], fp);
+    fp.ring = fused_ring(in_dim);
+    // fewer tiles than SMs: the output blocks of a tile go to several CTAs,
+    // as many as leave no SM with a second unit
+    const int tiles = (int)((M + BM - 1) / BM), n_ob = (out_dim + 255) / 256;
+    fp.nsplit = std::max(1, std::min(n_ob, num_sms / tiles));
+    const int units = tiles * fp.nsplit;
+    const int grid = units < num_sms ? units : num_sms;
+    mlp_fused_forward_kernel<<<grid, kFThreads, fused_smem_bytes(in_dim), s>>>(mx, mw[0], mw[1], mw[2], mw[3], fp);
     return cudaGetLastError();
 }
 
@@ -913,7 +1049,7 @@ cudaError_t fused_prepare() {
     std::lock_guard<std::mutex> lk(mu);
     if (dev < 64 && raised[dev]) return cudaSuccess;
     e = cudaFuncSetAttribute(mlp_fused_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)fused_smem_bytes());
+                             (int)std::max(fused_smem_bytes(192), fused_smem_bytes(256)));
     if (e == cudaSuccess && dev < 64) raised[dev] = 1;
     return e;
 }

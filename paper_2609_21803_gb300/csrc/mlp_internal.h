@@ -75,9 +75,10 @@ cudaError_t dw_bf16(const DwLayer* layers, int n, int64_t K, int num_sms, int* e
 bool tensor_maps_available();
 
 // Fused forward pass of the 4-layer MLP (width 256): x [M][in_dim] BF16
-// (in_dim 64 or 128), w[l] BF16 row-major [out][in] (K-major), biases FP32,
-// y [M][ld_y] FP32 (out_dim <= 256, a multiple of 16).  One persistent CTA
-// per SM (at most num_sms CTAs).
+// (in_dim 64, 128, 192 or 256), w[l] BF16 row-major [out][in] (K-major),
+// biases FP32, y [M][ld_y] FP32 (out_dim a multiple of 16, 16-byte rows).
+// One persistent CTA per SM (at most num_sms CTAs).
+bool fused_forward_fits(int in_dim, int width, int out_dim);
 cudaError_t mlp_forward_fused(const uint16_t* x, int64_t M, int in_dim, const uint16_t* const w[4], int out_dim,
                               const float* const bias[4], float* y, int64_t ld_y, int* err, int num_sms,
                               cudaStream_t s);
