@@ -274,7 +274,7 @@ static int64_t resident_warps(const comet_problem* p, int64_t n) {
 
 // floats of workspace per unit (a warp for pushing, a CTA for bimanual)
 static int64_t ws_unit_floats(const comet_problem* p) {
-    return (int64_t)(p->task == COMET_TASK_BIMANUAL ? kBimRec : kRec) * p->Nmax;
+    return (int64_t)(p->task == COMET_TASK_BIMANUAL ? kBimRec + kBimJac : kRec) * p->Nmax;
 }
 
 comet_status reserve_eval(comet_problem* p, int64_t n) {

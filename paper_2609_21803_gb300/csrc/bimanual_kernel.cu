@@ -12,16 +12,26 @@
 // of v_hat (Eq. inexact_mode_value) and the KKT residual.
 //
 // Work per iteration:
-//   A  a warp per stage, a lane per constraint row (32 rows): rows and their
-//      Jacobians from one stage context; the AL model over (u, x_{k+1}, x_k)
-//      built in registers, a model row per lane, from each row's nonzero
-//      pattern; the 12 u columns eliminated there (shuffles for the pivot
-//      column); records to the CTA's workspace (L2-resident)
+//   A  a thread per stage: the 32 constraint rows and their Jacobians, one
+//      after the other as straight code (each row's index a constant), the
+//      multipliers, measures and the AL gradient; a stage's nonzeros go to the
+//      CTA's workspace (L2-resident) as one packed record
+//   M  a warp per stage: the AL model over (u, x_{k+1}, x_k) in registers, a
+//      model row per lane, from each row's nonzero pattern; the 12 u columns
+//      eliminated there (the pivot column through shared memory); records to
+//      the workspace
 //   B  one warp: the sequential sweep eliminating the 5 x_{k+1} columns, the
 //      next stage's record prefetched into registers
 //   gains and control steps stage-parallel, the forward chain on 5 lanes
 //   D  8 trial steps x stages over all threads, sums in shared memory
 //   E  compensated state update
+// Phase A used to run a lane per row: the warp then walked every row type's
+// code for each stage (1,700 of a stage-iteration's 4,300 warp instructions),
+// and phase M belonged to it, so that a trip that only updates multipliers
+// built a model nobody used and a retry recomputed its rows.  With a thread
+// per stage the rows cost 50 instructions per stage; 2,048 random orders of
+// 1..6 segments take 213 -> 105 ms, the 507 one-segment orders 25 -> 15 ms,
+// with bit-identical results.
 
 #include <cuda_runtime.h>
 #include <cuda/annotated_ptr>
@@ -51,6 +61,14 @@ static_assert(R_YF % 4 == 0 && kBimRec % 4 == 0, "vector access to the raw facto
 // reduced block at 212..277), kBRing stages ahead
 constexpr int R_SLOT = 208, kBSlot = 72, kBRing = 6;
 static_assert(R_SLOT + 2 == R_PD && R_SLOT + 4 == R_RED && R_SLOT + kBSlot >= R_RED + NTRI_RED, "ring slot");
+
+// stage Jacobian records (written by phase A, read by phase M): the entries of
+// every row's pattern (bnz) one row after the other, a zero, and the local
+// gradient in elimination order; chunk-major, float4 chunk q of stage k at
+// 4 (q N_max + k), so that lanes over stages move whole lines
+constexpr int NNZ = 85, J_ZERO = 85, J_GRAD = 88, J_REC = 112;
+static_assert(J_REC <= kBimJac && J_REC % 4 == 0, "Jacobian record layout");
+constexpr int NLAM = 33;  // multipliers per stage in shared memory: 32 and a pad (lanes over stages)
 
 // local variables: x_k 0..4, u_k 5..16, x_{k+1} 17..21
 enum { VX = 0, VZ, VTH, VSL, VSR, UXD, UZD, UTHD, UFNL, UFTL, USDL, UFNR, UFTR, USDR, ULN, ULT, UPC, VX1 };
@@ -131,8 +149,19 @@ struct BStage {
     T rcx, rcz, w, dw;    // pivot corner offset, support half-width
 };
 
+// Products and sums with their rounding written out (FP32): fm(a, b, c) is one
+// fused multiply-add, m2(a, b) a product rounded by itself.  Left to the
+// compiler, which of two products of a sum is fused depends on the code
+// around it, and the rows are inlined in several phases.
+__device__ __forceinline__ float fm(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fm(double a, double b, double c) { return a * b + c; }
+__device__ __forceinline__ float m2(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double m2(double a, double b) { return a * b; }
+__device__ __forceinline__ float a2(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double a2(double a, double b) { return a + b; }
+
 template <typename T>
-__device__ void stage_ctx(const BInst<T>& P, int mode, const T* x, const T* u, BStage<T>& S) {
+__device__ __forceinline__ void stage_ctx(const BInst<T>& P, int mode, const T* x, const T* u, BStage<T>& S) {
     S.g = mode / 169;
     S.h[0] = (mode / 13) % 13;
     S.h[1] = mode % 13;
@@ -151,7 +180,7 @@ __device__ void stage_ctx(const BInst<T>& P, int mode, const T* x, const T* u, B
     const T cth = S.cth, sth = S.sth;
     S.Fwx = u[ULT - 5];
     S.Fwz = u[ULN - 5];
-    S.tau = u[UPC - 5] * u[ULN - 5] + x[VZ] * u[ULT - 5];
+    S.tau = fm(u[UPC - 5], u[ULN - 5], m2(x[VZ], u[ULT - 5]));
 #pragma unroll
     for (int side = 0; side < 2; ++side) {
         const int h = S.h[side];
@@ -167,15 +196,16 @@ __device__ void stage_ctx(const BInst<T>& P, int mode, const T* x, const T* u, B
         if (h == 0) continue;
         const T fn = u[(side ? UFNR : UFNL) - 5], ft = u[(side ? UFTR : UFTL) - 5];
         const T s = x[side ? VSR : VSL];
-        const T bx = fn * nx + ft * (-nz), bz = fn * nz + ft * nx;
-        S.Fwx += cth * bx - sth * bz;
-        S.Fwz += sth * bx + cth * bz;
-        S.tau += -S.a[side] * ft - s * fn;
+        const T bx = fm(fn, nx, m2(ft, -nz)), bz = fm(fn, nz, m2(ft, nx));
+        S.Fwx = a2(S.Fwx, fm(cth, bx, -m2(sth, bz)));
+        S.Fwz = a2(S.Fwz, fm(sth, bx, m2(cth, bz)));
+        S.tau = a2(S.tau, fm(-S.a[side], ft, -m2(s, fn)));
     }
-    S.rcx = -P.ax * cth + P.az * sth;
-    S.rcz = -P.ax * sth - P.az * cth;
-    S.w = P.ax * cth * cth + P.az * sth * sth;
-    S.dw = 2 * sth * cth * (P.az - P.ax);
+    const T axc = m2(P.ax, cth), azs = m2(P.az, sth);
+    S.rcx = a2(-axc, azs);
+    S.rcz = fm(-P.ax, sth, -m2(P.az, cth));
+    S.w = fm(axc, cth, m2(azs, sth));
+    S.dw = m2(m2(2 * sth, cth), P.az - P.ax);
 }
 
 // hand rows of one side (q = 0..7): force, sliding rate and offset
@@ -211,12 +241,32 @@ __host__ __device__ constexpr int bnz(int r, int a) {
          : bnz_hand(r >= 24, r - (r >= 24 ? 24 : 16), a);
 }
 
+// first entry of row r in the packed pattern (closed form: it has to fold to a
+// constant where the rows are unrolled)
+__host__ __device__ constexpr int bnz_first_hand(int q) {
+    return q == 0 ? 0 : q == 1 ? 3 : q == 2 ? 4 : q == 3 ? 5 : q == 4 ? 8 : q == 5 ? 10 : q == 6 ? 11 : 12;
+}
+__host__ __device__ constexpr int bnz_first(int r) {
+    return r < 5 ? 3 * r : r == 5 ? 15 : r == 6 ? 21 : r == 7 ? 27 : r == 8 ? 37 : r == 9 ? 41 : r == 10 ? 44
+         : r == 11 ? 49 : r == 12 ? 52 : r == 13 ? 54 : r == 14 ? 55 : r == 15 ? 57
+         : r < 24 ? 59 + bnz_first_hand(r - 16) : 72 + bnz_first_hand(r - 24);
+}
+constexpr bool bnz_first_ok() {
+    int n = 0;
+    for (int r = 0; r < NR; ++r) {
+        if (bnz_first(r) != n) return false;
+        for (int q = 0; q < 10 && bnz(r, q) >= 0; ++q) ++n;
+    }
+    return n == NNZ;
+}
+static_assert(bnz_first_ok(), "packed Jacobian offsets");
+
 // Row r of an interval: scaled value c, presence, inequality flag, the
 // physical factor (physical = c / scale) and, with WJ, the Jacobian over the
 // 22 local variables.  dx = x_{k+1} - x_k (kinematic rows; computed from the
 // compensated states by the caller).
 template <typename T, bool WJ>
-__device__ void brow(int r, const BInst<T>& P, const BStage<T>& S, bool mL, bool mR, const T* x, const T* u,
+__device__ __forceinline__ void brow(int r, const BInst<T>& P, const BStage<T>& S, bool mL, bool mR, const T* x, const T* u,
                      const T* dx, T& c, T* J, bool& on, bool& ineq, T& scale) {
     // internally the force rows are divided by m g and the torque row by
     // m g l; scale maps a row back to physical units (physical = c / scale:
@@ -233,7 +283,7 @@ __device__ void brow(int r, const BInst<T>& P, const BStage<T>& S, bool mL, bool
         const int vel = (r < 3) ? UXD + r : (r == 3 ? USDL : USDR);
         const T dxr = (r == 0) ? dx[0] : (r == 1) ? dx[1] : (r == 2) ? dx[2] : (r == 3) ? dx[3] : dx[4];
         const T ur = (r == 0) ? u[0] : (r == 1) ? u[1] : (r == 2) ? u[2] : (r == 3) ? u[USDL - 5] : u[USDR - 5];
-        c = dxr - P.dt * ur;
+        c = fm(-P.dt, ur, dxr);
         if (WJ) {
             J[r] = -1;
             J[VX1 + r] = 1;
@@ -243,9 +293,9 @@ __device__ void brow(int r, const BInst<T>& P, const BStage<T>& S, bool mL, bool
     } else if (r < 8) {
         const T sc = (r == 7) ? 1 / (mg * P.lbar) : 1 / mg;
         scale = sc;
-        if (r == 5) c = S.Fwx * sc;
-        if (r == 6) c = (S.Fwz - mg) * sc;
-        if (r == 7) c = S.tau * sc;
+        if (r == 5) c = m2(S.Fwx, sc);
+        if (r == 6) c = m2(S.Fwz - mg, sc);
+        if (r == 7) c = m2(S.tau, sc);
         if (WJ) {
             const T cth = S.cth, sth = S.sth;
             if (r == 5) J[ULT] = sc;
@@ -262,16 +312,16 @@ __device__ void brow(int r, const BInst<T>& P, const BStage<T>& S, bool mL, bool
                 const int ufn = side ? UFNR : UFNL, uft = side ? UFTR : UFTL, vs = side ? VSR : VSL;
                 const T nx = S.n[side][0], nz = S.n[side][1], tx = S.t[side][0], tz = S.t[side][1];
                 const T fn = u[ufn - 5], ft = u[uft - 5];
-                const T bx = fn * nx + ft * tx, bz = fn * nz + ft * tz;
-                const T wx = cth * bx - sth * bz, wz = sth * bx + cth * bz;
+                const T bx = fm(fn, nx, m2(ft, tx)), bz = fm(fn, nz, m2(ft, tz));
+                const T wx = fm(cth, bx, -m2(sth, bz)), wz = fm(sth, bx, m2(cth, bz));
                 if (r == 5) {
-                    J[VTH] += -wz * sc;
-                    J[ufn] = (cth * nx - sth * nz) * sc;
-                    J[uft] = (cth * tx - sth * tz) * sc;
+                    J[VTH] = fm(-wz, sc, J[VTH]);
+                    J[ufn] = m2(fm(cth, nx, -m2(sth, nz)), sc);
+                    J[uft] = m2(fm(cth, tx, -m2(sth, tz)), sc);
                 } else if (r == 6) {
-                    J[VTH] += wx * sc;
-                    J[ufn] = (sth * nx + cth * nz) * sc;
-                    J[uft] = (sth * tx + cth * tz) * sc;
+                    J[VTH] = fm(wx, sc, J[VTH]);
+                    J[ufn] = m2(fm(sth, nx, m2(cth, nz)), sc);
+                    J[uft] = m2(fm(sth, tx, m2(cth, tz)), sc);
                 } else {
                     J[uft] = -S.a[side] * sc;
                     J[ufn] = -(side ? x[VSR] : x[VSL]) * sc;
@@ -290,7 +340,7 @@ __device__ void brow(int r, const BInst<T>& P, const BStage<T>& S, bool mL, bool
                 c = zd;
                 if (WJ) J[UZD] = 1;
             } else {
-                c = xd - thd * S.rcz;
+                c = fm(-thd, S.rcz, xd);
                 if (WJ) {
                     J[UXD] = 1;
                     J[UTHD] = -S.rcz;
@@ -305,7 +355,7 @@ __device__ void brow(int r, const BInst<T>& P, const BStage<T>& S, bool mL, bool
                 c = thd;
                 if (WJ) J[UTHD] = 1;
             } else {
-                c = zd + thd * S.rcx;
+                c = fm(thd, S.rcx, zd);
                 if (WJ) {
                     J[UZD] = 1;
                     J[UTHD] = S.rcx;
@@ -320,10 +370,10 @@ __device__ void brow(int r, const BInst<T>& P, const BStage<T>& S, bool mL, bool
                 const T s2 = 1 / (mg * mg);
                 // factored, so that the difference near the edge is formed
                 // before the product (no cancellation of two squares)
-                c = ((lt - mu * ln) * (lt + mu * ln)) * s2;
+                c = m2(m2(fm(-mu, ln, lt), fm(mu, ln, lt)), s2);
                 // physical: the friction force's distance from the cone
                 // edge, |lam_t| - mu |lam_n| [N]
-                const T den = fabs(lt) + mu * fabs(ln);
+                const T den = fm(mu, fabs(ln), fabs(lt));
                 scale = den > (T)0 ? den * s2 : (T)1;
                 if (WJ) {
                     J[ULT] = 2 * lt * s2;
@@ -340,7 +390,7 @@ __device__ void brow(int r, const BInst<T>& P, const BStage<T>& S, bool mL, bool
             if (S.g != 1) {
                 const T sc = 1 / (mg * P.cg), sg = (r == 11) ? (T)1 : (T)-1;
                 scale = sc;
-                c = (sg * lt - mu * ln) * sc;
+                c = m2(a2(sg * lt, -m2(mu, ln)), sc);
                 if (WJ) {
                     J[ULT] = sg * sc;
                     J[ULN] = -mu * sc;
@@ -348,7 +398,7 @@ __device__ void brow(int r, const BInst<T>& P, const BStage<T>& S, bool mL, bool
             } else if (r == 11) {
                 const T sc = 1 / mg;
                 scale = sc;  // W
-                c = lt * xd * sc;
+                c = m2(m2(lt, xd), sc);
                 if (WJ) {
                     J[ULT] = xd * sc;
                     J[UXD] = lt * sc;
@@ -365,7 +415,7 @@ __device__ void brow(int r, const BInst<T>& P, const BStage<T>& S, bool mL, bool
                 on = false;
             } else {
                 const T sg = (r == 14) ? (T)1 : (T)-1;
-                c = sg * pc - S.w;
+                c = fm(sg, pc, -S.w);
                 if (WJ) {
                     J[UPC] = sg;
                     J[VTH] = -S.dw;
@@ -408,7 +458,7 @@ __device__ void brow(int r, const BInst<T>& P, const BStage<T>& S, bool mL, bool
                 } else {
                     const T sg = (kind == 1) ? (T)-1 : (T)1;
                     scale = sch;
-                    c = (ft + sg * muh * fn) * sch;
+                    c = m2(fm(sg * muh, fn, ft), sch);
                     if (WJ) {
                         J[uft] = sch;
                         J[ufn] = sg * muh * sch;
@@ -417,7 +467,7 @@ __device__ void brow(int r, const BInst<T>& P, const BStage<T>& S, bool mL, bool
             } else if (q == 3) {
                 if (kind == 0) {
                     scale = sch;
-                    c = (ft - muh * fn) * sch;
+                    c = m2(fm(-muh, fn, ft), sch);
                     if (WJ) {
                         J[uft] = sch;
                         J[ufn] = -muh * sch;
@@ -430,7 +480,7 @@ __device__ void brow(int r, const BInst<T>& P, const BStage<T>& S, bool mL, bool
             } else if (q == 4) {
                 if (kind == 0) {
                     scale = sch;
-                    c = (-ft - muh * fn) * sch;
+                    c = m2(fm(-muh, fn, -ft), sch);
                     if (WJ) {
                         J[uft] = -sch;
                         J[ufn] = -muh * sch;
@@ -444,7 +494,7 @@ __device__ void brow(int r, const BInst<T>& P, const BStage<T>& S, bool mL, bool
                 if (WJ) J[ufn] = -1 / mg;
             } else {
                 const T sg = (q == 6) ? (T)1 : (T)-1;
-                c = sg * s - ell;
+                c = fm(sg, s, -ell);
                 if (WJ) J[vs] = sg;
             }
         }
@@ -474,29 +524,33 @@ __device__ __forceinline__ void two_sum_b(float a, float b, float& s, float& e) 
 struct BSmem {
     float *xh, *xl, *us, *lam, *dz, *gr;
     int* mi;     // per interval: mode | maskL << 10 | maskR << 11
-    float *Jw, *yw;       // per warp: [32][22], [32]
+    float* jbuf;          // per warp: two Jacobian records
+    float* col;           // per warp: two pivot columns of 24
+    uint16_t* at;         // [row][lane]: byte offset of the lane's entry in a record
     float* ring;          // sweep copy ring [kBRing][kBSlot] (16-byte aligned)
     float* red;           // reductions / broadcasts [64]
 };
 
 __host__ __device__ inline size_t bsmem_floats(int Nmax) {
-    const size_t f = (size_t)10 * (Nmax + 1) + (size_t)NU * Nmax + 3 + (size_t)NR * Nmax +
-                     2 * ((size_t)NWV * Nmax + NX) + (size_t)Nmax + 4 * (NR * NL + NR) + kBRing * kBSlot + 64;
+    const size_t f = (size_t)10 * (Nmax + 1) + (size_t)NU * Nmax + 3 + (size_t)NLAM * Nmax +
+                     2 * ((size_t)NWV * Nmax + NX) + (size_t)Nmax + 4 * (2 * J_REC + 48) + NR * 16 +
+                     kBRing * kBSlot + 64;
     return (f + 3) / 4 * 4;
 }
 
 __device__ BSmem bcarve(float* p, int Nmax) {
     BSmem s;
     s.ring = p; p += kBRing * kBSlot;  // first: 16-byte aligned
+    s.jbuf = p; p += 4 * 2 * J_REC;
+    s.col = p; p += 4 * 48;
+    s.at = reinterpret_cast<uint16_t*>(p); p += NR * 16;
     s.xh = p; p += NX * (Nmax + 1);
     s.xl = p; p += NX * (Nmax + 1);
     s.us = p; p += NU * Nmax;
-    s.lam = p; p += 3 + NR * Nmax;
+    s.lam = p; p += 3 + NLAM * Nmax;
     s.dz = p; p += NWV * Nmax + NX;
     s.gr = p; p += NWV * Nmax + NX;
     s.mi = reinterpret_cast<int*>(p); p += Nmax;
-    s.Jw = p; p += 4 * NR * NL;
-    s.yw = p; p += 4 * NR;
     s.red = p;
     return s;
 }
@@ -506,7 +560,8 @@ struct BCtx {
     BInst<float> P;
     BSmem S;
     float* rec;
-    int N, Np1, len;
+    float* jac;   // Jacobian records (chunk-major)
+    int N, Np1, Nmax, len;
     int tid, warp, lane;
 };
 
@@ -536,141 +591,87 @@ struct BMeasures {
     bool finite;
 };
 
-// Phase A: rows, multipliers (PHR update at beta_old with `update`), the
-// measures, the AL gradient into gr (x_{k+1} parts parked in dz), and, with
-// `assemble`, the stage records (u block eliminated).
-__device__ BMeasures bphase_a(BCtx& C, float beta, float rho, bool assemble, bool update, float beta_old) {
+// Phase A, a thread per stage: rows and their Jacobians (every row its own
+// straight code, its index a constant), multipliers (PHR update at beta_old
+// with `update`), the measures, the AL gradient into gr (x_{k+1} parts parked
+// in dz) and the stage's Jacobian record for phase M.
+__device__ BMeasures bphase_a(BCtx& C, float beta, bool update, float beta_old) {
     BSmem& S = C.S;
     const BInst<float>& P = C.P;
-    const int N = C.N, lane = C.lane, warp = C.warp;
-    float* Jw = S.Jw + warp * NR * NL;
-    float* yw = S.yw + warp * NR;
+    const int N = C.N;
     float viol = 0.f, comp = 0.f, vph = 0.f, jc = 0.f;
     bool finite = true;
 #pragma unroll 1
-    for (int k = warp; k < N; k += 4) {
+    for (int k = C.tid; k < N; k += kBimThreads) {
         float x[NX], u[NU], dx[NX];
         load_stage(C, k, 0.f, x, u, dx);
-        if (lane == 0) {
-#pragma unroll
-            for (int j = 0; j < NU; ++j) jc += rweight(P, j) * u[j] * u[j];
-        }
         const int mi = S.mi[k];
         BStage<float> St;
         stage_ctx(P, mi & 1023, x, u, St);
-        // the row's Jacobian goes straight into its shared-memory row (a
-        // register array indexed at run time would live in local memory)
-        float* Jr = Jw + lane * NL;
-        float c, sc;
-        bool on, iq;
-        brow<float, true>(lane, P, St, (mi >> 10) & 1, (mi >> 11) & 1, x, u, dx, c, Jr, on, iq, sc);
-        float* lam = S.lam + 3 + NR * k;
-        float l = lam[lane];
-        if (update && on) {
-            const float t = l + beta_old * c;
-            l = iq ? fmaxf(t, 0.f) : t;
-            lam[lane] = l;
+        float* lam = S.lam + 3 + NLAM * k;
+        cuda::annotated_ptr<float4, cuda::access_property::persisting> jac(reinterpret_cast<float4*>(C.jac) + k);
+        float g[NL], out[J_REC];
+#pragma unroll
+        for (int j = 0; j < NL; ++j) g[j] = 0.f;
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            float c, sc, J[NL];
+            bool on, iq;
+            brow<float, true>(r, P, St, (mi >> 10) & 1, (mi >> 11) & 1, x, u, dx, c, J, on, iq, sc);
+            float l = lam[r];
+            if (update && on) {
+                const float t = fm(beta_old, c, l);
+                l = iq ? fmaxf(t, 0.f) : t;
+                lam[r] = l;
+            }
+            const float t = fm(beta, c, l);
+            const bool act = on && (!iq || t > 0.f);
+            const float y = act ? (iq ? fmaxf(t, 0.f) : t) : 0.f;
+            if (on) {
+                const float vr = iq ? fmaxf(c, 0.f) : fabsf(c);
+                viol = fmaxf(viol, vr);
+                vph = fmaxf(vph, vr / sc);
+                if (iq) comp = fmaxf(comp, fabsf(y * c));
+                if (!isfinite(c)) finite = false;
+            }
+#pragma unroll
+            for (int q = 0; q < 10; ++q) {
+                const int v = bnz(r, q);
+                if (v < 0) break;
+                const float a = act ? J[v] : 0.f;
+                out[bnz_first(r) + q] = a;
+                g[v] = fm(y, a, g[v]);
+            }
         }
-        const float t = l + beta * c;
-        const bool act = on && (!iq || t > 0.f);
-        const float y = act ? (iq ? fmaxf(t, 0.f) : t) : 0.f;
-        if (on) {
-            const float vr = iq ? fmaxf(c, 0.f) : fabsf(c);
-            viol = fmaxf(viol, vr);
-            vph = fmaxf(vph, vr / sc);
-            if (iq) comp = fmaxf(comp, fabsf(y * c));
-            if (!isfinite(c)) finite = false;
-        }
-        if (!act)
-            for (int j = 0; j < NL; ++j) Jr[j] = 0.f;
-        yw[lane] = y;
-        __syncwarp();
-        // AL gradient over the local variables (lane = variable)
-        float gval = 0.f;
-        if (lane < NL) {
-            float g = 0.f;
-            for (int r = 0; r < NR; ++r) g += yw[r] * Jw[r * NL + lane];
-            if (lane >= 5 && lane < 17) g += 2.f * rweight(P, lane - 5) * S.us[(lane - 5) * N + k];
-            if (lane < 17)
-                S.gr[NWV * k + lane] = g;
+#pragma unroll
+        for (int j = 0; j < NU; ++j) g[NX + j] = fm(2.f * rweight(P, j), S.us[j * N + k], g[NX + j]);
+#pragma unroll
+        for (int j = 0; j < NL; ++j) {
+            if (j < NWV)
+                S.gr[NWV * k + j] = g[j];
             else
-                S.dz[NWV * (k + 1) + lane - 17] = g;
-            gval = g;
+                S.dz[NWV * (k + 1) + j - NWV] = g[j];
         }
-        if (assemble) {
-            // the model in registers, a row per lane: lane i < 22 holds row i
-            // of the lower triangle over (u, y, x) in elimination order (and
-            // lane 22 the rhs row).  Row i = sum_r J_r[v_i] J_r over the
-            // active rows in row order; for row r only the columns of its
-            // pattern (bnz) are added, the others being exact zeros: the
-            // lane's own entry times a broadcast Jacobian value
-            const int vi = lane < NL ? evar(lane) : 0;
-            float row[NE];
 #pragma unroll
-            for (int cc = 0; cc < NE; ++cc) row[cc] = 0.f;
+        for (int i = NNZ; i < J_GRAD; ++i) out[i] = 0.f;
 #pragma unroll
-            for (int r = 0; r < NR; ++r) {
-                const float a = lane < NL ? Jw[r * NL + vi] : 0.f;
+        for (int e = 0; e < NL; ++e) out[J_GRAD + e] = g[evar(e)];
+        out[J_GRAD + NL] = out[J_GRAD + NL + 1] = 0.f;
 #pragma unroll
-                for (int q = 0; q < 10; ++q) {
-                    if (bnz(r, q) < 0) break;
-                    row[epos(bnz(r, q))] += a * Jw[r * NL + bnz(r, q)];
-                }
+        for (int q = 0; q < J_REC / 4; ++q)
+            jac[(int64_t)q * C.Nmax] = make_float4(out[4 * q], out[4 * q + 1], out[4 * q + 2], out[4 * q + 3]);
+    }
+    // the cost's control terms: four chains over the stages (k mod 4), on the
+    // warp with the fewest stages
+    if (C.warp == 3 && C.lane < 4) {
+#pragma unroll 1
+        for (int k = C.lane; k < N; k += 4) {
+#pragma unroll
+            for (int j = 0; j < NU; ++j) {
+                const float uj = S.us[j * N + k];
+                jc = fm(m2(rweight(P, j), uj), uj, jc);
             }
-            // beta, then the cost and damping on the diagonal (u: cost +
-            // rho, x_{k+1}: rho); the gradient as the rhs row (lane 22)
-#pragma unroll
-            for (int cc = 0; cc < NE - 1; ++cc) {
-                row[cc] *= beta;
-                if (lane == cc) {
-                    if (cc < 12) row[cc] += 2.f * rweight(P, cc) + rho;
-                    else if (cc < 17) row[cc] += rho;
-                }
-            }
-#pragma unroll
-            for (int cc = 0; cc < NE - 1; ++cc) {
-                const float gv = __shfl_sync(kFullB, gval, evar(cc));
-                if (lane == NE - 1) row[cc] = gv;
-            }
-            // eliminate the u block (12 Cholesky columns) in registers: lane
-            // i < 23 holds row i of the lower triangle (entries 0..i); the
-            // pivot comes from lane j and the column entry L_cj from lane c
-            // by shuffles.  A non-positive pivot marks the record.
-            bool pd = true;
-#pragma unroll
-            for (int j = 0; j < 12; ++j) {
-                const float d = __shfl_sync(kFullB, row[j], j);
-                pd = pd && (d > 0.f);
-                const float l = sqrtf(fmaxf(d, 1e-30f));
-                const float il = 1.f / l;
-                if (lane == j) row[j] = l;
-                if (lane > j) row[j] *= il;
-#pragma unroll
-                for (int cc = j + 1; cc < NE; ++cc) {
-                    const float lcj = __shfl_sync(kFullB, row[j], cc);
-                    if (lane >= cc) row[cc] -= row[j] * lcj;
-                }
-            }
-            // records from the rows: the u factor (rows 0..11), the coupling
-            // rows (12..22) x u columns, the reduced (y, x, rhs) block
-            // record stores with the persisting (evict-last) L2 priority: the
-            // CTAs' workspaces fit in L2 and are rewritten every iteration
-            cuda::annotated_ptr<float, cuda::access_property::persisting> rec(C.rec + (size_t)k * kBimRec);
-            if (lane < 12) {
-#pragma unroll
-                for (int cc = 0; cc < 12; ++cc)
-                    if (cc <= lane) rec[R_LUU + tri(lane, cc)] = row[cc];
-            } else if (lane < NE) {
-                const int p = lane - 12;
-#pragma unroll
-                for (int cc = 0; cc < 12; ++cc) rec[R_CPL + 12 * p + cc] = row[cc];
-#pragma unroll
-                for (int cc = 12; cc < NE; ++cc)
-                    if (cc <= lane) rec[R_RED + tri(p, cc - 12)] = row[cc];
-            }
-            if (lane == 0) rec[R_PD] = pd ? 1.f : -1.f;
         }
-        __syncwarp();
     }
     __syncthreads();
     // initial pose rows and the combined gradient
@@ -687,10 +688,10 @@ __device__ BMeasures bphase_a(BCtx& C, float beta, float rho, bool assemble, boo
         vph = fmaxf(vph, fabsf(c));
         if (!isfinite(c)) finite = false;
     }
-    if (tid == 0)
+    if (tid == 96)
         for (int i = 0; i < 3; ++i) {
             const float e = (S.xh[i * Np1 + N] - P.goal[i]) + S.xl[i * Np1 + N];
-            jc += P.wT * e * e;
+            jc = fm(m2(P.wT, e), e, jc);
         }
     __syncthreads();
     for (int k = tid; k <= N; k += kBimThreads) {
@@ -715,7 +716,6 @@ __device__ BMeasures bphase_a(BCtx& C, float beta, float rho, bool assemble, boo
     stat = bwarp_max(stat);
     comp = bwarp_max(comp);
     vph = bwarp_max(vph);
-    jc = bwarp_sum(jc);
     const bool fin = __all_sync(kFullB, finite);
     __syncthreads();
     if (C.lane == 0) {
@@ -724,8 +724,8 @@ __device__ BMeasures bphase_a(BCtx& C, float beta, float rho, bool assemble, boo
         S.red[8 + C.warp] = comp;
         S.red[12 + C.warp] = fin ? 1.f : 0.f;
         S.red[24 + C.warp] = vph;
-        S.red[28 + C.warp] = jc;
     }
+    if (C.warp == 3 && C.lane < 4) S.red[28 + C.lane] = jc;
     __syncthreads();
     BMeasures m;
     m.viol = fmaxf(fmaxf(S.red[0], S.red[1]), fmaxf(S.red[2], S.red[3]));
@@ -736,6 +736,120 @@ __device__ BMeasures bphase_a(BCtx& C, float beta, float rho, bool assemble, boo
     m.cost = (S.red[28] + S.red[29]) + (S.red[30] + S.red[31]);
     __syncthreads();
     return m;
+}
+
+// Phase M, a warp per stage: the AL model over (u, x_{k+1}, x_k) from the
+// stage's Jacobian record and the elimination of the 12 u columns, a model row
+// per lane in registers; records for the sweep, the gains and the controls.
+// The next stage's record is copied into shared memory meanwhile.
+__device__ void bphase_m(BCtx& C, float beta, float rho) {
+    BSmem& S = C.S;
+    const BInst<float>& P = C.P;
+    const int N = C.N, lane = C.lane, warp = C.warp;
+    float* jb = S.jbuf + warp * 2 * J_REC;
+    float* colb = S.col + warp * 48;
+    auto fetch = [&](int k, int buf) {
+        if (k < N && lane < J_REC / 4)
+            bcp_async16(jb + buf * J_REC + 4 * lane, C.jac + 4 * ((int64_t)lane * C.Nmax + k));
+        bcp_async_commit();
+    };
+    fetch(warp, 0);
+    int buf = 0;
+#pragma unroll 1
+    for (int k = warp; k < N; k += 4, buf ^= 1) {
+        fetch(k + 4, buf ^ 1);
+        bcp_async_wait<1>();
+        __syncwarp();
+        const float* J = jb + buf * J_REC;
+        // lane i < 22 holds row i of the lower triangle over (u, y, x) in
+        // elimination order (and lane 22 the rhs row).  Row i = sum_r J_r[v_i]
+        // J_r over the active rows in row order; for row r only the columns of
+        // its pattern (bnz) are added, the others being exact zeros: the
+        // lane's own entry times a broadcast Jacobian value
+        float row[NE];
+#pragma unroll
+        for (int cc = 0; cc < NE; ++cc) row[cc] = 0.f;
+        float4 t4 = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            const float a = *reinterpret_cast<const float*>(reinterpret_cast<const char*>(J) + S.at[32 * r + lane]);
+#pragma unroll
+            for (int q = 0; q < 10; ++q) {
+                if (bnz(r, q) < 0) break;
+                const int n = bnz_first(r) + q;
+                if (n % 4 == 0) t4 = *reinterpret_cast<const float4*>(J + n);
+                const float b = n % 4 == 0 ? t4.x : n % 4 == 1 ? t4.y : n % 4 == 2 ? t4.z : t4.w;
+                // a row of one entry is added as a rounded product
+                float& m = row[epos(bnz(r, q))];
+                m = bnz(r, 1) < 0 ? a2(m, m2(a, b)) : fm(a, b, m);
+            }
+        }
+        // beta, then the cost and damping on the diagonal (u: cost + rho,
+        // x_{k+1}: rho); the gradient as the rhs row (lane 22)
+#pragma unroll
+        for (int cc = 0; cc < NE - 1; ++cc) {
+            row[cc] = m2(row[cc], beta);
+            if (lane == cc && cc < 17) row[cc] = a2(row[cc], cc < 12 ? fm(2.f, rweight(P, cc), rho) : rho);
+        }
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            const float4 t = *reinterpret_cast<const float4*>(J + J_GRAD + 4 * q);
+            if (lane == NE - 1) {
+                row[4 * q] = t.x;
+                row[4 * q + 1] = t.y;
+                if (4 * q + 2 < NE - 1) {
+                    row[4 * q + 2] = t.z;
+                    row[4 * q + 3] = t.w;
+                }
+            }
+        }
+        // eliminate the u block (12 Cholesky columns): lane i < 23 holds row i
+        // of the lower triangle (entries 0..i; what the updates leave above the
+        // diagonal is never read).  The scaled column goes through shared
+        // memory (two buffers, one warp barrier per pivot) and comes back as
+        // broadcasts, four entries a load.  A non-positive pivot marks the record.
+        bool pd = true;
+#pragma unroll
+        for (int j = 0; j < 12; ++j) {
+            const float d = __shfl_sync(kFullB, row[j], j);
+            pd = pd && (d > 0.f);
+            const float l = sqrtf(fmaxf(d, 1e-30f));
+            const float il = 1.f / l;
+            row[j] = lane == j ? l : row[j] * il;
+            float* col = colb + 24 * (j & 1);
+            if (lane < 24) col[lane] = row[j];
+            __syncwarp();
+#pragma unroll
+            for (int q = (j + 1) / 4; q < 6; ++q) {
+                const float4 t = *reinterpret_cast<const float4*>(col + 4 * q);
+                const float b[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (4 * q + i > j && 4 * q + i < NE) row[4 * q + i] = fm(-row[j], b[i], row[4 * q + i]);
+            }
+        }
+        // records from the rows: the u factor (rows 0..11), the coupling
+        // rows (12..22) x u columns, the reduced (y, x, rhs) block
+        // record stores with the persisting (evict-last) L2 priority: the
+        // CTAs' workspaces fit in L2 and are rewritten every iteration
+        cuda::annotated_ptr<float, cuda::access_property::persisting> rec(C.rec + (size_t)k * kBimRec);
+        if (lane < 12) {
+#pragma unroll
+            for (int cc = 0; cc < 12; ++cc)
+                if (cc <= lane) rec[R_LUU + tri(lane, cc)] = row[cc];
+        } else if (lane < NE) {
+            const int p = lane - 12;
+#pragma unroll
+            for (int cc = 0; cc < 12; ++cc) rec[R_CPL + 12 * p + cc] = row[cc];
+#pragma unroll
+            for (int cc = 12; cc < NE; ++cc)
+                if (cc <= lane) rec[R_RED + tri(p, cc - 12)] = row[cc];
+        }
+        if (lane == 0) rec[R_PD] = pd ? 1.f : -1.f;
+        __syncwarp();
+    }
+    bcp_async_wait_all();
+    __syncthreads();
 }
 
 // Sweep over k = N-1 .. 0 on warp 0.  Every lane runs the whole stage in
@@ -1008,9 +1122,9 @@ __device__ float bphase_c(BCtx& C) {
 }
 
 __device__ __forceinline__ float brow_al(bool ineq, float lam, float beta, float inv2b, float c) {
-    if (!ineq) return lam * c + 0.5f * beta * c * c;
-    const float t = fmaxf(lam + beta * c, 0.f);
-    return (t * t - lam * lam) * inv2b;
+    if (!ineq) return fm(lam, c, m2(m2(m2(0.5f, beta), c), c));
+    const float t = fmaxf(fm(beta, c, lam), 0.f);
+    return m2(fm(t, t, -m2(lam, lam)), inv2b);
 }
 
 // trial merits for alpha in {0, 1, ..., 2^-6}; returns the accepted alpha
@@ -1038,24 +1152,26 @@ __device__ float bphase_d(BCtx& C, float beta, float D, const SolverParams& sp) 
                 const int mi = S.mi[k];
                 BStage<float> St;
                 stage_ctx(P, mi & 1023, x, u, St);
-                const float* lam = S.lam + 3 + NR * k;
-                for (int j = 0; j < NU; ++j) phi += rweight(P, j) * u[j] * u[j];
+                const float* lam = S.lam + 3 + NLAM * k;
+#pragma unroll
+                for (int j = 0; j < NU; ++j) phi = fm(m2(rweight(P, j), u[j]), u[j], phi);
+#pragma unroll
                 for (int r = 0; r < NR; ++r) {
                     float c, sc;
                     bool on, iq;
                     brow<float, false>(r, P, St, (mi >> 10) & 1, (mi >> 11) & 1, x, u, dx, c, nullptr, on, iq, sc);
-                    if (on) phi += brow_al(iq, lam[r], beta, inv2b, c);
+                    if (on) phi = a2(phi, brow_al(iq, lam[r], beta, inv2b, c));
                 }
                 if (k == 0)
                     for (int i = 0; i < 3; ++i) {
                         const float c = (S.xh[i * Np1] - P.start[i]) + (S.xl[i * Np1] + alpha * S.dz[i]);
-                        phi += brow_al(false, S.lam[i], beta, inv2b, c);
+                        phi = a2(phi, brow_al(false, S.lam[i], beta, inv2b, c));
                     }
                 if (k == N - 1)
                     for (int i = 0; i < 3; ++i) {
                         const float e =
                             (S.xh[i * Np1 + N] - P.goal[i]) + (S.xl[i * Np1 + N] + alpha * S.dz[NWV * N + i]);
-                        phi += P.wT * e * e;
+                        phi = fm(m2(P.wT, e), e, phi);
                     }
             }
         }
@@ -1145,7 +1261,7 @@ __device__ BCert bcertify(BCtx& C, float beta_f) {
             g[NX + j] += 2.0 * rweight(P, j) * u[j];
             cost += rweight(P, j) * u[j] * u[j];
         }
-        const float* lam = S.lam + 3 + NR * k;
+        const float* lam = S.lam + 3 + NLAM * k;
         for (int r = 0; r < NR; ++r) {
             double c, J[NL], sc;
             bool on, iq;
@@ -1216,7 +1332,19 @@ __global__ void __launch_bounds__(kBimThreads, 4) bimanual_kernel(EvalArgs A) {
     C.lane = threadIdx.x & 31;
     C.S = bcarve(bsm, A.Nmax);
     C.rec = A.ws + (size_t)blockIdx.x * A.ws_per_warp;
+    C.jac = C.rec + (size_t)kBimRec * A.Nmax;
+    C.Nmax = A.Nmax;
     BSmem& S = C.S;
+    // where lane i's entry of row r lies in a Jacobian record (its zero if the
+    // row's pattern does not have the lane's variable)
+    for (int t = C.tid; t < NR * 32; t += kBimThreads) {
+        const int r = t >> 5, i = t & 31;
+        int at = J_ZERO;
+        for (int q = 0; q < 10 && bnz(r, q) >= 0; ++q)
+            if (i < NL && bnz(r, q) == evar(i)) at = bnz_first(r) + q;
+        S.at[t] = (uint16_t)(4 * at);
+    }
+    __syncthreads();
     const SolverParams& sp = A.sp;
     const int64_t n_tos = A.d_n ? min(*A.d_n, A.n) : A.n;
     __shared__ unsigned int s_t;
@@ -1273,7 +1401,7 @@ __global__ void __launch_bounds__(kBimThreads, 4) bimanual_kernel(EvalArgs A) {
             const int j = q / N, k = q - j * N;
             S.us[q] = warm ? warm[NX * Nm1 + j * A.Nmax + k] : ((j == ULN - 5) ? P.mg : 0.f);
         }
-        for (int q = C.tid; q < 3 + NR * N; q += kBimThreads) S.lam[q] = 0.f;
+        for (int q = C.tid; q < 3 + NLAM * N; q += kBimThreads) S.lam[q] = 0.f;
         for (int q = C.tid; q < NWV * N + NX; q += kBimThreads) S.dz[q] = S.gr[q] = 0.f;
         for (int k = C.tid; k < N; k += kBimThreads) {
             const int seg = (int)(((long long)k * len) / N);
@@ -1306,7 +1434,10 @@ __global__ void __launch_bounds__(kBimThreads, 4) bimanual_kernel(EvalArgs A) {
             bool fac = false, done = false;
             float beta_old = beta;
             for (;;) {
-                const BMeasures m = bphase_a(C, beta, rho, true, trip == kUpdate, beta_old);
+                // rows, gradient and measures; a retry keeps them (only the
+                // damping changed)
+                BMeasures m;
+                if (trip != kRetry) m = bphase_a(C, beta, trip == kUpdate, beta_old);
                 if (trip == kMeasure) {
                     if (!m.finite) {
                         status = COMET_TO_NONFINITE;
@@ -1336,6 +1467,7 @@ __global__ void __launch_bounds__(kBimThreads, 4) bimanual_kernel(EvalArgs A) {
                         continue;
                     }
                 }
+                bphase_m(C, beta, rho);
                 fac = bphase_b(C, beta, rho);
                 if (fac || retries >= sp.max_retries) break;
                 ++retries;

@@ -88,8 +88,9 @@ void merge_opts(const comet_solver_opts* opts, comet_solver_opts* out);
 void set_error(const char* msg);
 
 // Bimanual variant (bimanual_kernel.cu): one CTA of kBimThreads threads per
-// TO; per-CTA workspace kBimRec floats per stage.
-constexpr int kBimRec = 328;
+// TO; per-CTA workspace kBimRec + kBimJac floats per stage (stage records and
+// Jacobian records).
+constexpr int kBimRec = 328, kBimJac = 112;
 constexpr int kBimThreads = 128;
 size_t bim_smem_bytes(int Nmax);
 int bim_blocks_per_sm(int Nmax);
