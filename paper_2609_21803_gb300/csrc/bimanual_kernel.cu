@@ -16,13 +16,14 @@
 //      after the other as straight code (each row's index a constant), the
 //      multipliers, measures and the AL gradient; a stage's nonzeros go to the
 //      CTA's workspace (L2-resident) as one packed record
-//   M  a warp per stage: the AL model over (u, x_{k+1}, x_k) in registers, a
-//      model row per lane, from each row's nonzero pattern; the 12 u columns
-//      eliminated there (the pivot column through shared memory); records to
-//      the workspace
-//   B  one warp: the sequential sweep eliminating the 5 x_{k+1} columns, the
-//      next stage's record prefetched into registers
+//   M  a warp per two stages: the AL model over (u, x_{k+1}, x_k) in
+//      registers, a model row per lane, from each row's nonzero pattern; the
+//      12 u columns eliminated there (the pivot column through shared
+//      memory); records to the workspace, in float4s
+//   B  one warp, a row per lane: the sequential sweep eliminating the 5
+//      x_{k+1} columns, the reduced blocks copied into shared memory ahead
 //   gains and control steps stage-parallel, the forward chain on 5 lanes
+//      from gains copied ahead
 //   D  8 trial steps x stages over all threads, sums in shared memory
 //   E  compensated state update
 // Phase A used to run a lane per row: the warp then walked every row type's
@@ -30,8 +31,15 @@
 // and phase M belonged to it, so that a trip that only updates multipliers
 // built a model nobody used and a retry recomputed its rows.  With a thread
 // per stage the rows cost 50 instructions per stage; 2,048 random orders of
-// 1..6 segments take 213 -> 105 ms, the 507 one-segment orders 25 -> 15 ms,
-// with bit-identical results.
+// 1..6 segments took 213 -> 105 ms, the 507 one-segment orders 25 -> 15 ms.
+// Then the sequential parts: a lane per row and copies ahead in B and the
+// forward chain, two stages side by side and vector records in M: 105 -> 92
+// ms and 15 -> 12.4 ms.  Results are bit-identical throughout.
+//
+// What bounds it (2,048 orders, cycles per TO-iteration with 4 CTAs on an
+// SM): M 126 k, B 70 k, A 28 k, C 27 k, trials 23 k.  Issue slots are 27 %
+// used: dependent chains (roots and reciprocals of 17 pivots per stage, one
+// warp in B while three wait) and instruction fetches, not memory.
 
 #include <cuda_runtime.h>
 #include <cuda/annotated_ptr>
@@ -50,17 +58,20 @@ constexpr int NE = 23;               // elimination order (u 12, y 5, x 5, rhs)
 constexpr int NRED = 11;             // reduced block (y 5, x 5, rhs)
 constexpr int NTRI_RED = NRED * (NRED + 1) / 2;  // 66
 // record layout (floats)
-constexpr int R_LUU = 0;     // 78: u-block factor, lower triangle
-constexpr int R_CPL = 78;    // 132: coupling rows (y, x, rhs) x 12 u columns
-constexpr int R_PD = 210;    // u-block pivots positive
-constexpr int R_RED = 212;   // 66: reduced (y, x, rhs) block
-constexpr int R_YF = 280;    // 15 + 30 raw y-factor (+3 pad), then 30 gains
-static_assert(R_YF + 48 <= kBimRec, "record layout");
+// Triangles are stored a row after the other, each row in whole float4s, so
+// that a lane writes its row in one to three vector stores
+__host__ __device__ constexpr int lrow(int i) { return i < 4 ? 4 * i : i < 8 ? 16 + 8 * (i - 4) : 48 + 12 * (i - 8); }
+constexpr int R_LUU = 0;     // 96: u-block factor, lower triangle (12 rows)
+constexpr int R_CPL = 96;    // 132: coupling rows (y, x, rhs) x 12 u columns
+constexpr int R_RED = 228;   // 84: reduced (y, x, rhs) block (11 rows), its last float the u-block's PD flag
+constexpr int R_PD = R_RED + lrow(10) + 11;
+constexpr int R_YF = R_RED;  // 15 + 30 raw y-factor (+3 pad), then 30 gains, over the consumed block
+static_assert(R_PD == R_RED + 83 && R_RED + 84 <= kBimRec, "record layout");
 static_assert(R_YF % 4 == 0 && kBimRec % 4 == 0, "vector access to the raw factor");
-// sweep copy ring: record floats 208..279 (the u-block flag at 210, the
-// reduced block at 212..277), kBRing stages ahead
-constexpr int R_SLOT = 208, kBSlot = 72, kBRing = 6;
-static_assert(R_SLOT + 2 == R_PD && R_SLOT + 4 == R_RED && R_SLOT + kBSlot >= R_RED + NTRI_RED, "ring slot");
+// sweep copy ring: the reduced blocks, kBRing stages ahead
+constexpr int kBSlot = 84, kBRing = 6;
+constexpr int kCRing = 12;  // stages of gains in the same ring (forward chain)
+static_assert(kCRing * 32 <= kBRing * kBSlot, "gains ring");
 
 // stage Jacobian records (written by phase A, read by phase M): the entries of
 // every row's pattern (bnz) one row after the other, a zero, and the local
@@ -524,8 +535,8 @@ __device__ __forceinline__ void two_sum_b(float a, float b, float& s, float& e) 
 struct BSmem {
     float *xh, *xl, *us, *lam, *dz, *gr;
     int* mi;     // per interval: mode | maskL << 10 | maskR << 11
-    float* jbuf;          // per warp: two Jacobian records
-    float* col;           // per warp: two pivot columns of 24
+    float* jbuf;          // per warp: two pairs of Jacobian records
+    float* col;           // per warp: two pairs of pivot columns of 24
     uint16_t* at;         // [row][lane]: byte offset of the lane's entry in a record
     float* ring;          // sweep copy ring [kBRing][kBSlot] (16-byte aligned)
     float* red;           // reductions / broadcasts [64]
@@ -533,7 +544,7 @@ struct BSmem {
 
 __host__ __device__ inline size_t bsmem_floats(int Nmax) {
     const size_t f = (size_t)10 * (Nmax + 1) + (size_t)NU * Nmax + 3 + (size_t)NLAM * Nmax +
-                     2 * ((size_t)NWV * Nmax + NX) + (size_t)Nmax + 4 * (2 * J_REC + 48) + NR * 16 +
+                     2 * ((size_t)NWV * Nmax + NX) + (size_t)Nmax + 4 * (4 * J_REC + 96) + NR * 16 +
                      kBRing * kBSlot + 64;
     return (f + 3) / 4 * 4;
 }
@@ -541,8 +552,8 @@ __host__ __device__ inline size_t bsmem_floats(int Nmax) {
 __device__ BSmem bcarve(float* p, int Nmax) {
     BSmem s;
     s.ring = p; p += kBRing * kBSlot;  // first: 16-byte aligned
-    s.jbuf = p; p += 4 * 2 * J_REC;
-    s.col = p; p += 4 * 48;
+    s.jbuf = p; p += 4 * 4 * J_REC;
+    s.col = p; p += 4 * 96;
     s.at = reinterpret_cast<uint16_t*>(p); p += NR * 16;
     s.xh = p; p += NX * (Nmax + 1);
     s.xl = p; p += NX * (Nmax + 1);
@@ -746,208 +757,249 @@ __device__ void bphase_m(BCtx& C, float beta, float rho) {
     BSmem& S = C.S;
     const BInst<float>& P = C.P;
     const int N = C.N, lane = C.lane, warp = C.warp;
-    float* jb = S.jbuf + warp * 2 * J_REC;
-    float* colb = S.col + warp * 48;
+    float* jb = S.jbuf + warp * 4 * J_REC;
+    float* colb = S.col + warp * 96;
     auto fetch = [&](int k, int buf) {
-        if (k < N && lane < J_REC / 4)
-            bcp_async16(jb + buf * J_REC + 4 * lane, C.jac + 4 * ((int64_t)lane * C.Nmax + k));
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            if (k + 4 * h < N && lane < J_REC / 4)
+                bcp_async16(jb + (2 * buf + h) * J_REC + 4 * lane, C.jac + 4 * ((int64_t)lane * C.Nmax + k + 4 * h));
         bcp_async_commit();
     };
     fetch(warp, 0);
     int buf = 0;
+    // Stages k and k + 4 side by side: a pivot is a chain of a shuffle, a
+    // square root, a division and a trip through shared memory (about 250
+    // cycles), which the other stage shares.  Six-segment orders, 64 of them /
+    // 2,048 of mixed length: one stage at a time 92 k / 139 k cycles per
+    // iteration, two with roots of their own 96 k / 158 k (the slow paths of
+    // the exact root and division keep the chains apart), with one root for
+    // both and vector records 70 k / 126 k.  A last stage without a partner
+    // is done twice.
 #pragma unroll 1
-    for (int k = warp; k < N; k += 4, buf ^= 1) {
-        fetch(k + 4, buf ^ 1);
+    for (int k = warp; k < N; k += 8, buf ^= 1) {
+        fetch(k + 8, buf ^ 1);
         bcp_async_wait<1>();
         __syncwarp();
-        const float* J = jb + buf * J_REC;
+        const bool two = k + 4 < N;
+        const float* J0 = jb + 2 * buf * J_REC;
+        const float* Js[2] = {J0, two ? J0 + J_REC : J0};
         // lane i < 22 holds row i of the lower triangle over (u, y, x) in
         // elimination order (and lane 22 the rhs row).  Row i = sum_r J_r[v_i]
         // J_r over the active rows in row order; for row r only the columns of
         // its pattern (bnz) are added, the others being exact zeros: the
         // lane's own entry times a broadcast Jacobian value
-        float row[NE];
+        float row[2][NE];
 #pragma unroll
-        for (int cc = 0; cc < NE; ++cc) row[cc] = 0.f;
-        float4 t4 = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int cc = 0; cc < NE; ++cc) row[h][cc] = 0.f;
+        float4 t4[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
-            const float a = *reinterpret_cast<const float*>(reinterpret_cast<const char*>(J) + S.at[32 * r + lane]);
+            const int at = S.at[32 * r + lane];
 #pragma unroll
-            for (int q = 0; q < 10; ++q) {
-                if (bnz(r, q) < 0) break;
-                const int n = bnz_first(r) + q;
-                if (n % 4 == 0) t4 = *reinterpret_cast<const float4*>(J + n);
-                const float b = n % 4 == 0 ? t4.x : n % 4 == 1 ? t4.y : n % 4 == 2 ? t4.z : t4.w;
-                // a row of one entry is added as a rounded product
-                float& m = row[epos(bnz(r, q))];
-                m = bnz(r, 1) < 0 ? a2(m, m2(a, b)) : fm(a, b, m);
+            for (int h = 0; h < 2; ++h) {
+                const float a = *reinterpret_cast<const float*>(reinterpret_cast<const char*>(Js[h]) + at);
+#pragma unroll
+                for (int q = 0; q < 10; ++q) {
+                    if (bnz(r, q) < 0) break;
+                    const int n = bnz_first(r) + q;
+                    if (n % 4 == 0) t4[h] = *reinterpret_cast<const float4*>(Js[h] + n);
+                    const float b = n % 4 == 0 ? t4[h].x : n % 4 == 1 ? t4[h].y : n % 4 == 2 ? t4[h].z : t4[h].w;
+                    // a row of one entry is added as a rounded product
+                    float& m = row[h][epos(bnz(r, q))];
+                    m = bnz(r, 1) < 0 ? a2(m, m2(a, b)) : fm(a, b, m);
+                }
             }
         }
         // beta, then the cost and damping on the diagonal (u: cost + rho,
         // x_{k+1}: rho); the gradient as the rhs row (lane 22)
 #pragma unroll
         for (int cc = 0; cc < NE - 1; ++cc) {
-            row[cc] = m2(row[cc], beta);
-            if (lane == cc && cc < 17) row[cc] = a2(row[cc], cc < 12 ? fm(2.f, rweight(P, cc), rho) : rho);
-        }
+            const float dg = cc < 12 ? fm(2.f, rweight(P, cc), rho) : rho;
 #pragma unroll
-        for (int q = 0; q < 6; ++q) {
-            const float4 t = *reinterpret_cast<const float4*>(J + J_GRAD + 4 * q);
-            if (lane == NE - 1) {
-                row[4 * q] = t.x;
-                row[4 * q + 1] = t.y;
-                if (4 * q + 2 < NE - 1) {
-                    row[4 * q + 2] = t.z;
-                    row[4 * q + 3] = t.w;
-                }
+            for (int h = 0; h < 2; ++h) {
+                row[h][cc] = m2(row[h][cc], beta);
+                if (lane == cc && cc < 17) row[h][cc] = a2(row[h][cc], dg);
             }
         }
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int q = 0; q < 6; ++q) {
+                const float4 t = *reinterpret_cast<const float4*>(Js[h] + J_GRAD + 4 * q);
+                if (lane == NE - 1) {
+                    row[h][4 * q] = t.x;
+                    row[h][4 * q + 1] = t.y;
+                    if (4 * q + 2 < NE - 1) {
+                        row[h][4 * q + 2] = t.z;
+                        row[h][4 * q + 3] = t.w;
+                    }
+                }
+            }
         // eliminate the u block (12 Cholesky columns): lane i < 23 holds row i
         // of the lower triangle (entries 0..i; what the updates leave above the
         // diagonal is never read).  The scaled column goes through shared
         // memory (two buffers, one warp barrier per pivot) and comes back as
         // broadcasts, four entries a load.  A non-positive pivot marks the record.
-        bool pd = true;
+        bool pd[2] = {true, true};
 #pragma unroll
         for (int j = 0; j < 12; ++j) {
-            const float d = __shfl_sync(kFullB, row[j], j);
-            pd = pd && (d > 0.f);
-            const float l = sqrtf(fmaxf(d, 1e-30f));
+            float* col = colb + 48 * (j & 1);
+            // the lower half-warp takes stage k's pivot, the upper one k + 4's,
+            // so that both roots and reciprocals cost one pass
+            const float d0 = __shfl_sync(kFullB, row[0][j], j), d1 = __shfl_sync(kFullB, row[1][j], j);
+            pd[0] = pd[0] && (d0 > 0.f);
+            pd[1] = pd[1] && (d1 > 0.f);
+            const float l = sqrtf(fmaxf(lane < 16 ? d0 : d1, 1e-30f));
             const float il = 1.f / l;
-            row[j] = lane == j ? l : row[j] * il;
-            float* col = colb + 24 * (j & 1);
-            if (lane < 24) col[lane] = row[j];
+            const float lx = __shfl_xor_sync(kFullB, l, 16), ilx = __shfl_xor_sync(kFullB, il, 16);
+            row[0][j] = lane == j ? l : m2(row[0][j], lane < 16 ? il : ilx);  // j < 16: l is the lane's own
+            row[1][j] = lane == j ? lx : m2(row[1][j], lane < 16 ? ilx : il);
+            if (lane < 24) {
+                col[lane] = row[0][j];
+                col[24 + lane] = row[1][j];
+            }
             __syncwarp();
 #pragma unroll
-            for (int q = (j + 1) / 4; q < 6; ++q) {
-                const float4 t = *reinterpret_cast<const float4*>(col + 4 * q);
-                const float b[4] = {t.x, t.y, t.z, t.w};
+            for (int q = (j + 1) / 4; q < 6; ++q)
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    if (4 * q + i > j && 4 * q + i < NE) row[4 * q + i] = fm(-row[j], b[i], row[4 * q + i]);
-            }
+                for (int h = 0; h < 2; ++h) {
+                    const float4 t = *reinterpret_cast<const float4*>(col + 24 * h + 4 * q);
+                    const float b[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (4 * q + i > j && 4 * q + i < NE)
+                            row[h][4 * q + i] = fm(-row[h][j], b[i], row[h][4 * q + i]);
+                }
         }
         // records from the rows: the u factor (rows 0..11), the coupling
         // rows (12..22) x u columns, the reduced (y, x, rhs) block
         // record stores with the persisting (evict-last) L2 priority: the
         // CTAs' workspaces fit in L2 and are rewritten every iteration
-        cuda::annotated_ptr<float, cuda::access_property::persisting> rec(C.rec + (size_t)k * kBimRec);
-        if (lane < 12) {
 #pragma unroll
-            for (int cc = 0; cc < 12; ++cc)
-                if (cc <= lane) rec[R_LUU + tri(lane, cc)] = row[cc];
-        } else if (lane < NE) {
-            const int p = lane - 12;
-#pragma unroll
-            for (int cc = 0; cc < 12; ++cc) rec[R_CPL + 12 * p + cc] = row[cc];
-#pragma unroll
-            for (int cc = 12; cc < NE; ++cc)
-                if (cc <= lane) rec[R_RED + tri(p, cc - 12)] = row[cc];
+        for (int h = 0; h < 2; ++h) {
+            if (h == 1 && !two) break;
+            float* rk = C.rec + (size_t)(k + 4 * h) * kBimRec;
+            const float* w = row[h];
+            if (lane < NE) {
+                cuda::annotated_ptr<float4, cuda::access_property::persisting> rec(
+                    reinterpret_cast<float4*>(rk + (lane < 12 ? R_LUU + lrow(lane) : R_CPL + 12 * (lane - 12))));
+                rec[0] = make_float4(w[0], w[1], w[2], w[3]);
+                if (lane >= 4) rec[1] = make_float4(w[4], w[5], w[6], w[7]);
+                if (lane >= 8) rec[2] = make_float4(w[8], w[9], w[10], w[11]);
+            }
+            if (lane >= 12 && lane < NE) {
+                cuda::annotated_ptr<float4, cuda::access_property::persisting> rec(
+                    reinterpret_cast<float4*>(rk + R_RED + lrow(lane - 12)));
+                rec[0] = make_float4(w[12], w[13], w[14], w[15]);
+                if (lane >= 16) rec[1] = make_float4(w[16], w[17], w[18], w[19]);
+                if (lane >= 20) rec[2] = make_float4(w[20], w[21], w[22], pd[h] ? 1.f : -1.f);
+            }
         }
-        if (lane == 0) rec[R_PD] = pd ? 1.f : -1.f;
         __syncwarp();
     }
     bcp_async_wait_all();
     __syncthreads();
 }
 
-// Sweep over k = N-1 .. 0 on warp 0.  Every lane runs the whole stage in
-// registers (the sequential chain is short and dependent): the reduced
-// 11 x 11 lower triangle (rows y 0..4, x 0..4, rhs) arrives from the record
-// through a cp.async ring kBRing stages ahead and is read as shared-memory
-// broadcasts, V_{k+1} and v_{k+1} stay in registers, the 5 y columns are
-// eliminated with SFU reciprocal pivots, and lane 0 writes the raw y-factor
-// columns (15 y-y entries, then the (x, rhs) rows) for the gains.  Then the
-// x_0 block; publishes the factorisation status to all threads and dx0 into
-// red[16..20].
+// Sweep over k = N-1 .. 0 on warp 0, a lane per row of the reduced 11 x 11
+// lower triangle (y 0..4, x 0..4, rhs; the lanes above repeat the rhs row).
+// The block arrives from the record through a cp.async ring kBRing stages
+// ahead.  V_{k+1} and v_{k+1} are the rows 5.. of the stage before: a shuffle
+// of five values moves V to the y rows, v stays in the rhs lane.  Per pivot
+// the lanes take the raw pivot column by shuffles while the SFU reciprocal of
+// the pivot is under way; a lane writes its row's raw y-factor entries (15 y-y
+// entries, then the (x, rhs) rows) for the gains.  Every lane running the
+// whole stage (330 instructions, about 1,100 cycles) took 57 k cycles per
+// iteration on 64 six-segment orders and 78 k on 2,048 mixed ones, this takes
+// 56 k and 70 k.  Then the x_0 block; publishes the
+// factorisation status to all threads and dx0 into red[16..20].
 __device__ bool bphase_b(BCtx& C, float beta, float rho) {
     BSmem& S = C.S;
     const BInst<float>& P = C.P;
     const int N = C.N, Np1 = C.Np1, lane = C.lane;
     if (C.warp == 0) {
-        float V[15], v[5];
+        const int row = min(lane, 10), at0 = lrow(row);
+        // rows 5.. of "stage N": the terminal cost's V_N (lanes 5..9), v_N (lane 10)
+        float m[11];
 #pragma unroll
-        for (int i = 0; i < 5; ++i) {
+        for (int l = 0; l < 11; ++l) m[l] = 0.f;
 #pragma unroll
-            for (int j = 0; j <= i; ++j) V[tri(i, j)] = (i == j && i < 3) ? 2.f * P.wT : 0.f;
-            v[i] = i < 3 ? 2.f * P.wT * ((S.xh[i * Np1 + N] - P.goal[i]) + S.xl[i * Np1 + N]) : 0.f;
+        for (int l = 0; l < 3; ++l) {
+            if (lane == 5 + l) m[5 + l] = 2.f * P.wT;
+            if (row == 10) m[5 + l] = 2.f * P.wT * ((S.xh[l * Np1 + N] - P.goal[l]) + S.xl[l * Np1 + N]);
         }
 #pragma unroll
         for (int d = 0; d < kBRing; ++d) {
             const int kk = N - 1 - d;
             if (kk >= 0 && lane < kBSlot / 4)
-                bcp_async16(S.ring + d * kBSlot + 4 * lane, C.rec + (size_t)kk * kBimRec + R_SLOT + 4 * lane);
+                bcp_async16(S.ring + d * kBSlot + 4 * lane, C.rec + (size_t)kk * kBimRec + R_RED + 4 * lane);
             bcp_async_commit();
         }
         bool ok = true;
         int slot = kBRing - 1;  // ring slot of stage k: (N - 1 - k) mod kBRing
+        // where the lane's y-factor entries go: row i < 5 its entries 0..i, the
+        // others five entries each
+        const int out0 = R_YF + (row < 5 ? row * (row + 1) / 2 : 15 + 5 * (row - 5));
 #pragma unroll 1
         for (int k = N - 1; k >= 0; --k) {
             slot = (slot == kBRing - 1) ? 0 : slot + 1;
             bcp_async_wait<kBRing - 1>();
             __syncwarp();
-            const float4* sl = reinterpret_cast<const float4*>(S.ring + slot * kBSlot);
-            const float4 hd = sl[0];  // record floats 208..211: the u-block flag at 210
-            float m[68];
+            const float* sl = S.ring + slot * kBSlot;
+            bool pd = sl[R_PD - R_RED] > 0.f;
+            float V[5];
 #pragma unroll
-            for (int q = 0; q < 17; ++q) {
-                const float4 t = sl[1 + q];
-                m[4 * q] = t.x;
-                m[4 * q + 1] = t.y;
-                m[4 * q + 2] = t.z;
-                m[4 * q + 3] = t.w;
+            for (int l = 0; l < 5; ++l) {
+                const float t = __shfl_sync(kFullB, m[5 + l], (lane + 5) & 31);
+                V[l] = row == 10 ? m[5 + l] : t;
             }
-            bool pd = hd.z > 0.f;
+            // entries past the row's own are never used (they stay inside the slot)
+#pragma unroll
+            for (int l = 0; l < 11; ++l) m[l] = sl[at0 + l];
             __syncwarp();
             {
                 const int kk = k - kBRing;
                 if (kk >= 0 && lane < kBSlot / 4)
-                    bcp_async16(S.ring + slot * kBSlot + 4 * lane, C.rec + (size_t)kk * kBimRec + R_SLOT + 4 * lane);
+                    bcp_async16(S.ring + slot * kBSlot + 4 * lane, C.rec + (size_t)kk * kBimRec + R_RED + 4 * lane);
                 bcp_async_commit();
             }
 #pragma unroll
-            for (int t = 0; t < 15; ++t) m[t] += V[t];
-#pragma unroll
-            for (int j = 0; j < 5; ++j) m[tri(10, j)] += v[j];
+            for (int l = 0; l < 5; ++l)
+                if (row < 5 || row == 10) m[l] = a2(m[l], V[l]);
 #pragma unroll
             for (int j = 0; j < 5; ++j) {
-                const float p = m[tri(j, j)];
+                const float p = __shfl_sync(kFullB, m[j], j);
+                float c[11];
+#pragma unroll
+                for (int l = j + 1; l < 11; ++l) c[l] = __shfl_sync(kFullB, m[j], l);
                 pd = pd && (p > 0.f);
-                const float ip = brcp_approx(p);
+                const float a = m2(m[j], brcp_approx(p));
+                if (row > j) {
 #pragma unroll
-                for (int i = j + 1; i < 11; ++i) {
-                    const float a = m[tri(i, j)] * ip;
-#pragma unroll
-                    for (int l = j + 1; l <= i; ++l)
-                        if (!(i == 10 && l == 10)) m[tri(i, l)] -= a * m[tri(l, j)];
+                    for (int l = j + 1; l < 11; ++l) m[l] = fm(-a, c[l], m[l]);
                 }
             }
-            if (!__all_sync(kFullB, pd)) {
+            if (!pd) {  // the same on every lane
                 ok = false;
                 break;
             }
-            if (lane == 0) {
-                // 45 raw factor entries (+3 pad) as 12 vector stores
-                float o[48];
+            if (lane < 11) {
+                cuda::annotated_ptr<float, cuda::access_property::persisting> o(C.rec + (size_t)k * kBimRec + out0);
 #pragma unroll
-                for (int t = 0; t < 15; ++t) o[t] = m[t];
-#pragma unroll
-                for (int c = 0; c < 6; ++c)
-#pragma unroll
-                    for (int j = 0; j < 5; ++j) o[15 + 5 * c + j] = m[tri(5 + c, j)];
-                o[45] = o[46] = o[47] = 0.f;
-                cuda::annotated_ptr<float4, cuda::access_property::persisting> r4(
-                    reinterpret_cast<float4*>(C.rec + (size_t)k * kBimRec + R_YF));
-#pragma unroll
-                for (int q = 0; q < 12; ++q) r4[q] = make_float4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
+                for (int j = 0; j < 5; ++j)
+                    if (row >= 5 || j <= row) o[j] = m[j];
             }
+        }
+        // V_0, v_0 to every lane
+        float V[15], v[5];
 #pragma unroll
-            for (int i = 0; i < 5; ++i) {
+        for (int i = 0; i < 5; ++i) {
 #pragma unroll
-                for (int j = 0; j <= i; ++j) V[tri(i, j)] = m[tri(5 + i, 5 + j)];
-                v[i] = m[tri(10, 5 + i)];
-            }
+            for (int j = 0; j <= i; ++j) V[tri(i, j)] = __shfl_sync(kFullB, m[5 + j], 5 + i);
+            v[i] = __shfl_sync(kFullB, m[5 + i], 10);
         }
         bcp_async_wait_all();
         __syncwarp();
@@ -1067,19 +1119,37 @@ __device__ float bphase_c(BCtx& C) {
         float dxv[5];
         #pragma unroll
         for (int i = 0; i < 5; ++i) dxv[i] = __shfl_sync(kFullB, dxi, i);
+        // the gains arrive through a copy ring kCRing stages ahead (a stage's
+        // 32 floats per slot); read from the workspace one stage at a time,
+        // the chain waited for the L2 at every stage (gains, chain and control
+        // steps together 44 k cycles per iteration of 2,048 orders, now 27 k)
+        auto fetch = [&](int k) {
+            if (k < N && C.lane < 8)
+                bcp_async16(S.ring + (k % kCRing) * 32 + 4 * C.lane, C.rec + (size_t)k * kBimRec + R_YF + 4 * C.lane);
+            bcp_async_commit();
+        };
+#pragma unroll
+        for (int k = 0; k < kCRing; ++k) fetch(k);
+        const int gl = C.lane < 5 ? 6 * C.lane : 0;
 #pragma unroll 1
         for (int k = 0; k < N; ++k) {
-            float w = 0.f;
-            if (C.lane < 5) {
-                const float* g = C.rec + (size_t)k * kBimRec + R_YF + 6 * C.lane;
-                w = g[5];
-                #pragma unroll
-                for (int j = 0; j < 5; ++j) w += g[j] * dxv[j];
-                S.dz[NWV * (k + 1) + C.lane] = w;
-            }
+            bcp_async_wait<kCRing - 1>();
+            __syncwarp();
+            const float* g = S.ring + (k % kCRing) * 32 + gl;
+            float gv[6];
+            #pragma unroll
+            for (int j = 0; j < 6; ++j) gv[j] = g[j];
+            __syncwarp();
+            fetch(k + kCRing);
+            float w = gv[5];
+            #pragma unroll
+            for (int j = 0; j < 5; ++j) w = fm(gv[j], dxv[j], w);
+            if (C.lane < 5) S.dz[NWV * (k + 1) + C.lane] = w;
             #pragma unroll
             for (int i = 0; i < 5; ++i) dxv[i] = __shfl_sync(kFullB, w, i);
         }
+        bcp_async_wait_all();
+        __syncwarp();
     }
     __syncthreads();
 #pragma unroll 1
@@ -1091,21 +1161,43 @@ __device__ float bphase_c(BCtx& C) {
             xa[i] = S.dz[NWV * k + i];
             xb[i] = S.dz[NWV * (k + 1) + i];
         }
+        // R = l_rhs + l_y dx_{k+1} + l_x dx_k over the u columns, then
+        // L^T du = -R; the record's rows as vector loads
+        auto vec = [&](int at, int q) { return *reinterpret_cast<const float4*>(rec + at + 4 * q); };
         float R[NU];
         #pragma unroll
-        for (int j = 0; j < NU; ++j) {
-            float s = rec[R_CPL + 10 * 12 + j];
-            #pragma unroll
-            for (int i = 0; i < 5; ++i) s += rec[R_CPL + i * 12 + j] * xb[i] + rec[R_CPL + (5 + i) * 12 + j] * xa[i];
-            R[j] = s;
+        for (int q = 0; q < 3; ++q) {
+            const float4 t = vec(R_CPL + 12 * 10, q);
+            R[4 * q] = t.x, R[4 * q + 1] = t.y, R[4 * q + 2] = t.z, R[4 * q + 3] = t.w;
         }
+        #pragma unroll
+        for (int i = 0; i < 5; ++i)
+            #pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                const float4 y = vec(R_CPL + 12 * i, q), x = vec(R_CPL + 12 * (5 + i), q);
+                const float yv[4] = {y.x, y.y, y.z, y.w}, xv[4] = {x.x, x.y, x.z, x.w};
+                #pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    R[4 * q + e] = a2(R[4 * q + e], fm(yv[e], xb[i], m2(xv[e], xa[i])));
+            }
+        float L[78];
+        #pragma unroll
+        for (int i = 0; i < NU; ++i)
+            #pragma unroll
+            for (int q = 0; q <= i / 4; ++q) {
+                const float4 t = vec(R_LUU + lrow(i), q);
+                const float v[4] = {t.x, t.y, t.z, t.w};
+                #pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (4 * q + e <= i) L[tri(i, 4 * q + e)] = v[e];
+            }
         float du[NU];
         #pragma unroll
         for (int j = NU - 1; j >= 0; --j) {
             float s = -R[j];
             #pragma unroll
-            for (int i = j + 1; i < NU; ++i) s -= rec[R_LUU + tri(i, j)] * du[i];
-            du[j] = s / rec[R_LUU + tri(j, j)];
+            for (int i = j + 1; i < NU; ++i) s = fm(-L[tri(i, j)], du[i], s);
+            du[j] = s / L[tri(j, j)];
         }
         #pragma unroll
         for (int j = 0; j < NU; ++j) S.dz[NWV * k + NX + j] = du[j];

@@ -90,7 +90,7 @@ void set_error(const char* msg);
 // Bimanual variant (bimanual_kernel.cu): one CTA of kBimThreads threads per
 // TO; per-CTA workspace kBimRec + kBimJac floats per stage (stage records and
 // Jacobian records).
-constexpr int kBimRec = 328, kBimJac = 112;
+constexpr int kBimRec = 312, kBimJac = 112;
 constexpr int kBimThreads = 128;
 size_t bim_smem_bytes(int Nmax);
 int bim_blocks_per_sm(int Nmax);
