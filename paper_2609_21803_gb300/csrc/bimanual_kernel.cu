@@ -1610,9 +1610,16 @@ __global__ void __launch_bounds__(kBimThreads, 4) bimanual_kernel(EvalArgs A) {
 
 size_t bim_smem_bytes(int Nmax) { return bsmem_floats(Nmax) * sizeof(float); }
 
+namespace {
+SmemLimit g_smem_limit;
+cudaError_t set_smem(size_t smem) {
+    return cudaFuncSetAttribute(bimanual_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
+}  // namespace
+
 int bim_blocks_per_sm(int Nmax) {
     const size_t smem = bim_smem_bytes(Nmax);
-    if (cudaFuncSetAttribute(bimanual_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    if (g_smem_limit.raise(smem, set_smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }

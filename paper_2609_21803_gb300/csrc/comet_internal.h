@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
+
 #include "comet.h"
 
 namespace comet {
@@ -86,6 +88,28 @@ SolverParams make_params(const comet_solver_opts& o, int max_iters);
 comet_status check_instances(const comet_instance_desc* inst, int32_t n_instances, int* Nmax_out);
 void merge_opts(const comet_solver_opts* opts, comet_solver_opts* out);
 void set_error(const char* msg);
+
+// A kernel's shared-memory limit on each device, only ever raised: problems of
+// several sizes are alive at once, and creating a small one (which asks for the
+// occupancy at its own size) must not take a larger one's launches away.
+// `set(bytes)` sets the attribute on the current device.
+class SmemLimit {
+    std::mutex m_;
+    size_t at_[64] = {};
+
+public:
+    template <class Set>
+    cudaError_t raise(size_t smem, Set set) {
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        std::lock_guard<std::mutex> lock(m_);
+        if (dev < 64 && at_[dev] >= smem) return cudaSuccess;
+        e = set(smem);
+        if (e == cudaSuccess && dev < 64) at_[dev] = smem;
+        return e;
+    }
+};
 
 // Bimanual variant (bimanual_kernel.cu): one CTA of kBimThreads threads per
 // TO; per-CTA workspace kBimRec + kBimJac floats per stage (stage records and

@@ -1668,11 +1668,12 @@ cudaError_t set_smem_all(size_t smem) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(eval_kernel<false, true, 2>, at, b);
     return e;
 }
+SmemLimit g_smem_limit;
 }  // namespace
 
 int eval_blocks_per_sm(int warps_per_block, size_t smem_per_block) {
     int nb = 0;
-    if (set_smem_all(smem_per_block) != cudaSuccess) {
+    if (g_smem_limit.raise(smem_per_block, set_smem_all) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -1686,18 +1687,10 @@ int eval_blocks_per_sm(int warps_per_block, size_t smem_per_block) {
 
 cudaError_t launch_eval(const EvalArgs& a, int total_warps, int warps_per_block, cudaStream_t s) {
     const size_t smem = smem_per_warp_bytes(a.Nmax) * warps_per_block;
-    // the attribute is raised to the largest size seen on this device; it is
     // not a stream operation, so raising it outside of a capture keeps
     // launches capturable (problem creation raises it first)
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    const cudaError_t e = g_smem_limit.raise(smem, set_smem_all);
     if (e != cudaSuccess) return e;
-    static size_t raised[64] = {};
-    if (dev < 64 && raised[dev] < smem) {
-        e = set_smem_all(smem);
-        if (e != cudaSuccess) return e;
-        raised[dev] = smem;
-    }
     const int blocks = (total_warps + warps_per_block - 1) / warps_per_block;
     const bool refine = a.sp.refine && a.sp.refine_beta < a.sp.beta_max;
     const bool unr2 = a.unroll == 2 && !refine;

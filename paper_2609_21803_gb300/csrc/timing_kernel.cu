@@ -1434,9 +1434,16 @@ size_t timing_smem_per_warp_bytes(int Nmax) { return tsmem_floats(Nmax) * sizeof
 
 int64_t timing_ws_per_warp_floats(int Nmax) { return (int64_t)kTRec * Nmax; }
 
+namespace {
+SmemLimit g_smem_limit;
+cudaError_t set_smem(size_t smem) {
+    return cudaFuncSetAttribute(timing_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
+}  // namespace
+
 int timing_blocks_per_sm(int warps_per_block, int Nmax) {
     const size_t smem = timing_smem_per_warp_bytes(Nmax) * warps_per_block;
-    if (cudaFuncSetAttribute(timing_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    if (g_smem_limit.raise(smem, set_smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -1450,7 +1457,7 @@ int timing_blocks_per_sm(int warps_per_block, int Nmax) {
 
 cudaError_t launch_timing(const TimingArgs& a, int total_warps, int warps_per_block, cudaStream_t s) {
     const size_t smem = timing_smem_per_warp_bytes(a.e.Nmax) * warps_per_block;
-    cudaError_t e = cudaFuncSetAttribute(timing_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = g_smem_limit.raise(smem, set_smem);
     if (e != cudaSuccess) return e;
     const int blocks = (total_warps + warps_per_block - 1) / warps_per_block;
     timing_kernel<<<blocks, warps_per_block * 32, smem, s>>>(a);
