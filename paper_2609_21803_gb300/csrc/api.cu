@@ -272,9 +272,11 @@ static int64_t resident_warps(const comet_problem* p, int64_t n) {
     return ((std::min<int64_t>(resident, std::max<int64_t>(n, 1)) + wpb - 1) / wpb) * wpb;
 }
 
-// floats of workspace per unit (a warp for pushing, a CTA for bimanual)
+// floats of workspace per unit (a warp for pushing, whose records lie by rows
+// of 32 stages; a CTA for bimanual)
 static int64_t ws_unit_floats(const comet_problem* p) {
-    return (int64_t)(p->task == COMET_TASK_BIMANUAL ? kBimRec + kBimJac : kRec) * p->Nmax;
+    if (p->task == COMET_TASK_BIMANUAL) return (int64_t)(kBimRec + kBimJac) * p->Nmax;
+    return (int64_t)kRec * round32(p->Nmax);
 }
 
 comet_status reserve_eval(comet_problem* p, int64_t n) {

@@ -14,6 +14,8 @@ namespace comet {
 // Floats per stage record in the per-warp workspace: the u-block Cholesky
 // factor and coupling (33), the reduced (y, x, rhs) matrix (44), padded.
 constexpr int kRec = 80;
+// Records of one TO take whole rows of 32 stages.
+constexpr int round32(int n) { return (n + 31) / 32 * 32; }
 // Largest number of intervals of one TO.
 constexpr int kMaxN = 4096;
 

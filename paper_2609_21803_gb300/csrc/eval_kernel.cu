@@ -380,24 +380,39 @@ struct Ctx {
     uint16_t modes[COMET_MAX_SEGMENTS];
     int len, N, Nmax;
     Smem sm;
-    float* rec;  // this warp's stage records (chunk-major, see rec_chunk)
+    float* rec;  // this warp's stage records (see rec_chunk)
     int lane;
 };
 
-// Stage records are stored chunk-major: float4 chunk q (record floats
-// 4q .. 4q+3) of stage k sits at rec + 4 (q N_max + k), so that the
-// stage-parallel passes (lane = stage) move whole 128-byte lines, while the
-// sequential passes still fetch a stage's chunks 16 bytes at a time.
-__device__ __forceinline__ float4* rec_chunk(const Ctx& C, int q, int k) {
-    return reinterpret_cast<float4*>(C.rec + 4 * ((size_t)q * C.Nmax + k));
+// Stage records lie by the lane that eliminates the stage: with `per` stages
+// a lane (phase B), stage k = per l + j has float4 chunk q (record floats
+// 4q .. 4q+3) at float4 (kRec / 4 j + q) 32 + l.  Phase B's lanes then take
+// a chunk as whole 128-byte lines, phases A and C (32 consecutive stages) as
+// `per` runs of a row, and the chunks of a record are constant offsets apart.
+// In stage order the lanes of phase B read 16 bytes of every per-th place, a
+// sector each: 20,736 orders of N = 80 took 67.0 ms against 64.6 now, 16,384
+// mixed ones (N up to 145) 64.4 against 59.1.
+constexpr int kRecRow = 32 * (kRec / 4);  // float4s of one stage of every lane
+
+__device__ __forceinline__ float4* rec_chunk(const Ctx& C, int q, int at) {
+    return reinterpret_cast<float4*>(C.rec) + at + 32 * q;
+}
+
+// place (chunk 0) of stage k
+__device__ __forceinline__ int rec_at(const Ctx& C, int k) {
+    const int per = (C.N + 31) >> 5;
+    // k / per: (k + 1/2) / per is at least 1 / (2 per) off an integer, and the
+    // approximate reciprocal's error is below k / per 2^-21, k < kMaxN
+    const int l = (int)(((float)k + 0.5f) * __fdividef(1.f, (float)per));
+    return kRecRow * (k - l * per) + l;
 }
 
 // Record stores carry the persisting (evict-last) L2 priority: the records
 // of all resident warps (about 47 MB at N = 80) fit in L2 and are rewritten
 // every iteration, and with the normal priority they were written back to
 // DRAM at 1.1 GB per 4,096 TOs; with it, 46 MB, at the same speed.
-__device__ __forceinline__ void rec_st(const Ctx& C, int q, int k, float4 v) {
-    cuda::annotated_ptr<float4, cuda::access_property::persisting> p(rec_chunk(C, q, k));
+__device__ __forceinline__ void rec_st(const Ctx& C, int q, int at, float4 v) {
+    cuda::annotated_ptr<float4, cuda::access_property::persisting> p(rec_chunk(C, q, at));
     *p = v;
 }
 
@@ -583,6 +598,7 @@ __device__ Measures phase_a(Ctx& C, float beta, float rho, bool curvature, bool 
 #pragma unroll
                     for (int i = c; i < 12; ++i) A[tri(i, c)] -= A[tri(i, j)] * A[tri(c, j)];
             }
+            const int at = rec_at(C, k);
             float rec[kRec];
             rec[0] = A[tri(0, 0)]; rec[1] = A[tri(1, 0)]; rec[2] = A[tri(1, 1)];
             rec[3] = A[tri(2, 0)]; rec[4] = A[tri(2, 1)]; rec[5] = A[tri(2, 2)];
@@ -600,7 +616,7 @@ __device__ Measures phase_a(Ctx& C, float beta, float rho, bool curvature, bool 
                     if (!(i == 11 && j == 11)) rec[36 + tri(i - 3, j - 3)] = A[tri(i, j)];
 #pragma unroll
             for (int q = 0; q < kRec / 4; ++q)
-                rec_st(C, q, k, make_float4(rec[4 * q], rec[4 * q + 1], rec[4 * q + 2], rec[4 * q + 3]));
+                rec_st(C, q, at, make_float4(rec[4 * q], rec[4 * q + 1], rec[4 * q + 2], rec[4 * q + 3]));
         }
     }
     __syncwarp();
@@ -691,13 +707,13 @@ __device__ Measures phase_a(Ctx& C, float beta, float rho, bool curvature, bool 
 
 constexpr int kElem = 44;  // 9 x 9 lower triangle without the (rhs, rhs) entry
 
-// record floats 36..79 (the reduced matrix) of stage k as an element, with
-// the boundary terms of the first and the last stage
-__device__ __forceinline__ void load_elem(const Ctx& C, int k, float e[kElem], float beta, float rho,
+// record floats 36..79 (the reduced matrix) of stage k (at `at`) as an
+// element, with the boundary terms of the first and the last stage
+__device__ __forceinline__ void load_elem(const Ctx& C, int k, int at, float e[kElem], float beta, float rho,
                                           bool rhs_from_gr) {
 #pragma unroll
     for (int q = 0; q < 11; ++q) {
-        const float4 t = *rec_chunk(C, 9 + q, k);
+        const float4 t = *rec_chunk(C, 9 + q, at);
         e[4 * q] = t.x;
         e[4 * q + 1] = t.y;
         e[4 * q + 2] = t.z;
@@ -730,8 +746,8 @@ __device__ __forceinline__ void load_elem(const Ctx& C, int k, float e[kElem], f
 
 // Eliminate the node shared by e (over (y = m, x = a)) and f (over (y = b,
 // x = m)); e becomes the element over (y = b, x = a).  Stores (L, Y) of node
-// m in record `km` when `store`; returns false on a non-positive pivot.
-__device__ __forceinline__ bool combine(const Ctx& C, float e[kElem], const float f[kElem], int km, bool store) {
+// m in the record at `at` when `store`; returns false on a non-positive pivot.
+__device__ __forceinline__ bool combine(const Ctx& C, float e[kElem], const float f[kElem], int at, bool store) {
     // S = E_yy + F_xx and its Cholesky factor (il = 1 / l_jj on the diagonal)
     float L[10];
 #pragma unroll
@@ -788,12 +804,12 @@ __device__ __forceinline__ bool combine(const Ctx& C, float e[kElem], const floa
 #pragma unroll
     for (int t = 0; t < kElem; ++t) e[t] = g[t];
     if (store) {
-        *reinterpret_cast<float2*>(reinterpret_cast<float*>(rec_chunk(C, 8, km)) + 2) = make_float2(L[0], L[1]);
-        rec_st(C, 9, km, make_float4(L[2], L[3], L[4], L[5]));
-        rec_st(C, 10, km, make_float4(L[6], L[7], L[8], L[9]));
+        *reinterpret_cast<float2*>(reinterpret_cast<float*>(rec_chunk(C, 8, at)) + 2) = make_float2(L[0], L[1]);
+        rec_st(C, 9, at, make_float4(L[2], L[3], L[4], L[5]));
+        rec_st(C, 10, at, make_float4(L[6], L[7], L[8], L[9]));
 #pragma unroll
         for (int q = 0; q < 9; ++q)
-            rec_st(C, 11 + q, km, make_float4(Y[(4 * q) / 9][(4 * q) % 9], Y[(4 * q + 1) / 9][(4 * q + 1) % 9],
+            rec_st(C, 11 + q, at, make_float4(Y[(4 * q) / 9][(4 * q) % 9], Y[(4 * q + 1) / 9][(4 * q + 1) % 9],
                                               Y[(4 * q + 2) / 9][(4 * q + 2) % 9],
                                               Y[(4 * q + 3) / 9][(4 * q + 3) % 9]));
     }
@@ -801,14 +817,14 @@ __device__ __forceinline__ bool combine(const Ctx& C, float e[kElem], const floa
 }
 
 // dx_m = -L^{-T} (Y_b dx_b + Y_a dx_a + y_r) from node m's stored (L, Y)
-__device__ __forceinline__ void back_node(const Ctx& C, int km, const float xa[4], const float xb[4], float xm[4]) {
+__device__ __forceinline__ void back_node(const Ctx& C, int at, const float xa[4], const float xb[4], float xm[4]) {
     float v[48];
-    const float2 h = *reinterpret_cast<const float2*>(reinterpret_cast<const float*>(rec_chunk(C, 8, km)) + 2);
+    const float2 h = *reinterpret_cast<const float2*>(reinterpret_cast<const float*>(rec_chunk(C, 8, at)) + 2);
     v[0] = h.x;
     v[1] = h.y;
 #pragma unroll
     for (int q = 0; q < 11; ++q) {
-        const float4 t = *rec_chunk(C, 9 + q, km);
+        const float4 t = *rec_chunk(C, 9 + q, at);
         v[2 + 4 * q] = t.x;
         v[3 + 4 * q] = t.y;
         v[4 + 4 * q] = t.z;
@@ -848,8 +864,8 @@ __device__ bool phase_b(Ctx& C, float beta, float rho, bool rhs_from_gr = false)
 #pragma unroll
     for (int t = 0; t < kElem; ++t) e[t] = 0.f;
     if (own) {
-        pd = reinterpret_cast<const float*>(rec_chunk(C, 8, k0))[1] > 0.f;
-        load_elem(C, k0, e, beta, rho, rhs_from_gr);
+        pd = reinterpret_cast<const float*>(rec_chunk(C, 8, lane))[1] > 0.f;
+        load_elem(C, k0, lane, e, beta, rho, rhs_from_gr);
     }
     // 1-2. one loop, one elimination call site: steps 0 .. per-2 fold the
     // lane's next stage (the u-block pivot flag of phase A checked on the
@@ -859,22 +875,23 @@ __device__ bool phase_b(Ctx& C, float beta, float rho, bool rhs_from_gr = false)
     for (int st = 0; st < nsteps; ++st) {
         float f[kElem];
         bool act;
-        int km;
+        int at;
         if (st < per - 1) {  // warp-uniform
-            km = k0 + 1 + st;
+            const int km = k0 + 1 + st;
             act = own && km < k1;
+            at = kRecRow * (st + 1) + lane;
             if (act) {
-                pd = pd && reinterpret_cast<const float*>(rec_chunk(C, 8, km))[1] > 0.f;
-                load_elem(C, km, f, beta, rho, rhs_from_gr);
+                pd = pd && reinterpret_cast<const float*>(rec_chunk(C, 8, at))[1] > 0.f;
+                load_elem(C, km, at, f, beta, rho, rhs_from_gr);
             }
         } else {
             const int d = 1 << (st - (per - 1));
 #pragma unroll
             for (int t = 0; t < kElem; ++t) f[t] = __shfl_down_sync(kFull, e[t], d);
             act = (lane & (2 * d - 1)) == 0 && lane + d < nl;
-            km = (lane + d) * per;
+            at = lane + d;  // the first node of lane l + d's span
         }
-        if (act) pd = combine(C, e, f, km, true) && pd;
+        if (act) pd = combine(C, e, f, at, true) && pd;
     }
     // 3. lane 0 solves the root element over (x_N, x_0): an 8 x 8 Cholesky
     float xl[4] = {0.f, 0.f, 0.f, 0.f}, xr[4] = {0.f, 0.f, 0.f, 0.f};
@@ -931,9 +948,9 @@ __device__ bool phase_b(Ctx& C, float beta, float rho, bool rhs_from_gr = false)
 #pragma unroll
             for (int i = 0; i < 4; ++i) xc[i] = xr[i];
         const bool act = tree ? ((lane & (2 * d - 1)) == 0 && lane + d < nl) : (own && k0 + 1 + st < k1);
-        const int km = tree ? (lane + d) * per : k0 + 1 + st;
+        const int km = k0 + 1 + st;
         float xm[4] = {0.f, 0.f, 0.f, 0.f};
-        if (act) back_node(C, km, xl, tree ? xr : xc, xm);
+        if (act) back_node(C, tree ? lane + d : kRecRow * (st + 1) + lane, xl, tree ? xr : xc, xm);
         if (tree) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -975,10 +992,11 @@ __device__ float phase_c(Ctx& C) {
     for (int k = lane; k < N; k += 32) {
         // record floats 0..35 as 9 vector loads (u-block factor, 1 / l_jj on
         // its diagonal, and the coupling columns)
+        const int at = rec_at(C, k);
         float f[36];
 #pragma unroll
         for (int q = 0; q < 9; ++q) {
-            const float4 t = *rec_chunk(C, q, k);
+            const float4 t = *rec_chunk(C, q, at);
             f[4 * q] = t.x;
             f[4 * q + 1] = t.y;
             f[4 * q + 2] = t.z;

@@ -123,7 +123,7 @@ extern "C" comet_status comet_eval_modes_noalloc(const comet_instance_desc* inst
         comet::eval_blocks_per_sm(warps_per_block, comet::smem_per_warp_bytes(Nmax) * warps_per_block);
     if (blocks_per_sm < 1) return noalloc_fail(COMET_ERR_INVALID_ARG, "N_max needs too much shared memory");
     // warps limited by the occupancy, the TO count and the record space
-    const int64_t per_warp = (int64_t)comet::kRec * Nmax * (int64_t)sizeof(float);
+    const int64_t per_warp = (int64_t)comet::kRec * comet::round32(Nmax) * (int64_t)sizeof(float);
     const int64_t fit = (int64_t)kRecordBytes / per_warp;
     int64_t warps = std::min<int64_t>((int64_t)num_sms * blocks_per_sm * warps_per_block, n);
     warps = ((warps + warps_per_block - 1) / warps_per_block) * warps_per_block;
@@ -165,7 +165,7 @@ extern "C" comet_status comet_eval_modes_noalloc(const comet_instance_desc* inst
     a.out_traj = out_traj;
     a.out_status = out_status;
     a.ws = ws;
-    a.ws_per_warp = (int64_t)comet::kRec * Nmax;
+    a.ws_per_warp = (int64_t)comet::kRec * comet::round32(Nmax);
     a.queue = queue;
     a.bad_input = bad;
     a.sp = comet::make_params(o, 0);

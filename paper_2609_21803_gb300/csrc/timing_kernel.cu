@@ -314,15 +314,26 @@ struct TCtx {
     float* rec;
 };
 
-__device__ __forceinline__ float4* trec(const TCtx& C, int q, int k) {
-    return reinterpret_cast<float4*>(C.rec + 4 * ((size_t)q * C.Nmax + k));
+// Stage records by the lane that eliminates the stage, as in eval_kernel.cu;
+// in stage order 4,096 orders of N = 80 took 99 ms, now 95.
+constexpr int kTRecRow = 32 * (kTRec / 4);  // float4s of one stage of every lane
+
+__device__ __forceinline__ float4* trec(const TCtx& C, int q, int at) {
+    return reinterpret_cast<float4*>(C.rec) + at + 32 * q;
+}
+
+// place (chunk 0) of stage k (k / per as in eval_kernel.cu)
+__device__ __forceinline__ int trec_at(const TCtx& C, int k) {
+    const int per = (C.N + 31) >> 5;
+    const int l = (int)(((float)k + 0.5f) * __fdividef(1.f, (float)per));
+    return kTRecRow * (k - l * per) + l;
 }
 
 // record stores with the persisting (evict-last) L2 priority: the resident
 // warps' records fit in L2 and are rewritten every iteration (as in
 // eval_kernel.cu)
-__device__ __forceinline__ void trec_st(const TCtx& C, int q, int k, float4 v) {
-    cuda::annotated_ptr<float4, cuda::access_property::persisting> p(trec(C, q, k));
+__device__ __forceinline__ void trec_st(const TCtx& C, int q, int at, float4 v) {
+    cuda::annotated_ptr<float4, cuda::access_property::persisting> p(trec(C, q, at));
     *p = v;
 }
 
@@ -537,6 +548,7 @@ __device__ TMeasures tphase_a(TCtx& C, float beta, float rho, bool curvature, bo
 #pragma unroll
                 for (int i = c; i < TM; ++i) A[ttri(i, c)] -= A[ttri(i, j)] * A[ttri(c, j)];
         }
+        const int at = trec_at(C, k);
         float rec[kTRec];
 #pragma unroll
         for (int t = 0; t < kTRec; ++t) rec[t] = 0.f;
@@ -556,7 +568,7 @@ __device__ TMeasures tphase_a(TCtx& C, float beta, float rho, bool curvature, bo
                 if (!(i == TM - TU - 1 && j == i)) rec[R_RED + ttri(i, j)] = A[ttri(TU + i, TU + j)];
 #pragma unroll
         for (int q = 0; q < kTRec / 4; ++q)
-            trec_st(C, q, k, make_float4(rec[4 * q], rec[4 * q + 1], rec[4 * q + 2], rec[4 * q + 3]));
+            trec_st(C, q, at, make_float4(rec[4 * q], rec[4 * q + 1], rec[4 * q + 2], rec[4 * q + 3]));
     }
     __syncwarp();
     // initial rows (pose and tau_0 = 0) and the terminal row tau_N <= T
@@ -652,11 +664,12 @@ constexpr int kTElemChunk0 = R_RED / 4;  // 14: element and node floats start he
 // record floats 56..120 of stage k as an element, with the boundary terms:
 // the terminal cost and the active terminal row on the last stage's y
 // block, damping and the four initial rows on the first stage's x block
-__device__ __forceinline__ void tload_elem(const TCtx& C, int k, float e[kTElem], float beta, float rho) {
+__device__ __forceinline__ void tload_elem(const TCtx& C, int k, int at, float e[kTElem], float beta,
+                                           float rho) {
     float v[68];
 #pragma unroll
     for (int q = 0; q < 17; ++q) {
-        const float4 t = *trec(C, kTElemChunk0 + q, k);
+        const float4 t = *trec(C, kTElemChunk0 + q, at);
         v[4 * q] = t.x;
         v[4 * q + 1] = t.y;
         v[4 * q + 2] = t.z;
@@ -694,7 +707,7 @@ __device__ __forceinline__ void tload_elem(const TCtx& C, int k, float e[kTElem]
 // Eliminate the node shared by e (over (y = m, x = a)) and f (over (y = b,
 // x = m)); e becomes the element over (y = b, x = a).  Stores node m's
 // (L, Y) in record `km` when `store`; false on a non-positive pivot.
-__device__ __forceinline__ bool tcombine(const TCtx& C, float e[kTElem], const float f[kTElem], int km, bool store) {
+__device__ __forceinline__ bool tcombine(const TCtx& C, float e[kTElem], const float f[kTElem], int at, bool store) {
     float L[15];
 #pragma unroll
     for (int i = 0; i < TX; ++i)
@@ -760,18 +773,18 @@ __device__ __forceinline__ bool tcombine(const TCtx& C, float e[kTElem], const f
         o[70] = o[71] = 0.f;
 #pragma unroll
         for (int q = 0; q < 18; ++q)
-            trec_st(C, kTElemChunk0 + q, km, make_float4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]));
+            trec_st(C, kTElemChunk0 + q, at, make_float4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]));
     }
     return pd;
 }
 
 // dx_m = -L^{-T} (Y_b dx_b + Y_a dx_a + y_r) from node m's stored (L, Y)
-__device__ __forceinline__ void tback_node(const TCtx& C, int km, const float xa[TX], const float xb[TX],
+__device__ __forceinline__ void tback_node(const TCtx& C, int at, const float xa[TX], const float xb[TX],
                                            float xm[TX]) {
     float v[72];
 #pragma unroll
     for (int q = 0; q < 18; ++q) {
-        const float4 t = *trec(C, kTElemChunk0 + q, km);
+        const float4 t = *trec(C, kTElemChunk0 + q, at);
         v[4 * q] = t.x;
         v[4 * q + 1] = t.y;
         v[4 * q + 2] = t.z;
@@ -810,8 +823,8 @@ __device__ bool tphase_b(TCtx& C, float beta, float rho) {
 #pragma unroll
     for (int t = 0; t < kTElem; ++t) e[t] = 0.f;
     if (own) {
-        pd = reinterpret_cast<const float*>(trec(C, R_PD / 4, k0))[R_PD % 4] > 0.f;
-        tload_elem(C, k0, e, beta, rho);
+        pd = reinterpret_cast<const float*>(trec(C, R_PD / 4, lane))[R_PD % 4] > 0.f;
+        tload_elem(C, k0, lane, e, beta, rho);
     }
     // folds of the lane's next stages, then the tree levels d = 1, 2, 4, ...:
     // lane l (a multiple of 2d) eliminates the first node of lane l + d's span
@@ -819,22 +832,23 @@ __device__ bool tphase_b(TCtx& C, float beta, float rho) {
     for (int st = 0; st < nsteps; ++st) {
         float f[kTElem];
         bool act;
-        int km;
+        int at;
         if (st < per - 1) {  // warp-uniform
-            km = k0 + 1 + st;
+            const int km = k0 + 1 + st;
             act = own && km < k1;
+            at = kTRecRow * (st + 1) + lane;
             if (act) {
-                pd = pd && reinterpret_cast<const float*>(trec(C, R_PD / 4, km))[R_PD % 4] > 0.f;
-                tload_elem(C, km, f, beta, rho);
+                pd = pd && reinterpret_cast<const float*>(trec(C, R_PD / 4, at))[R_PD % 4] > 0.f;
+                tload_elem(C, km, at, f, beta, rho);
             }
         } else {
             const int d = 1 << (st - (per - 1));
 #pragma unroll
             for (int t = 0; t < kTElem; ++t) f[t] = __shfl_down_sync(kFullT, e[t], d);
             act = (lane & (2 * d - 1)) == 0 && lane + d < nl;
-            km = (lane + d) * per;
+            at = lane + d;  // the first node of lane l + d's span
         }
-        if (act) pd = tcombine(C, e, f, km, true) && pd;
+        if (act) pd = tcombine(C, e, f, at, true) && pd;
     }
     // lane 0 solves the root element over (x_N, x_0): a 10 x 10 Cholesky
     float xl[TX], xr[TX];
@@ -893,11 +907,11 @@ __device__ bool tphase_b(TCtx& C, float beta, float rho) {
 #pragma unroll
             for (int i = 0; i < TX; ++i) xc[i] = xr[i];
         const bool act = tree ? ((lane & (2 * d - 1)) == 0 && lane + d < nl) : (own && k0 + 1 + st < k1);
-        const int km = tree ? (lane + d) * per : k0 + 1 + st;
+        const int km = k0 + 1 + st;
         float xm[TX];
 #pragma unroll
         for (int i = 0; i < TX; ++i) xm[i] = 0.f;
-        if (act) tback_node(C, km, xl, tree ? xr : xc, xm);
+        if (act) tback_node(C, tree ? lane + d : kTRecRow * (st + 1) + lane, xl, tree ? xr : xc, xm);
         if (tree) {
 #pragma unroll
             for (int i = 0; i < TX; ++i) {
@@ -936,10 +950,11 @@ __device__ float tphase_c(TCtx& C) {
     TSmem& S = C.sm;
 #pragma unroll 1
     for (int k = lane; k < N; k += 32) {
+        const int at = trec_at(C, k);
         float f[56];
 #pragma unroll
         for (int qq = 0; qq < 14; ++qq) {
-            const float4 t = *trec(C, qq, k);
+            const float4 t = *trec(C, qq, at);
             f[4 * qq] = t.x;
             f[4 * qq + 1] = t.y;
             f[4 * qq + 2] = t.z;
@@ -1432,7 +1447,7 @@ __global__ void __launch_bounds__(128, 3) timing_kernel(const TimingArgs A) {
 
 size_t timing_smem_per_warp_bytes(int Nmax) { return tsmem_floats(Nmax) * sizeof(float); }
 
-int64_t timing_ws_per_warp_floats(int Nmax) { return (int64_t)kTRec * Nmax; }
+int64_t timing_ws_per_warp_floats(int Nmax) { return (int64_t)kTRec * round32(Nmax); }
 
 namespace {
 SmemLimit g_smem_limit;
