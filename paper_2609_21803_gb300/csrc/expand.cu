@@ -14,6 +14,7 @@
 #include "comet.h"
 #include "comet_internal.h"
 #include "expand_internal.h"
+#include "launch.h"
 
 namespace comet {
 namespace {
@@ -168,6 +169,8 @@ __device__ __forceinline__ TopKey load_key(const TopKey* in_keys, const Frontier
 // pass: 0 reads V, odd passes write top_a and even ones top_b
 __global__ void __launch_bounds__(32 * kRankWarps) topk_rank_kernel(FrontierDev F0, const FrontierDev* Fs, int pass,
                                                                     int chunk, int k) {
+    launch_next();
+    await_previous();
     __shared__ TopKey tile[kRankTile];
     __shared__ int part[kRankWarps][32];
     const FrontierDev F = Fs ? Fs[blockIdx.y] : F0;
@@ -308,6 +311,8 @@ __device__ int neighbour_r(const FrontierDev& F, const uint16_t* s, int L, int j
 constexpr int kNbThreads = 256;
 
 __global__ void __launch_bounds__(kNbThreads) neighbour_kernel(FrontierDev F0, const FrontierDev* Fs, int in_b, int k) {
+    launch_next();
+    await_previous();
     __shared__ uint16_t par[kNbThreads][COMET_MAX_SEGMENTS];
     __shared__ int par_len[kNbThreads];
     const FrontierDev F = Fs ? Fs[blockIdx.y] : F0;
@@ -347,6 +352,8 @@ __global__ void __launch_bounds__(kNbThreads) neighbour_kernel(FrontierDev F0, c
 // Winners (the first proposal of each unseen code) keep their code, the
 // other slots lose it; the winners of each block of kScan slots are counted.
 __global__ void __launch_bounds__(kScan) winner_kernel(FrontierDev F0, const FrontierDev* Fs, int k) {
+    launch_next();
+    await_previous();
     const FrontierDev F = Fs ? Fs[blockIdx.y] : F0;
     const int64_t total = (int64_t)k * F.slots, o = blockIdx.x * (int64_t)kScan + threadIdx.x;
     if (blockIdx.x * (int64_t)kScan >= total) return;
@@ -367,6 +374,8 @@ __global__ void __launch_bounds__(kScan) winner_kernel(FrontierDev F0, const Fro
 // entry of the candidate table.
 __global__ void __launch_bounds__(kScan) compact_kernel(FrontierDev F0, const FrontierDev* Fs, int k, int batch_in,
                                                         int64_t budget) {
+    launch_next();
+    await_previous();
     __shared__ int warp_sums[32];
     const FrontierDev F = Fs ? Fs[blockIdx.y] : F0;
     const int64_t total = (int64_t)k * F.slots;
@@ -470,8 +479,7 @@ cudaError_t topk(const FrontierDev& F, const FrontierDev* d_fs, int n_f, int64_t
         const int64_t chunk = last ? (std::max<int64_t>(n_in, k) + 31) / 32 * 32 : rank_chunk(k);
         const int64_t chunks = last ? 1 : (n_in + chunk - 1) / chunk;
         const dim3 grid((unsigned)(chunks * (chunk / 32)), (unsigned)n_f);
-        topk_rank_kernel<<<grid, 32 * kRankWarps, 0, s>>>(F, d_fs, pass, (int)chunk, k);
-        const cudaError_t e = cudaGetLastError();
+        const cudaError_t e = launch_chained(topk_rank_kernel, grid, 32 * kRankWarps, 0, s, F, d_fs, pass, (int)chunk, k);
         if (e != cudaSuccess) return e;
         *in_b = pass & 1;
         if (last) return cudaSuccess;
@@ -488,12 +496,9 @@ cudaError_t expand(const FrontierDev& F, const FrontierDev* d_fs, int n_f, int64
     if (e != cudaSuccess) return e;
     const dim3 g1((unsigned)std::min<int64_t>((total + kNbThreads - 1) / kNbThreads, 65535), (unsigned)n_f);
     const dim3 g2((unsigned)((total + kScan - 1) / kScan), (unsigned)n_f);
-    neighbour_kernel<<<g1, kNbThreads, 0, s>>>(F, d_fs, in_b ? 1 : 0, k);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    winner_kernel<<<g2, kScan, 0, s>>>(F, d_fs, k);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    compact_kernel<<<g2, kScan, 0, s>>>(F, d_fs, k, batch, budget);
-    return cudaGetLastError();
+    if ((e = launch_chained(neighbour_kernel, g1, kNbThreads, 0, s, F, d_fs, in_b ? 1 : 0, k)) != cudaSuccess) return e;
+    if ((e = launch_chained(winner_kernel, g2, kScan, 0, s, F, d_fs, k)) != cudaSuccess) return e;
+    return launch_chained(compact_kernel, g2, kScan, 0, s, F, d_fs, k, batch, budget);
 }
 
 }  // namespace

@@ -23,6 +23,7 @@
 #include "comet_internal.h"
 #include "comet_proposal.h"
 #include "expand_internal.h"
+#include "launch.h"
 #include "mlp_internal.h"
 #include "problem_internal.h"
 
@@ -212,6 +213,8 @@ __global__ void quantize_kernel(const float* p, int64_t n, LayerTab t) {
 // *d_step (incremented by the loss kernel of the same step)
 __global__ void adamw_kernel(float* p, const float* g, float* m, float* v, int64_t n, LayerTab t,
                              const int64_t* d_step, float lr, float b1, float b2, float eps, float wd) {
+    comet::launch_next();
+    comet::await_previous();
     const float st = (float)(*d_step);
     const float bc1 = 1.f - powf(b1, st), bc2 = 1.f - powf(b2, st);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -237,6 +240,8 @@ __global__ void adamw_kernel(float* p, const float* g, float* m, float* v, int64
 // where X allows it (vec).
 __global__ void features_kernel(const comet_mode_seq* seqs, int64_t n_rows, const int64_t* d_n, const float* fi,
                                 int n_inst, int l_max, int n_modes, int in_dim, uint16_t* X, int bim, int vec) {
+    comet::launch_next();
+    comet::await_previous();
     const int slot_w = bim ? kBimSlot : n_modes + 1;
     const int64_t nn = d_n ? min(*d_n, n_rows) : n_rows;
     const int chunks = in_dim / 8;
@@ -352,6 +357,8 @@ int grid_for(int64_t work, int threads = 256) {
 __global__ void predict_rollout_kernel(const float* Y, int out_dim, const comet_mode_seq* seqs, const int* row_of,
                                        int64_t n_rows, const int64_t* d_n, const comet::DevInstance* inst, int n_inst,
                                        int n_max, float* merit, float* warm, int64_t stride) {
+    comet::launch_next();
+    comet::await_previous();
     const int64_t nn = d_n ? min(*d_n, n_rows) : n_rows;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nn; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t r = row_of ? (int64_t)row_of[i] : i;
@@ -409,6 +416,8 @@ __global__ void predict_rollout_kernel(const float* Y, int out_dim, const comet_
 __global__ void predict_post_kernel(const float* Y, int out_dim, const comet_mode_seq* seqs, const int* row_of,
                                     int64_t n_rows, const int64_t* d_n, const comet::DevInstance* inst, int n_inst,
                                     int n_max, float* merit, float* warm, int64_t stride, int bim) {
+    comet::launch_next();
+    comet::await_previous();
     const int64_t nn = d_n ? min(*d_n, n_rows) : n_rows;
     const int lane = threadIdx.x & 31, nx = bim ? 5 : 4, nc = bim ? 12 : 3, Nm1 = n_max + 1;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -461,13 +470,11 @@ cudaError_t launch_post(const comet_proposal* q, const comet_mode_seq* seqs, con
                         const int64_t* d_n, float* merit, float* warm, cudaStream_t s) {
     if (n < 1) return cudaSuccess;
     if (q->desc.warm_mode == 0 && !q->bim && warm)
-        predict_rollout_kernel<<<grid_for(n, 128), 128, 0, s>>>(q->Y, q->out_dim, seqs, row_of, n, d_n, q->p->d_inst,
-                                                                q->n_inst, q->n_max, merit, warm, q->p->stride);
-    else
-        predict_post_kernel<<<(unsigned)std::min<int64_t>((n + 7) / 8, 65536), 256, 0, s>>>(
-            q->Y, q->out_dim, seqs, row_of, n, d_n, q->p->d_inst, q->n_inst, q->n_max, merit, warm, q->p->stride,
-            q->bim);
-    return cudaGetLastError();
+        return comet::launch_chained(predict_rollout_kernel, grid_for(n, 128), 128, 0, s, q->Y, q->out_dim, seqs, row_of,
+                                     n, d_n, q->p->d_inst, q->n_inst, q->n_max, merit, warm, q->p->stride);
+    return comet::launch_chained(predict_post_kernel, (unsigned)std::min<int64_t>((n + 7) / 8, 65536), 256, 0, s, q->Y,
+                                 q->out_dim, seqs, row_of, n, d_n, q->p->d_inst, q->n_inst, q->n_max, merit, warm,
+                                 q->p->stride, q->bim);
 }
 
 __global__ void encode_kernel(const comet_mode_seq* seqs, int64_t n_rows, const int64_t* d_n, int n_modes,
@@ -513,6 +520,8 @@ __global__ void set_count_kernel(int64_t* n_next, int keep) {
 // two-byte scatter.
 __global__ void __launch_bounds__(256) transpose_kernel(const uint16_t* X, int64_t n, int in_dim, uint16_t* Xt,
                                                         int64_t ld) {
+    comet::launch_next();
+    comet::await_previous();
     __shared__ uint16_t tile[64][66];
     const int64_t b0 = (int64_t)blockIdx.x * 64;
     const int c0 = blockIdx.y * 64;
@@ -686,16 +695,14 @@ cudaError_t backward_update(comet_proposal* q, int64_t M, const comet_adamw_opts
         dw[l] = DwLayer{q->Gt[l], (l > 0) ? q->Ht[l - 1] : q->Xt, q->ld_t, q->dout[l], q->din[l],
                         q->grad + q->w_off[l], q->grad + q->b_off[l]};
     if ((e = dw_bf16(dw, kLayers, M, q->p->num_sms, q->d_err, s)) != cudaSuccess) return e;
-    adamw_kernel<<<grid_for(q->n_params), 256, 0, s>>>(q->master, q->grad, q->m1, q->m2, q->n_params, layer_tab(q),
-                                                       q->d_step, (float)o.lr, (float)o.beta1, (float)o.beta2,
-                                                       (float)o.eps, (float)o.weight_decay);
-    return cudaGetLastError();
+    return comet::launch_chained(adamw_kernel, grid_for(q->n_params), 256, 0, s, q->master, q->grad, q->m1, q->m2,
+                                 q->n_params, layer_tab(q), q->d_step, (float)o.lr, (float)o.beta1, (float)o.beta2,
+                                 (float)o.eps, (float)o.weight_decay);
 }
 
 cudaError_t transpose_x(comet_proposal* q, const uint16_t* x, int64_t n, cudaStream_t s) {
-    transpose_kernel<<<dim3((unsigned)((n + 63) / 64), (unsigned)(q->in_dim / 64)), 256, 0, s>>>(x, n, q->in_dim, q->Xt,
-                                                                                               q->ld_t);
-    return cudaGetLastError();
+    return comet::launch_chained(transpose_kernel, dim3((unsigned)((n + 63) / 64), (unsigned)(q->in_dim / 64)), 256, 0, s,
+                                 x, n, q->in_dim, q->Xt, q->ld_t);
 }
 
 comet_status check_err(comet_proposal* q, cudaStream_t s) {
@@ -783,9 +790,9 @@ comet_problem* proposal_problem(const comet_proposal* q) { return q ? q->p : nul
 comet_status proposal_predict_device(comet_proposal* q, const comet_mode_seq* seqs, int64_t n, float* merit,
                                      float* warm, cudaStream_t s) {
     QTRY(ensure_rows(q, n), "proposal activations");
-    features_kernel<<<grid_for(n * q->in_dim / 8), 256, 0, s>>>(seqs, n, nullptr, q->feat_inst, q->n_inst, q->l_max,
-                                                                q->n_modes, q->in_dim, q->X, q->bim, 1);
-    QTRY(cudaGetLastError(), "features");
+    QTRY(comet::launch_chained(features_kernel, grid_for(n * q->in_dim / 8), 256, 0, s, seqs, n, nullptr, q->feat_inst,
+                               q->n_inst, q->l_max, q->n_modes, q->in_dim, q->X, q->bim, 1),
+         "features");
     QTRY(forward(q, n, nullptr, s), "forward");
     QTRY(launch_post(q, seqs, nullptr, n, nullptr, merit, warm, s), "predict");
     return COMET_OK;

@@ -21,6 +21,7 @@
 // Every mbarrier wait is bounded (about one second of clock cycles); when
 // one runs out the CTA records the failure in the error flag, skips the rest
 // of its work, waits (bounded) for the copies it issued and frees its TMEM.
+#include "launch.h"
 #include "mlp_internal.h"
 
 #include <cuda_bf16.h>
@@ -309,6 +310,8 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap* map_a, const CUtens
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = bars->tmem_base;
+    launch_next();
+    await_previous();
 
     if (warp == 0 && lane == 0) {
         // ---- producer
@@ -613,7 +616,6 @@ __global__ void __launch_bounds__(kFThreads, 1)
     const int n_units = (fp.M + BM - 1) / BM * fp.nsplit;
     const CUtensorMap* wmap[4] = {&map_w0, &map_w1, &map_w2, &map_w3};
 
-    for (int t = threadIdx.x; t < 3 * 256; t += kFThreads) bs[t] = fp.bias[t >> 8][t & 255];
     if (threadIdx.x == 0) {
         mbar_init(smem_u32(&bars->x_full), 1);
         mbar_init(smem_u32(&bars->x_free), 1);
@@ -642,6 +644,10 @@ __global__ void __launch_bounds__(kFThreads, 1)
     tc_fence_after();
     const uint32_t tmem = bars->tmem_base;
     volatile uint32_t* failed = &bars->failed;
+    launch_next();
+    await_previous();
+    for (int t = threadIdx.x; t < 3 * 256; t += kFThreads) bs[t] = fp.bias[t >> 8][t & 255];
+    __syncthreads();
 
     // A unit's steps: the hidden layers 0..2, then its output blocks split,
     // split + nsplit, ...; step number g (over all units) uses accumulator
@@ -950,7 +956,8 @@ cudaError_t gemm_bf16(const Mat& A, const Mat& B, int64_t M, int N, int K, int k
     const int vec = rows_vectorise(ep);
     if (ep.kind == kEpiLoss && (!vec || N % 16)) return cudaErrorInvalidValue;
 #define COMET_GEMM(kind) \
-    gemm_bf16_kernel<kind><<<grid, kThreads, smem_req, s>>>(ma, mb, (int)M, N, K, k_chunk, bn, tmem_cols, vec, ep)
+    e = launch_chained(gemm_bf16_kernel<kind>, grid, kThreads, smem_req, s, ma, mb, (int)M, N, K, k_chunk, bn, \
+                       tmem_cols, vec, ep)
     switch (ep.kind) {
         case kEpiStore: COMET_GEMM(kEpiStore); break;
         case kEpiBiasGelu: COMET_GEMM(kEpiBiasGelu); break;
@@ -960,7 +967,7 @@ cudaError_t gemm_bf16(const Mat& A, const Mat& B, int64_t M, int N, int K, int k
         default: return cudaErrorInvalidValue;
     }
 #undef COMET_GEMM
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t dw_bf16(const DwLayer* layers, int n, int64_t K, int num_sms, int* err, cudaStream_t s) {
@@ -993,8 +1000,7 @@ cudaError_t dw_bf16(const DwLayer* layers, int n, int64_t K, int num_sms, int* e
     const cudaError_t e = gemm_prepare();
     if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)tiles, (unsigned)((K + P.k_chunk - 1) / P.k_chunk));
-    dw_kernel<<<grid, kThreads, smem_request(kMaxBN), s>>>(maps, P);
-    return cudaGetLastError();
+    return launch_chained(dw_kernel, grid, kThreads, smem_request(kMaxBN), s, maps, P);
 }
 
 bool fused_forward_fits(int in_dim, int width, int out_dim) {
@@ -1036,8 +1042,8 @@ cudaError_t mlp_forward_fused(const uint16_t* x, int64_t M, int in_dim, const ui
     fp.nsplit = std::max(1, std::min(n_ob, num_sms / tiles));
     const int units = tiles * fp.nsplit;
     const int grid = units < num_sms ? units : num_sms;
-    mlp_fused_forward_kernel<<<grid, kFThreads, fused_smem_bytes(in_dim), s>>>(mx, mw[0], mw[1], mw[2], mw[3], fp);
-    return cudaGetLastError();
+    return launch_chained(mlp_fused_forward_kernel, grid, kFThreads, fused_smem_bytes(in_dim), s, mx, mw[0], mw[1],
+                          mw[2], mw[3], fp);
 }
 
 cudaError_t fused_prepare() {
