@@ -244,21 +244,24 @@ namespace comet {
 
 // Shape of a pushing launch of n TOs.  A CTA's warps start every trip of the
 // solver together (`in_step`) so that they share instruction fetches, which
-// pays once the SMs are full.  A launch that leaves a quarter of the resident
-// warps idle is bound by its slowest solves instead: there nobody waits for a
-// CTA mate, and long TOs run one to a CTA, which spreads them over all SMs.
-// Measured: 500 TOs at N = 80 7.1 ms one to a CTA, 7.5 four to a CTA out of
-// step, 9.3 in step; 1,400 (9.2 per SM) 11.3 against 12.0 in step; 1,824 (12
-// per SM, the resident limit) 12.6 against 12.4; 4,000 20.4 against 18.6.
-// At N = 16 (one pass of the stage loops) 144 TOs take 2.11 ms four to a
-// CTA and 2.13 one to a CTA.
+// pays once the SMs are full and stay full.  A launch without a queue behind
+// it is bound by its slowest solves instead: there nobody waits for a CTA
+// mate, and while SMs have room, long TOs run one to a CTA, which spreads them
+// over all SMs.  Measured (ms; one to a CTA / four / four in step; N = 80 with
+// 1,824 resident, and mixed orders up to N = 145 with 1,216):
+//   N = 80:  624 TOs  7.2 /  7.3 /  8.8    mixed:  624   8.5 /  9.3 / 11.1
+//          1,400     10.6 / 11.3 / 11.1          1,000  11.5 / 11.4 / 13.1
+//          1,800     12.1 / 11.9 / 12.2          1,400  13.2 / 13.2 / 13.7
+//          2,600     14.5 / 14.9 / 13.7          2,200  16.3 / 15.7 / 15.0
+// and full launches of N = 80 64 / 64 / 54.  At N = 16 (one pass of the stage
+// loops) 144 TOs take 2.0 ms either way.
 struct LaunchShape {
     int wpb, in_step;
 };
 static LaunchShape launch_shape(int num_sms, int blocks_per_sm, int warps_per_block, int Nmax, int64_t n) {
     const int64_t resident = (int64_t)num_sms * blocks_per_sm * warps_per_block;
-    if (4 * n > 3 * resident) return {warps_per_block, 1};
-    return {Nmax > 32 ? 1 : warps_per_block, 0};
+    if (4 * n > 5 * resident) return {warps_per_block, 1};
+    return {Nmax > 32 && 8 * n <= 7 * resident ? 1 : warps_per_block, 0};
 }
 
 static int64_t resident_warps(const comet_problem* p, int64_t n) {

@@ -48,6 +48,7 @@
 
 #include "comet.h"
 #include "comet_internal.h"
+#include "launch.h"
 
 namespace comet {
 namespace {
@@ -1631,8 +1632,7 @@ int bim_blocks_per_sm(int Nmax) {
 
 cudaError_t launch_bimanual(const EvalArgs& a, int n_ctas, cudaStream_t s) {
     const size_t smem = bim_smem_bytes(a.Nmax);
-    bimanual_kernel<<<n_ctas, kBimThreads, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_persistent(bimanual_kernel, n_ctas, kBimThreads, smem, s, a);
 }
 
 }  // namespace comet

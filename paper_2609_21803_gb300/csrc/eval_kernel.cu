@@ -33,6 +33,7 @@
 #include <stdint.h>
 
 #include "comet_internal.h"
+#include "launch.h"
 
 namespace comet {
 namespace {
@@ -1713,22 +1714,12 @@ cudaError_t launch_eval(const EvalArgs& a, int total_warps, int warps_per_block,
     const bool refine = a.sp.refine && a.sp.refine_beta < a.sp.beta_max;
     const bool unr2 = a.unroll == 2 && !refine;
     const unsigned threads = warps_per_block * 32;
-    if (a.sp.free_motion) {
-        if (refine)
-            eval_kernel<true, true, 1><<<blocks, threads, smem, s>>>(a);
-        else if (unr2)
-            eval_kernel<false, true, 2><<<blocks, threads, smem, s>>>(a);
-        else
-            eval_kernel<false, true, 1><<<blocks, threads, smem, s>>>(a);
-    } else {
-        if (refine)
-            eval_kernel<true, false, 1><<<blocks, threads, smem, s>>>(a);
-        else if (unr2)
-            eval_kernel<false, false, 2><<<blocks, threads, smem, s>>>(a);
-        else
-            eval_kernel<false, false, 1><<<blocks, threads, smem, s>>>(a);
-    }
-    return cudaGetLastError();
+    void (*kernel)(EvalArgs) = nullptr;
+    if (a.sp.free_motion)
+        kernel = refine ? eval_kernel<true, true, 1> : unr2 ? eval_kernel<false, true, 2> : eval_kernel<false, true, 1>;
+    else
+        kernel = refine ? eval_kernel<true, false, 1> : unr2 ? eval_kernel<false, false, 2> : eval_kernel<false, false, 1>;
+    return launch_persistent(kernel, blocks, threads, smem, s, a);
 }
 
 }  // namespace comet

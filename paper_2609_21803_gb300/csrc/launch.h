@@ -1,4 +1,5 @@
-// launch.h -- chained kernel launches (programmatic dependent launch).
+// launch.h -- launches with attributes: chains of short kernels (programmatic
+// dependent launch) and the persistent evaluators.
 //
 // A chain of short kernels on one stream pays at every boundary for draining,
 // launching and filling the device.  Chained, a training step of 4,096 samples
@@ -37,6 +38,40 @@ cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t s
     c.attrs = &at;
     c.numAttrs = 1;
     const cudaError_t e = cudaLaunchKernelEx(&c, kernel, std::forward<A>(args)...);
+    if (e != cudaSuccess) cudaGetLastError();  // reported here, not by a later call
+    return e;
+}
+
+// Launch of a persistent evaluator, whose CTAs are all resident: the SM's
+// on-chip memory is split between shared memory and L1 by what this launch
+// puts on an SM, not by what the kernel's occupancy would allow (the default).
+// Stage records come back through L1, and a launch that leaves SMs partly idle
+// is bound by the latency of its slowest solves: 624 mixed pushing orders (N up
+// to 145, a warp per CTA) take 10.3 ms with the default split (28 KB of L1),
+// 8.4 with this one, 150 orders 9.6 and 7.9; full launches keep their split.
+// Shared memory keeps at least 44 % (100 KB), so that another stream's CTAs
+// still fit beside a small launch; without that floor the times are the same.
+template <class K, class A>
+cudaError_t launch_persistent(K kernel, int blocks, unsigned threads, size_t smem, cudaStream_t s, const A& args) {
+    int dev = 0, sms = 0, per_sm = 0, reserved = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
+    if (e != cudaSuccess) return e;
+    const size_t need = (size_t)((blocks + sms - 1) / sms) * (smem + (size_t)reserved);
+    const size_t percent = (100 * need + (size_t)per_sm - 1) / (size_t)per_sm;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    at.val.sharedMemCarveout = (unsigned)(percent < 44 ? 44 : percent > 100 ? 100 : percent);
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3((unsigned)blocks);
+    c.blockDim = dim3(threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    e = cudaLaunchKernelEx(&c, kernel, args);
     if (e != cudaSuccess) cudaGetLastError();  // reported here, not by a later call
     return e;
 }

@@ -12,11 +12,14 @@
 //     accumulator barrier.
 //   * warp 2 allocates and frees the TMEM columns.
 //   * all four warps: epilogue.  Warp w reads TMEM lanes 32w..32w+31 (rows
-//     of the tile) 32 columns at a time with tcgen05.ld, turns each 32 x 32
-//     block around in shared memory and applies the fused epilogue (bias,
-//     GELU, GELU' gating, BF16 conversion, the transposed copy the
-//     weight-gradient GEMM consumes, or split-K atomics) with coalesced
-//     stores.
+//     of the tile) 32 columns at a time with tcgen05.ld and applies the fused
+//     epilogue (bias, GELU, GELU' gating, the loss, BF16 conversion, the
+//     transposed copy the weight-gradient GEMM consumes, or split-K atomics):
+//     aligned rows from registers, a row per lane; ragged blocks and split-K
+//     sums turned around in shared memory, lanes along a row.
+//
+// The kernels are chained (launch.h): the successor may start once the TMEM
+// columns are held, and nothing global is touched before await_previous().
 //
 // Every mbarrier wait is bounded (about one second of clock cycles); when
 // one runs out the CTA records the failure in the error flag, skips the rest

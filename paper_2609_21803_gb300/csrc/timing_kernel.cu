@@ -34,6 +34,7 @@
 #include <stdint.h>
 
 #include "comet_internal.h"
+#include "launch.h"
 
 namespace comet {
 namespace {
@@ -1475,8 +1476,7 @@ cudaError_t launch_timing(const TimingArgs& a, int total_warps, int warps_per_bl
     const cudaError_t e = g_smem_limit.raise(smem, set_smem);
     if (e != cudaSuccess) return e;
     const int blocks = (total_warps + warps_per_block - 1) / warps_per_block;
-    timing_kernel<<<blocks, warps_per_block * 32, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_persistent(timing_kernel, blocks, (unsigned)warps_per_block * 32, smem, s, a);
 }
 
 }  // namespace comet

@@ -57,7 +57,8 @@ def _l(inst, K, L):
 @pytest.mark.parametrize("K,L", [(9, 1), (11, 3), (20, 4)])
 def test_results_do_not_depend_on_the_launch_size(P, timed, K, L):
     # 5 orders alone (a CTA each past N = 32, out of step) and the same ones
-    # tiled to a launch that fills the device (four warps a CTA, in step);
+    # tiled to launches of the resident warps (four a CTA, out of step) and of
+    # one and a half times as many (in step);
     # instances of two segment lengths, so that the longest start first
     insts = [_l(W.push_l4_instance(0), K, L), _l(W.push_l4_instance(1), K + 1, L)]
     rng = np.random.default_rng(3)
@@ -66,13 +67,14 @@ def test_results_do_not_depend_on_the_launch_size(P, timed, K, L):
     prob = P.Problem(insts)
     c = P.comet_get_launch_config(prob.handle)
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    tiles = (sms * c["blocks_per_sm"] * c["warps_per_block"]) // 5 + 3
+    resident = sms * c["blocks_per_sm"] * c["warps_per_block"]
     few = _run(P, prob, _dev(P, seqs, idx), timed, 60)
-    many = _run(P, prob, _dev(P, seqs * tiles, np.tile(idx, tiles)), timed, 60)
+    for tiles in (resident // 5 + 1, resident * 3 // 10 + 1):
+        many = _run(P, prob, _dev(P, seqs * tiles, np.tile(idx, tiles)), timed, 60)
+        for a, b in zip(few, many):
+            b = b.reshape((tiles,) + a.shape)
+            assert (b.view(np.int32) == a.view(np.int32)[None]).all()
     prob.close()
-    for a, b in zip(few, many):
-        b = b.reshape((tiles,) + a.shape)
-        assert (b.view(np.int32) == a.view(np.int32)[None]).all()
 
 
 @pytest.mark.parametrize("task", ["push", "timed", "bimanual"])
