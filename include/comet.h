@@ -210,7 +210,7 @@ comet_status comet_debug_stall_staging(comet_problem* p, int32_t on);
  * loops where an allocation (and the synchronisation cudaMalloc / cudaFree
  * can imply) is not allowed after start-up, or hosts that forbid the CUDA
  * allocator.  No problem object is needed and nothing is allocated or freed:
- * the evaluator's scratch lives in one fixed 32 MiB device array inside the
+ * the evaluator's scratch lives in one fixed 48 MiB device array inside the
  * library, which every device that loads the library holds until the
  * process exits.
  *   inst, n_instances  host descriptors, 1 <= n_instances <= 64 (more is

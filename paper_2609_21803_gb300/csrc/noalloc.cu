@@ -10,7 +10,7 @@
 // comet_eval_modes_noalloc() runs the same evaluator kernel with its scratch
 // in one fixed, file-scope device array instead.
 //
-// The array holds kNoallocScratchBytes (32 MiB) on every device that loads
+// The array holds kNoallocScratchBytes (48 MiB) on every device that loads
 // the library, until the process exits.  Its device address is looked up
 // (cudaGetSymbolAddress, with the device current) on every call: the lookup
 // is cheap, and an address cached across calls would go stale if the caller
@@ -35,7 +35,9 @@
 
 namespace {
 
-constexpr size_t kNoallocScratchBytes = 32u << 20;
+// Records take rows of 32 stages: with 48 MiB every N_max runs at least as many
+// warps as 32 MiB gave when they took N_max stages (N = 80: 1,636, 1,308 then).
+constexpr size_t kNoallocScratchBytes = 48u << 20;
 constexpr int kNoallocMaxInstances = 64;
 
 // scratch layout: [header 256 B: work counter, error flag]
@@ -130,7 +132,7 @@ extern "C" comet_status comet_eval_modes_noalloc(const comet_instance_desc* inst
     warps = std::min<int64_t>(warps, (fit / warps_per_block) * warps_per_block);
     if (warps < warps_per_block)
         return noalloc_fail(COMET_ERR_INVALID_ARG,
-                            "comet_eval_modes_noalloc: N_max too large for the 32 MiB scratch");
+                            "comet_eval_modes_noalloc: N_max too large for the 48 MiB scratch");
 
     cudaStream_t s = (cudaStream_t)cuda_stream;
     unsigned int* queue = reinterpret_cast<unsigned int*>(base);
@@ -169,7 +171,7 @@ extern "C" comet_status comet_eval_modes_noalloc(const comet_instance_desc* inst
     a.queue = queue;
     a.bad_input = bad;
     a.sp = comet::make_params(o, 0);
-    a.in_step = 4 * n > 3 * warps;  // the rule of the problem's launches (api.cu)
+    a.in_step = 4 * n > 5 * warps;  // the rule of the problem's launches (api.cu)
     for (int i = 0; i < n_instances; ++i) a.sp.free_motion |= inst[i].n_modes == 13;
     e = comet::launch_eval(a, (int)warps, warps_per_block, s);
     if (e != cudaSuccess) return noalloc_fail(COMET_ERR_CUDA, cudaGetErrorString(e));

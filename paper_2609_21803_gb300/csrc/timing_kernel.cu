@@ -56,7 +56,7 @@ __host__ __device__ constexpr int tinit_comp(int i) { return i < 3 ? i : 4; }
 // local model order: u 0..3, y = x_{k+1} 4..8, x = x_k 9..13, rhs 14
 constexpr int LU = 0, LY = 4, LX = 9, LR = 14;
 
-// Stage record (kTRec floats, chunk-major float4 chunks as in eval_kernel):
+// Stage record (kTRec floats, float4 chunks laid out as in eval_kernel):
 //   R_UF  0..9    u-block Cholesky factor (lower triangle, 1/l_jj on the diagonal)
 //   R_CP  10..53  coupling columns: local row 4 + c (c = 0..10) x u column j at 10 + 4c + j
 //   R_PD  54      +1 / -1: the u block was positive definite
