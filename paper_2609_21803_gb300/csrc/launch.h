@@ -12,8 +12,10 @@
 // await_previous(), in every thread, before it touches global memory.  The
 // latter returns when the predecessor has completed and its writes are
 // visible; since every kernel of a chain waits so, all earlier ones have
-// completed too.  Behind a kernel that is not part of a chain, a copy or a
-// memset the launch is an ordinary one, and so is whatever follows a chain.
+// completed too.  Its inputs may be written during its own lifetime, so it
+// reads them by ordinary loads, not through the read-only path.  Behind a
+// kernel that is not part of a chain, a copy or a memset the launch is an
+// ordinary one, and so is whatever follows a chain.
 #pragma once
 
 #include <cuda_runtime.h>

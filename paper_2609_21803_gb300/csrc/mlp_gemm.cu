@@ -214,7 +214,7 @@ __device__ __forceinline__ void epilogue_rows(const Epilogue& ep, uint32_t taddr
         const float4* z = reinterpret_cast<const float4*>(ep.bias + nb);
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
-            const float4 t = whole || 4 * q < ncol ? __ldg(z + q) : make_float4(0.f, 0.f, 0.f, 0.f);
+            const float4 t = whole || 4 * q < ncol ? z[q] : make_float4(0.f, 0.f, 0.f, 0.f);
             x[4 * q] = t.x, x[4 * q + 1] = t.y, x[4 * q + 2] = t.z, x[4 * q + 3] = t.w;
         }
     } else {
@@ -806,7 +806,7 @@ __global__ void __launch_bounds__(kFThreads, 1)
                     const bool col_ok = c0 + 4 * j8 < ncol;  // out_dim is a multiple of 16
                     const int64_t col = 256 * (int64_t)b + c0 + 4 * j8;
                     float4 bv = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (col_ok) bv = __ldg(reinterpret_cast<const float4*>(fp.bias[3] + col));
+                    if (col_ok) bv = *reinterpret_cast<const float4*>(fp.bias[3] + col);
                     float v[32];
                     tmem_ld32(tmem + lanes + (g & 1u) * 256 + (uint32_t)c0, v);
                     // 8 lanes turn their 8 x 8 groups of four columns around
