@@ -1117,9 +1117,14 @@ comet_status comet_proposal_train_batch(comet_proposal* q, const uint16_t* x, co
         comet_default_adamw_opts(&o);
     cudaStream_t s = q->p->stream;
     QTRY(ensure_rows(q, n), "proposal activations");
-    // arrays on the device are used in place (the call waits for its work)
-    // unless their alignment forbids 16-byte rows
-    auto in_place = [](const void* v) { return (reinterpret_cast<uintptr_t>(v) & 15u) == 0 && qdev(v); };
+    // arrays on the problem's device are used in place (the call waits for its
+    // work) where 16-byte rows can be read
+    auto in_place = [&](const void* v) {
+        cudaPointerAttributes at;
+        if (cudaPointerGetAttributes(&at, v) == cudaSuccess) return comet::mlp::usable_in_place(at, q->p->device, v);
+        cudaGetLastError();
+        return false;
+    };
     Batch in{x, target, weight};
     if (!in_place(x)) {
         QTRY(to_device(q->X, x, sizeof(uint16_t) * n * q->in_dim, s), "copy x");

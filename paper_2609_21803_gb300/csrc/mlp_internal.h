@@ -57,6 +57,14 @@ struct Mat {
 cudaError_t gemm_bf16(const Mat& A, const Mat& B, int64_t M, int N, int K, int k_splits, const Epilogue& ep,
                       cudaStream_t s);
 
+// Whether kernels on `device` may read the array at v (attributes `at`) where
+// it lies, by 16-byte rows: memory of that device itself.  Another GPU's is
+// not mapped there without peer access, and managed memory migrates; both are
+// copied, as host arrays are.
+inline bool usable_in_place(const cudaPointerAttributes& at, int device, const void* v) {
+    return at.type == cudaMemoryTypeDevice && at.device == device && (reinterpret_cast<uintptr_t>(v) & 15u) == 0;
+}
+
 // Weight and bias gradients of up to kDwMax layers in one launch, added to dw
 // and db: dw = G^T H, db = column sums of G, from the transposed copies
 // g_t [dout][ld] and h_t [din + 1][ld], whose last row holds ones.
