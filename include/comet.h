@@ -202,6 +202,11 @@ comet_status comet_eval_check(comet_problem* p, int32_t* out_flag);
  * left in flight).  Off by default; no production path sets it. */
 comet_status comet_debug_stall_staging(comet_problem* p, int32_t on);
 
+/* Test hook: the shape that a fixed-step launch of n orders on this pushing
+ * problem has: TOs per CTA, and whether a CTA's warps run in step (both
+ * nullable). */
+comet_status comet_debug_launch_shape(comet_problem* p, int64_t n, int32_t* warps_per_block, int32_t* in_step);
+
 /* Solve one mode-conditioned TO per order without allocating any memory.
  * (An addition of this library; the paper has no counterpart.)
  *
@@ -372,7 +377,12 @@ typedef struct {
 comet_status comet_get_launch_config(comet_problem* p, comet_launch_config* out);
 
 /* Set the launch shape (warps_per_block in 1..4, blocks_per_sm in 1..the
- * occupancy limit, unroll 0, 1 or 2; INVALID_ARG otherwise).  Results never
+ * occupancy limit, unroll 0, 1 or 2; INVALID_ARG otherwise).  Launches of any
+ * size then run warps_per_block TOs per CTA.  A problem whose shape was not
+ * set takes it as the shape of launches that fill the SMs: those of at most
+ * 7/8 of the resident warps (SMs x blocks_per_sm x warps_per_block) with N_max
+ * > 32 run one TO per CTA, and those of more than 5/4 of them start every
+ * solver trip of a CTA's TOs together.  Results never
  * depend on warps_per_block and blocks_per_sm: every shape solves each TO in
  * one warp with the same arithmetic.  The unrolled build of the stage loops
  * is the same solver compiled with other multiply-add contractions, so its
@@ -383,9 +393,13 @@ comet_status comet_set_launch_config(comet_problem* p, const comet_launch_config
  * times the evaluator on the n orders of `sample` (host or device) with an
  * iteration budget max_iters (0 = the solver's) under every candidate shape
  * -- 1..4 TOs per CTA, each at its occupancy limit and at three quarters of
- * it, each with the stage loops unrolled 1 and 2 times -- keeps the fastest
- * for p and caches it per (device, N_max) for problems created later in the
- * process.  out (nullable) receives the pick, out_ms (nullable, >= 16
+ * it, each with the stage loops unrolled 1 and 2 times -- and keeps the
+ * fastest for p.  The sample should be as large as the launches to come: if it
+ * exceeds 5/4 of the resident warps of every candidate (1,824 warps at N_max =
+ * 80), the pick is for launches that fill the SMs (smaller ones follow the
+ * rule above) and is cached per (device, N_max) for problems created later in
+ * the process; a smaller sample's pick stays with p, as if it had been set.
+ * out (nullable) receives the pick, out_ms (nullable, >= 16
  * floats) the time of each candidate in order, and n_candidates (nullable)
  * their number.  Synchronises. */
 comet_status comet_autotune(comet_problem* p, const comet_mode_seq* sample, int64_t n, int32_t max_iters,

@@ -125,7 +125,7 @@ assert MODE_SEQ_DTYPE.itemsize == ctypes.sizeof(ModeSeq) == MODE_SEQ_BYTES
 EXPORTS = (
     "comet_default_opts", "comet_problem_create", "comet_problem_destroy", "comet_traj_stride",
     "comet_eval_modes", "comet_eval_modes_budget", "comet_eval_stats", "comet_eval_check",
-    "comet_debug_stall_staging", "comet_mode_code",
+    "comet_debug_stall_staging", "comet_debug_launch_shape", "comet_mode_code",
     "comet_eval_modes_timed",
     "comet_last_error", "comet_eval_modes_noalloc", "comet_fp32_fma_peak", "comet_fp32_fma_peak_threads",
     "comet_frontier_create", "comet_frontier_destroy", "comet_frontier_add", "comet_expand",
@@ -174,6 +174,7 @@ def lib(build_if_missing: bool = False):
             L.comet_eval_stats.argtypes = [vp, vp, vp, vp, vp]
             L.comet_eval_check.argtypes = [vp, vp]
             L.comet_debug_stall_staging.argtypes = [vp, i32]
+            L.comet_debug_launch_shape.argtypes = [vp, i64, ctypes.POINTER(i32), ctypes.POINTER(i32)]
             L.comet_eval_modes_timed.argtypes = [vp, ctypes.POINTER(TimingOpts), vp, i64, vp, i32, vp, vp, vp]
             L.comet_fp32_fma_peak.argtypes = [vp, i32, vp, ctypes.POINTER(ctypes.c_double),
                                               ctypes.POINTER(ctypes.c_double)]
@@ -346,6 +347,13 @@ def comet_eval_check(problem) -> int:
 
 def comet_debug_stall_staging(problem, on: bool):
     _check(lib().comet_debug_stall_staging(problem, int(bool(on))))
+
+
+def comet_debug_launch_shape(problem, n: int) -> tuple[int, bool]:
+    """(TOs per CTA, warps in step) of a fixed-step launch of n orders."""
+    w, s = ctypes.c_int32(), ctypes.c_int32()
+    _check(lib().comet_debug_launch_shape(problem, n, ctypes.byref(w), ctypes.byref(s)))
+    return w.value, bool(s.value)
 
 
 def comet_eval_modes_timed(problem, timing: dict, mode_seqs, n, warm_starts, max_iters, out_cost, out_traj,

@@ -255,13 +255,18 @@ namespace comet {
 //          2,600     14.5 / 14.9 / 13.7          2,200  16.3 / 15.7 / 15.0
 // and full launches of N = 80 64 / 64 / 54.  At N = 16 (one pass of the stage
 // loops) 144 TOs take 2.0 ms either way.
+// A shape that the caller set, or that the autotuner is timing, is launched as
+// it is (`exact`): its CTAs hold warps_per_block TOs at any n.
 struct LaunchShape {
     int wpb, in_step;
 };
-static LaunchShape launch_shape(int num_sms, int blocks_per_sm, int warps_per_block, int Nmax, int64_t n) {
+static LaunchShape launch_shape(int num_sms, int blocks_per_sm, int warps_per_block, bool exact, int Nmax, int64_t n) {
     const int64_t resident = (int64_t)num_sms * blocks_per_sm * warps_per_block;
-    if (4 * n > 5 * resident) return {warps_per_block, 1};
-    return {Nmax > 32 && 8 * n <= 7 * resident ? 1 : warps_per_block, 0};
+    if (4 * n > 5 * resident) return {warps_per_block, warps_per_block > 1};
+    return {!exact && Nmax > 32 && 8 * n <= 7 * resident ? 1 : warps_per_block, 0};
+}
+static LaunchShape launch_shape(const comet_problem* p, int64_t n) {
+    return launch_shape(p->num_sms, p->blocks_per_sm, p->warps_per_block, p->shape_exact, p->Nmax, n);
 }
 
 static int64_t resident_warps(const comet_problem* p, int64_t n) {
@@ -271,7 +276,7 @@ static int64_t resident_warps(const comet_problem* p, int64_t n) {
     // resident warps: every SM filled, never more warps than TOs; the grid is
     // whole CTAs and any warp may pick any TO, so the workspace covers them all
     const int64_t resident = (int64_t)p->num_sms * p->blocks_per_sm * p->warps_per_block;
-    const int wpb = launch_shape(p->num_sms, p->blocks_per_sm, p->warps_per_block, p->Nmax, n).wpb;
+    const int wpb = launch_shape(p, n).wpb;
     return ((std::min<int64_t>(resident, std::max<int64_t>(n, 1)) + wpb - 1) / wpb) * wpb;
 }
 
@@ -356,7 +361,7 @@ comet_status launch_eval_device(comet_problem* p, const comet_mode_seq* d_seqs, 
     if (p->task == COMET_TASK_BIMANUAL) {
         CUDA_TRY(launch_bimanual(a, (int)warps, s), "bimanual evaluator launch");
     } else {
-        const LaunchShape sh = launch_shape(p->num_sms, p->blocks_per_sm, p->warps_per_block, p->Nmax, n_max);
+        const LaunchShape sh = launch_shape(p, n_max);
         a.in_step = sh.in_step;
         CUDA_TRY(launch_eval(a, (int)warps, sh.wpb, s), "evaluator launch");
     }
@@ -612,6 +617,16 @@ comet_status comet_debug_stall_staging(comet_problem* p, int32_t on) {
     return COMET_OK;
 }
 
+comet_status comet_debug_launch_shape(comet_problem* p, int64_t n, int32_t* warps_per_block, int32_t* in_step) {
+    if (!p || n < 0) return fail(COMET_ERR_INVALID_ARG, "bad arguments");
+    if (p->task != COMET_TASK_PUSHER_SLIDER)
+        return fail(COMET_ERR_INVALID_ARG, "the bimanual evaluator runs one CTA per TO; its shape is fixed");
+    const comet::LaunchShape sh = comet::launch_shape(p, n);
+    if (warps_per_block) *warps_per_block = sh.wpb;
+    if (in_step) *in_step = sh.in_step;
+    return COMET_OK;
+}
+
 comet_status comet_eval_modes(comet_problem* p, const comet_mode_seq* seqs, int64_t n, const float* warm,
                               float* out_cost, float* out_traj, int32_t* out_status) {
     return comet_eval_modes_budget(p, seqs, n, warm, 0, out_cost, out_traj, out_status);
@@ -652,7 +667,7 @@ comet_status comet_eval_modes_timed(comet_problem* p, const comet_timing_opts* t
     const int bps = comet::timing_blocks_per_sm(wpb, p->Nmax);
     if (bps < 1) return fail(COMET_ERR_CUDA, "timing kernel: no resident block");
     const int64_t resident = (int64_t)p->num_sms * bps * wpb;
-    const comet::LaunchShape sh = comet::launch_shape(p->num_sms, bps, wpb, p->Nmax, n);  // as for the fixed step
+    const comet::LaunchShape sh = comet::launch_shape(p->num_sms, bps, wpb, false, p->Nmax, n);  // as for the fixed step
     wpb = sh.wpb;
     const int64_t warps = ((std::min<int64_t>(resident, n) + wpb - 1) / wpb) * wpb;
     const int64_t ws_floats = comet::timing_ws_per_warp_floats(p->Nmax) * warps;

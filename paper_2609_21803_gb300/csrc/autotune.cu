@@ -2,8 +2,12 @@
 // warp per TO, 1..4), resident CTAs per SM and the unrolling of the stage
 // loops (1 or 2 stages per trip).  comet_autotune times the evaluator on a
 // sample of the caller's orders under every candidate shape and keeps the
-// fastest; the pick is cached per (device, N_max) for the process, and
-// problems created later with the same key start from it.
+// fastest.  A pick timed on more than 5/4 of the resident warps of every
+// candidate holds for launches that fill the SMs, whose CTAs run in step (see
+// launch_shape in api.cu): it is cached per (device, N_max) for the process,
+// and problems created later with the same key start from it.  A pick timed on
+// fewer orders says nothing about those: it stays with its problem, whose
+// launches then run it at every size.
 //
 // Every (TOs per CTA, CTAs per SM) shape solves each TO in one warp with the
 // same arithmetic, so the results do not depend on it, only the time does;
@@ -91,6 +95,7 @@ comet_status comet_set_launch_config(comet_problem* p, const comet_launch_config
     p->warps_per_block = c->warps_per_block;
     p->blocks_per_sm = c->blocks_per_sm;
     p->unroll = c->unroll == 2 ? 2 : 1;
+    p->shape_exact = true;
     return COMET_OK;
 }
 
@@ -136,6 +141,10 @@ comet_status comet_autotune(comet_problem* p, const comet_mode_seq* sample, int6
     if (e == cudaSuccess) e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
     const int w0 = p->warps_per_block, b0 = p->blocks_per_sm, u0 = p->unroll;
+    const bool x0 = p->shape_exact;
+    p->shape_exact = true;  // time each candidate as it is
+    bool full = true;
+    for (const Shape& c : cand) full = full && 4 * n > 5 * (int64_t)p->num_sms * c.bps * c.wpb;
     float best_ms = 0.f;
     int best = -1;
     comet_status st = COMET_OK;
@@ -170,13 +179,15 @@ comet_status comet_autotune(comet_problem* p, const comet_mode_seq* sample, int6
         p->warps_per_block = w0;
         p->blocks_per_sm = b0;
         p->unroll = u0;
+        p->shape_exact = x0;
         if (st != COMET_OK) return st;
         return tcuda(e, "autotune");
     }
     p->warps_per_block = cand[best].wpb;
     p->blocks_per_sm = cand[best].bps;
     p->unroll = cand[best].unroll;
-    {
+    p->shape_exact = !full;
+    if (full) {
         std::lock_guard<std::mutex> lk(g_mu);
         g_cache[{p->device, p->Nmax}] = cand[best];
     }

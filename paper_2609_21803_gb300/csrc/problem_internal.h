@@ -22,6 +22,7 @@ struct comet_problem {
     int num_sms = 0;
     int warps_per_block = 4;
     int blocks_per_sm = 0;
+    bool shape_exact = false;  // launches of any size run warps_per_block TOs per CTA (api.cu)
     int unroll = 1;  // stages per trip of the evaluator's stage loops
     int stall_staging = 0;  // test hook of comet_debug_stall_staging
     float* d_ws = nullptr;
