@@ -94,7 +94,8 @@ void set_error(const char* msg);
 // A kernel's shared-memory limit on each device, only ever raised: problems of
 // several sizes are alive at once, and creating a small one (which asks for the
 // occupancy at its own size) must not take a larger one's launches away.
-// `set(bytes)` sets the attribute on the current device.
+// `set(bytes)` sets the attribute on the current device.  What was set stays:
+// the runtime keeps a function's limit over a device reset.
 class SmemLimit {
     std::mutex m_;
     size_t at_[64] = {};
