@@ -5,8 +5,8 @@
 // warm-start the orders of an expansion round (Algorithm 1).
 //
 // Every GEMM runs on the hand-written tcgen05 kernel (mlp_gemm.cu) with a
-// fused epilogue; the element-wise parts (features, targets, loss gradient,
-// bias gradients, AdamW, mini-batch gather, warm-start rollout) are plain
+// fused epilogue, the loss and its gradient among them; the element-wise parts
+// (features, targets, AdamW, mini-batch gather, warm-start rollout) are plain
 // CUDA kernels.  A training step is captured once as a CUDA graph and
 // replayed; its step counter lives in device memory.
 
@@ -51,6 +51,7 @@ struct comet_proposal {
     int din[kLayers], dout[kLayers];
     float* master = nullptr;  // [n_params]
     float* grad = nullptr;
+    float* grad_block = nullptr;  // the splits' bias gradients, grad, the loss, the error flag
     float* m1 = nullptr;
     float* m2 = nullptr;
     uint16_t* wq[kLayers] = {};   // bf16 W_l [dout][din]
@@ -209,24 +210,53 @@ __global__ void quantize_kernel(const float* p, int64_t n, LayerTab t) {
     }
 }
 
+// place of bias i of the flat vector among all biases
+__device__ __forceinline__ int bias_of(const LayerTab& t, int64_t i) {
+    int at = 0;
+#pragma unroll
+    for (int j = 0; j < kLayers; ++j) {
+        const int64_t o = i - t.b_off[j];
+        if (o >= 0 && o < t.dout[j]) return at + (int)o;
+        at += t.dout[j];
+    }
+    return 0;
+}
+
 // AdamW with bias-corrected moments and decoupled weight decay at step t =
-// *d_step (incremented by the loss kernel of the same step)
-__global__ void adamw_kernel(float* p, const float* g, float* m, float* v, int64_t n, LayerTab t,
-                             const int64_t* d_step, float lr, float b1, float b2, float eps, float wd) {
+// *d_step (incremented by the last GEMM of the same step's forward pass).  A
+// bias gradient is the sum of its splits' parts [splits][ld_parts], taken here
+// in their order and left in g.
+__global__ void adamw_kernel(float* p, float* g, const float* parts, int splits, int ld_parts, float* m, float* v,
+                             int64_t n, LayerTab t, const int64_t* d_step, float lr, float b1, float b2, float eps,
+                             float wd) {
     comet::launch_next();
     comet::await_previous();
     const float st = (float)(*d_step);
     const float bc1 = 1.f - powf(b1, st), bc2 = 1.f - powf(b2, st);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float gi = g[i];
-        const float mi = b1 * m[i] + (1.f - b1) * gi;
-        const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
+        float gi = g[i];
+        const float m0 = m[i], v0 = v[i], p0 = p[i];
+        int l, r, c;
+        const bool weight = weight_of(t, i, l, r, c);
+        if (!weight) {
+            const float* part = parts + bias_of(t, i);
+            gi = 0.f;
+            for (int k = 0; k < splits; k += 16) {  // 16 loads in flight
+                float x[16];
+#pragma unroll
+                for (int j = 0; j < 16; ++j) x[j] = k + j < splits ? part[(int64_t)(k + j) * ld_parts] : 0.f;
+#pragma unroll
+                for (int j = 0; j < 16; ++j) gi += x[j];
+            }
+            g[i] = gi;
+        }
+        const float mi = b1 * m0 + (1.f - b1) * gi;
+        const float vi = b2 * v0 + (1.f - b2) * gi * gi;
         m[i] = mi;
         v[i] = vi;
-        const float pi = p[i] - lr * ((mi / bc1) / (sqrtf(vi / bc2) + eps) + wd * p[i]);
+        const float pi = p0 - lr * ((mi / bc1) / (sqrtf(vi / bc2) + eps) + wd * p0);
         p[i] = pi;
-        int l, r, c;
-        if (weight_of(t, i, l, r, c)) {
+        if (weight) {
             const uint16_t b = bf16_bits(pi);
             t.wq[l][(int64_t)r * t.din[l] + c] = b;
             t.wqt[l][(int64_t)c * t.dout[l] + r] = b;
@@ -609,9 +639,36 @@ struct Batch {
     const float *target, *weight;
 };
 
-// gradients and the loss of a step start at zero (one block, see create)
-cudaError_t zero_step(comet_proposal* q, cudaStream_t s) {
-    return cudaMemsetAsync(q->grad, 0, sizeof(float) * (q->n_params + 1), s);
+int bias_count(const comet_proposal* q) {
+    int n = 0;
+    for (int l = 0; l < kLayers; ++l) n += q->dout[l];
+    return n;
+}
+
+// The weight gradients of a step of M rows, its splits and where their bias
+// gradients begin (they end where grad begins)
+struct StepGrads {
+    comet::mlp::DwLayer dw[kLayers];
+    int splits;
+    float* parts;
+};
+StepGrads step_grads(const comet_proposal* q, int64_t M) {
+    StepGrads g;
+    for (int l = 0; l < kLayers; ++l)
+        g.dw[l] = {q->Gt[l], (l > 0) ? q->Ht[l - 1] : q->Xt, q->ld_t, q->dout[l], q->din[l], q->grad + q->w_off[l],
+                   nullptr};
+    g.splits = comet::mlp::dw_splits(g.dw, kLayers, M, q->p->num_sms);
+    g.parts = q->grad - (int64_t)g.splits * bias_count(q);
+    float* db = g.parts;
+    for (int l = 0; l < kLayers; db += q->dout[l++]) g.dw[l].db = db;
+    return g;
+}
+
+// gradients and the loss of a step of M rows start at zero (one block, see
+// create); `err` clears the error flag too
+cudaError_t zero_step(comet_proposal* q, int64_t M, bool err, cudaStream_t s) {
+    float* from = step_grads(q, M).parts;
+    return cudaMemsetAsync(from, 0, sizeof(float) * (q->grad - from + q->n_params + (err ? 2 : 1)), s);
 }
 
 // Forward pass of M rows: inference from q->X into q->Y, or of a training
@@ -690,14 +747,12 @@ cudaError_t backward_update(comet_proposal* q, int64_t M, const comet_adamw_opts
     }
     // every dW_l = G_l^T H_{l-1} and db_l in one launch, from the transposed
     // copies (four weight-gradient launches and four bias reductions before)
-    DwLayer dw[kLayers];
-    for (int l = 0; l < kLayers; ++l)
-        dw[l] = DwLayer{q->Gt[l], (l > 0) ? q->Ht[l - 1] : q->Xt, q->ld_t, q->dout[l], q->din[l],
-                        q->grad + q->w_off[l], q->grad + q->b_off[l]};
-    if ((e = dw_bf16(dw, kLayers, M, q->p->num_sms, q->d_err, s)) != cudaSuccess) return e;
-    return comet::launch_chained(adamw_kernel, grid_for(q->n_params), 256, 0, s, q->master, q->grad, q->m1, q->m2,
-                                 q->n_params, layer_tab(q), q->d_step, (float)o.lr, (float)o.beta1, (float)o.beta2,
-                                 (float)o.eps, (float)o.weight_decay);
+    const StepGrads g = step_grads(q, M);
+    const int biases = bias_count(q);
+    if ((e = dw_bf16(g.dw, kLayers, M, biases, q->p->num_sms, q->d_err, s)) != cudaSuccess) return e;
+    return comet::launch_chained(adamw_kernel, grid_for(q->n_params), 256, 0, s, q->master, q->grad, g.parts, g.splits,
+                                 biases, q->m1, q->m2, q->n_params, layer_tab(q), q->d_step, (float)o.lr,
+                                 (float)o.beta1, (float)o.beta2, (float)o.eps, (float)o.weight_decay);
 }
 
 cudaError_t transpose_x(comet_proposal* q, const uint16_t* x, int64_t n, cudaStream_t s) {
@@ -874,15 +929,18 @@ comet_status comet_proposal_create(comet_problem* p, const comet_proposal_desc* 
         comet_proposal_destroy(q);
         return st;
     };
+    const int64_t parts = comet::mlp::dw_parts_max(bias_count(q), p->num_sms);
     cudaError_t e = cudaSuccess;
     cudaStream_t s = p->stream;
-    if ((e = qalloc(q, &q->master, off)) != cudaSuccess || (e = qalloc(q, &q->grad, off + 2)) != cudaSuccess ||
+    if ((e = qalloc(q, &q->master, off)) != cudaSuccess ||
+        (e = qalloc(q, &q->grad_block, parts + off + 2)) != cudaSuccess ||
         (e = qalloc(q, &q->m1, off)) != cudaSuccess || (e = qalloc(q, &q->m2, off)) != cudaSuccess ||
         (e = qalloc(q, &q->feat_inst, (size_t)q->n_inst * kInstFeat)) != cudaSuccess ||
         (e = qalloc(q, &q->d_step, 1)) != cudaSuccess)
         return cleanup(qcuda(e, "proposal allocation"));
-    // the loss and the error flag lie behind the gradients, cleared and read
-    // back together
+    // the splits' bias gradients lie before the gradients, the loss and the
+    // error flag behind them: cleared and read back together
+    q->grad = q->grad_block + parts;
     q->d_loss = q->grad + off;
     q->d_err = reinterpret_cast<int*>(q->grad + off + 1);
     for (int l = 0; l < kLayers; ++l)
@@ -931,7 +989,7 @@ comet_status comet_proposal_create(comet_problem* p, const comet_proposal_desc* 
     if ((e = cudaGetLastError()) != cudaSuccess) return cleanup(qcuda(e, "proposal init"));
     cudaMemsetAsync(q->m1, 0, sizeof(float) * off, s);
     cudaMemsetAsync(q->m2, 0, sizeof(float) * off, s);
-    cudaMemsetAsync(q->grad, 0, sizeof(float) * (off + 2), s);
+    cudaMemsetAsync(q->grad_block, 0, sizeof(float) * (parts + off + 2), s);
     cudaMemsetAsync(q->d_step, 0, sizeof(int64_t), s);
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cleanup(qcuda(e, "proposal init"));
     *out = q;
@@ -1138,7 +1196,7 @@ comet_status comet_proposal_train_batch(comet_proposal* q, const uint16_t* x, co
         QTRY(to_device(q->Om, weight, sizeof(float) * n * q->out_dim, s), "copy weight");
         in.weight = q->Om;
     }
-    QTRY(cudaMemsetAsync(q->grad, 0, sizeof(float) * (q->n_params + 2), s), "reset");
+    QTRY(zero_step(q, n, true, s), "reset");
     // X^T for the first layer's weight gradient
     QTRY(transpose_x(q, in.x, n, s), "transpose");
     QTRY(forward(q, n, &in, s), "forward");
@@ -1260,7 +1318,7 @@ comet_status comet_proposal_train(comet_proposal* q, int64_t steps, int32_t batc
     if (e == cudaSuccess) e = cudaMemsetAsync(q->d_err, 0, sizeof(int), s);
     if (e == cudaSuccess) e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        cudaError_t ce = zero_step(q, s);
+        cudaError_t ce = zero_step(q, batch, false, s);
         if (ce == cudaSuccess) {
             gather_kernel<<<grid_for((int64_t)batch * 32), 256, 0, s>>>(q->ds_X, q->ds_T, q->ds_Om, q->ds_n, batch,
                                                                        q->d_step, (unsigned long long)seed, q->in_dim,

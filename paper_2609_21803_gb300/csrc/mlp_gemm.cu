@@ -408,7 +408,9 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap* map_a, const CUtens
                     if (ok) ep.out_f32[(int64_t)row * ep.ld_out + col] = a + bias;
                 } else if (KIND == kEpiAtomicAdd) {
                     // the last column of a weight gradient with a row of ones
-                    // under its second operand is the bias gradient
+                    // under its second operand is the split's bias gradient,
+                    // the only sum that its zeroed place gets (a branch to a
+                    // plain store costs the launch 1.5 us)
                     if (ok)
                         atomicAdd(ep.bias_grad && col == N - 1 ? ep.bias_grad + row
                                                                : ep.out_f32 + (int64_t)row * ep.ld_out + col,
@@ -475,6 +477,7 @@ struct DwParams {
     int n, K, k_chunk, first[kDwMax + 1], M[kDwMax], N[kDwMax], cols[kDwMax];
     float* dw[kDwMax];
     float* db[kDwMax];
+    int64_t ld_db;
     int* err;
 };
 
@@ -487,7 +490,7 @@ __global__ void __launch_bounds__(kThreads, 1) dw_kernel(const __grid_constant__
     ep.kind = kEpiAtomicAdd;
     ep.out_f32 = P.dw[l];
     ep.ld_out = P.N[l] - 1;
-    ep.bias_grad = P.db[l];
+    ep.bias_grad = P.db[l] + blockIdx.y * P.ld_db;
     ep.err = P.err;
     gemm_tile<kEpiAtomicAdd>(&maps.a[l], &maps.b[l],
                              Tile{P.M[l], P.N[l], t / P.cols[l] * BM, t % P.cols[l] * kMaxBN, k_begin,
@@ -973,13 +976,35 @@ cudaError_t gemm_bf16(const Mat& A, const Mat& B, int64_t M, int N, int K, int k
     return e;
 }
 
-cudaError_t dw_bf16(const DwLayer* layers, int n, int64_t K, int num_sms, int* err, cudaStream_t s) {
+// tiles of a layer's gradient with its bias column: rows x columns
+static int dw_cols(const DwLayer& L) { return (L.din + kMaxBN) / kMaxBN; }
+static int dw_tiles(const DwLayer& L) { return (L.dout + BM - 1) / BM * dw_cols(L); }
+
+// rows of a split: one wave of two CTAs per SM, at least 256 rows each
+static int dw_chunk(const DwLayer* layers, int n, int64_t K, int num_sms) {
+    int tiles = 0;
+    for (int l = 0; l < n; ++l) tiles += dw_tiles(layers[l]);
+    const int64_t splits = std::max<int64_t>(1, std::min<int64_t>(2 * num_sms / tiles, K / 256));
+    return (int)(((K + splits - 1) / splits + BK - 1) / BK * BK);
+}
+
+int dw_splits(const DwLayer* layers, int n, int64_t K, int num_sms) {
+    const int chunk = dw_chunk(layers, n, K, num_sms);
+    return (int)((K + chunk - 1) / chunk);
+}
+
+// splits <= max(1, 2 num_sms / tiles) (whole chunks cover K with no more), and
+// a tile has at most BM of the outputs
+int64_t dw_parts_max(int64_t sum_dout, int num_sms) { return std::max<int64_t>(sum_dout, 2 * (int64_t)num_sms * BM); }
+
+cudaError_t dw_bf16(const DwLayer* layers, int n, int64_t K, int64_t ld_db, int num_sms, int* err, cudaStream_t s) {
     if (n < 1 || n > kDwMax || K < 1 || K > (int64_t)INT32_MAX) return cudaErrorInvalidValue;
     DwMaps maps;
     DwParams P;
     memset(&P, 0, sizeof(P));
     P.n = n;
     P.K = (int)K;
+    P.ld_db = ld_db;
     P.err = err;
     for (int l = 0; l < n; ++l) {
         const DwLayer& L = layers[l];
@@ -991,18 +1016,15 @@ cudaError_t dw_bf16(const DwLayer* layers, int n, int64_t K, int num_sms, int* e
             return cudaErrorInvalidValue;
         P.M[l] = L.dout;
         P.N[l] = L.din + 1;
-        P.cols[l] = (L.din + kMaxBN) / kMaxBN;
+        P.cols[l] = dw_cols(L);
         P.dw[l] = L.dw;
         P.db[l] = L.db;
-        P.first[l + 1] = P.first[l] + (L.dout + BM - 1) / BM * P.cols[l];
+        P.first[l + 1] = P.first[l] + dw_tiles(L);
     }
-    // splits of the batch: one wave of two CTAs per SM, at least 256 rows each
-    const int tiles = P.first[n];
-    const int64_t splits = std::max<int64_t>(1, std::min<int64_t>(2 * num_sms / tiles, K / 256));
-    P.k_chunk = (int)(((K + splits - 1) / splits + BK - 1) / BK * BK);
+    P.k_chunk = dw_chunk(layers, n, K, num_sms);
     const cudaError_t e = gemm_prepare();
     if (e != cudaSuccess) return e;
-    const dim3 grid((unsigned)tiles, (unsigned)((K + P.k_chunk - 1) / P.k_chunk));
+    const dim3 grid((unsigned)P.first[n], (unsigned)dw_splits(layers, n, K, num_sms));
     return launch_chained(dw_kernel, grid, kThreads, smem_request(kMaxBN), s, maps, P);
 }
 

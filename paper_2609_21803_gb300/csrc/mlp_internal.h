@@ -66,8 +66,13 @@ inline bool usable_in_place(const cudaPointerAttributes& at, int device, const v
 }
 
 // Weight and bias gradients of up to kDwMax layers in one launch, added to dw
-// and db: dw = G^T H, db = column sums of G, from the transposed copies
-// g_t [dout][ld] and h_t [din + 1][ld], whose last row holds ones.
+// and db: dw = G^T H, db = column sums of G, from the transposed copies g_t
+// [dout][ld] and h_t [din + 1][ld], whose last row holds ones.  The batch is
+// split; split s has places of its own for its bias sums, db + s ld_db, and
+// the reader adds the splits up in order, so that a bias gradient does not
+// depend on which CTA ends first (a weight's does: its splits are atomic sums).
+// dw_splits() is the number of splits of K rows, and splits x the sum of dout
+// stays within dw_parts_max().
 constexpr int kDwMax = 4;
 struct DwLayer {
     const uint16_t* g_t;
@@ -77,7 +82,9 @@ struct DwLayer {
     float* dw;
     float* db;
 };
-cudaError_t dw_bf16(const DwLayer* layers, int n, int64_t K, int num_sms, int* err, cudaStream_t s);
+int dw_splits(const DwLayer* layers, int n, int64_t K, int num_sms);
+int64_t dw_parts_max(int64_t sum_dout, int num_sms);
+cudaError_t dw_bf16(const DwLayer* layers, int n, int64_t K, int64_t ld_db, int num_sms, int* err, cudaStream_t s);
 
 // The tensor-map encoder from the driver (resolved once); false if absent.
 bool tensor_maps_available();
