@@ -140,80 +140,114 @@ __global__ void add_many_kernel(const FrontierDev* Fs, const comet_mode_seq* seq
 }
 
 // ---------------------------------------------------------------- top-k
-// The k smallest keys of each chunk of the input, in order, by counting: a
-// key's place is the number of smaller keys in its chunk.  A CTA places 32
-// keys (a lane each); its 8 warps share the chunk, an eighth of each tile
-// each, read as shared-memory broadcasts.  Keys are unique in practice; equal
-// ones (the padding of an earlier pass) keep their input order.
+// The k smallest keys of V, in order.  Pass 0 ranks every run of kRun keys by
+// counting: a key's place is the number of smaller keys in its run (read as
+// shared-memory broadcasts), and the first min(k, kRun) stay.  Each later pass
+// merges kMerge sorted runs: a key's place is its own plus, by binary search,
+// the number of smaller keys in each of the others; the first k stay.  Keys
+// are unique in practice; equal ones keep their input order.
 //
-// Counting does n^2 compares where a sort does n log^2 n, but without its 78
-// barriers, and spread over all SMs: a 4,096-key bitonic sort in one CTA took
-// about 80 us of every round, counting the 3,000 keys of a set of at most 7,096 takes 17 us.
-// Chunks bound the square: the first pass of a large set runs on chunks of
-// max(4096, 4 k) keys, each leaving k.
+// Counting needs no barriers and spreads over all SMs, but costs n times the
+// run; searching costs n log(run).  So runs are short and the rest is merged.
+// Before, every pass counted in chunks of max(4096, 4 k) keys, in one chunk up
+// to 16,384; before that, chunks of 4,096 were sorted in a CTA each (78
+// barriers, 80 us however small the set).  A comet_frontier_best call, which
+// copies k keys back and waits (us: sorted chunks / counted chunks / now):
+//      n = 8,000  k = 64     249 /   65 /  46    k = 2,048   254 /   67 /  60
+//         20,736             249 /   69 /  55                480 /  127 /  83
+//        105,000             251 /  164 /  69                699 /  403 / 109
+//        420,000             357 /  537 / 108                921 / 1329 / 222
+//      1,048,576             454 / 1321 / 193               1131 / 3173 / 438
+struct Runs {
+    int64_t n;      // sorted runs, one after the other
+    int len, tail;  // length of every run but the last, and of the last
+};
 
-constexpr int kRankWarps = 8, kRankTile = 1024;
-
-// chunk of a pass that is not the last
-__host__ __device__ inline int rank_chunk(int k) { return ((4 * k > kChunk ? 4 * k : kChunk) + 31) / 32 * 32; }
-
-__device__ __forceinline__ TopKey load_key(const TopKey* in_keys, const FrontierDev& F, int64_t i) {
-    if (in_keys) return in_keys[i];
-    TopKey key;
-    key.mk = float_key(F.merit[i]);
-    key.idx = (uint32_t)i;
-    key.code = F.codes[i];
-    return key;
+// the runs that pass `pass` >= 1 finds
+__device__ Runs runs_at(int64_t n_keys, int pass, int k) {
+    Runs R;
+    R.n = (n_keys + kRun - 1) / kRun;
+    R.len = min(k, kRun);
+    R.tail = (int)min((int64_t)k, n_keys - (R.n - 1) * kRun);
+    for (int p = 1; p < pass; ++p) {
+        const int64_t m = (R.n + kMerge - 1) / kMerge;
+        const int64_t last = (R.n - (m - 1) * kMerge - 1) * R.len + R.tail;
+        R.n = m;
+        R.len = min(k, kMerge * R.len);
+        R.tail = (int)min((int64_t)k, last);
+    }
+    return R;
 }
 
-// pass: 0 reads V, odd passes write top_a and even ones top_b
-__global__ void __launch_bounds__(32 * kRankWarps) topk_rank_kernel(FrontierDev F0, const FrontierDev* Fs, int pass,
-                                                                    int chunk, int k) {
+// whether o comes before me; `ties`: also if they are equal (no branches)
+__device__ __forceinline__ bool key_before(const TopKey& o, const TopKey& me, bool ties) {
+    return (o.mk < me.mk) | ((o.mk == me.mk) & ((o.code < me.code) | (ties & (o.code == me.code))));
+}
+
+// |V| may have run past the capacity (flagged on add): never read beyond it
+__device__ __forceinline__ int64_t keys_of(const FrontierDev& F) {
+    return (int64_t)min(*F.nV, (unsigned long long)F.capacity);
+}
+
+__global__ void __launch_bounds__(kRun) topk_rank_kernel(FrontierDev F0, const FrontierDev* Fs, int k) {
     launch_next();
     await_previous();
-    __shared__ TopKey tile[kRankTile];
-    __shared__ int part[kRankWarps][32];
+    __shared__ TopKey run[kRun];
     const FrontierDev F = Fs ? Fs[blockIdx.y] : F0;
-    const TopKey* in_keys = pass == 0 ? nullptr : (pass & 1) ? F.top_a : F.top_b;
-    TopKey* out = (pass & 1) ? F.top_b : F.top_a;
-    // |V| may have run past the capacity (flagged on add): never read beyond it
-    int64_t n_max = F.capacity;  // keys that this pass can hold
-    for (int q = 0; q < pass; ++q) n_max = (n_max + rank_chunk(k) - 1) / rank_chunk(k) * k;
-    const int64_t n_in = pass == 0 ? min((int64_t)*F.nV, F.capacity) : n_max;
-    const int per = chunk / 32;  // CTAs of a chunk
-    const int c = blockIdx.x / per, i0 = (blockIdx.x - c * per) * 32;
-    const int64_t base = (int64_t)c * chunk;
-    if (c > 0 && base >= n_max) return;  // a smaller frontier than the launch's largest
-    const int len = (int)max((int64_t)0, min((int64_t)chunk, n_in - base));
-    if (i0 >= len && i0 >= k) return;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int i = i0 + lane;
+    const int64_t base = (int64_t)blockIdx.x * kRun;
+    const int len = (int)min((int64_t)kRun, keys_of(F) - base), i = threadIdx.x;
+    if (len <= 0) return;
     TopKey me;
-    me.mk = 0xffffffffu;
-    me.idx = 0xffffffffu;
-    me.code = ~0ull;
-    if (i < len) me = load_key(in_keys, F, base + i);
-    int rank = 0;
-    for (int t0 = 0; t0 < len; t0 += kRankTile) {
-        const int tn = min(kRankTile, len - t0);
-        __syncthreads();
-        for (int t = threadIdx.x; t < tn; t += blockDim.x) tile[t] = load_key(in_keys, F, base + t0 + t);
-        __syncthreads();
-        const int j1 = min(tn, (warp + 1) * (kRankTile / kRankWarps));
-#pragma unroll 4
-        for (int j = warp * (kRankTile / kRankWarps); j < j1; ++j) {
-            const TopKey o = tile[j];
-            rank += o.mk < me.mk;
-            if (o.mk == me.mk) rank += o.code < me.code || (o.code == me.code && t0 + j < i);
-        }
+    if (i < len) {
+        me.mk = float_key(F.merit[base + i]);
+        me.idx = (uint32_t)(base + i);
+        me.code = F.codes[base + i];
+        run[i] = me;
     }
-    part[warp][lane] = rank;
     __syncthreads();
-    if (warp == 0) {
-        for (int w = 1; w < kRankWarps; ++w) rank += part[w][lane];
-        if (i >= len) rank = i;  // padding after the chunk's keys
-        if (rank < k && i < chunk) out[(int64_t)c * k + rank] = me;
+    if (i >= len) return;
+    int rank = 0;
+#pragma unroll 4
+    for (int j = 0; j < len; ++j) rank += key_before(run[j], me, j < i);
+    if (rank < k) F.top_a[blockIdx.x * (int64_t)min(k, kRun) + rank] = me;
+}
+
+// pass 1 reads top_a and writes top_b, pass 2 the other way round, ...
+__global__ void __launch_bounds__(256) topk_merge_kernel(FrontierDev F0, const FrontierDev* Fs, int pass, int k) {
+    launch_next();
+    await_previous();
+    const FrontierDev F = Fs ? Fs[blockIdx.y] : F0;
+    const TopKey* in = (pass & 1) ? F.top_a : F.top_b;
+    TopKey* out = (pass & 1) ? F.top_b : F.top_a;
+    const Runs R = runs_at(keys_of(F), pass, k);
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (R.n == 0 || t >= (R.n - 1) * R.len + R.tail) return;
+    const int64_t run = t / R.len, group = run / kMerge;
+    const TopKey me = in[t];
+    // A search is a chain of dependent loads, so all runs of the group are
+    // searched side by side, without branches: a step past a run's end (its own
+    // run counts as empty) looks at the key itself, which is not before it
+    int at[kMerge] = {}, n[kMerge];
+#pragma unroll
+    for (int u = 0; u < kMerge; ++u) {
+        const int64_t j = group * kMerge + u;
+        n[u] = j >= R.n || j == run ? 0 : j == R.n - 1 ? R.tail : R.len;
     }
+    const TopKey* first = in + group * kMerge * R.len;
+    const int own = (int)(run - group * kMerge);
+    for (int step = 1 << (31 - __clz(R.len)); step > 0; step >>= 1) {
+        TopKey o[kMerge];
+#pragma unroll
+        for (int u = 0; u < kMerge; ++u)
+            o[u] = *(at[u] + step <= n[u] ? first + (int64_t)u * R.len + at[u] + step - 1 : in + t);
+#pragma unroll
+        for (int u = 0; u < kMerge; ++u)
+            if ((at[u] + step <= n[u]) & key_before(o[u], me, u < own)) at[u] += step;
+    }
+    int64_t rank = t - run * R.len;
+#pragma unroll
+    for (int u = 0; u < kMerge; ++u) rank += at[u];
+    if (rank < k) out[group * min(k, kMerge * R.len) + rank] = me;
 }
 
 // --------------------------------------------------------- neighbourhood
@@ -471,20 +505,18 @@ namespace {
 // `capacity`); *in_b tells whether the keys are in top_b (else top_a).
 cudaError_t topk(const FrontierDev& F, const FrontierDev* d_fs, int n_f, int64_t capacity, int k, bool* in_b,
                  cudaStream_t s) {
-    // one pass over up to kRankOnce keys; else chunk passes until that fits
-    // (each chunk of at least 4 k keys leaves k)
-    int64_t n_in = capacity;
-    for (int pass = 0;; ++pass) {
-        const bool last = n_in <= kRankOnce;
-        const int64_t chunk = last ? (std::max<int64_t>(n_in, k) + 31) / 32 * 32 : rank_chunk(k);
-        const int64_t chunks = last ? 1 : (n_in + chunk - 1) / chunk;
-        const dim3 grid((unsigned)(chunks * (chunk / 32)), (unsigned)n_f);
-        const cudaError_t e = launch_chained(topk_rank_kernel, grid, 32 * kRankWarps, 0, s, F, d_fs, pass, (int)chunk, k);
-        if (e != cudaSuccess) return e;
+    int64_t runs = (capacity + kRun - 1) / kRun;
+    int len = std::min(k, kRun);
+    *in_b = false;
+    cudaError_t e = launch_chained(topk_rank_kernel, dim3((unsigned)runs, (unsigned)n_f), kRun, 0, s, F, d_fs, k);
+    for (int pass = 1; runs > 1 && e == cudaSuccess; ++pass) {
+        const dim3 grid((unsigned)((runs * len + 255) / 256), (unsigned)n_f);
+        e = launch_chained(topk_merge_kernel, grid, 256, 0, s, F, d_fs, pass, k);
         *in_b = pass & 1;
-        if (last) return cudaSuccess;
-        n_in = chunks * k;
+        runs = (runs + kMerge - 1) / kMerge;
+        len = std::min(k, kMerge * len);
     }
+    return e;
 }
 
 // One expansion round of one frontier (F; batch) or of n_f frontiers (d_fs,

@@ -11,16 +11,27 @@
 
 namespace comet {
 
-constexpr int kChunk = 4096;         // smallest chunk of a top-k pass; the largest k
-constexpr int64_t kRankOnce = 16384;  // keys ranked in one pass
+constexpr int kTopMax = 4096;         // the largest k of a top-k
+constexpr int kRun = 256;             // keys of a run ranked by counting
+constexpr int kMerge = 8;             // runs merged at a time
 constexpr int kScan = 1024;           // slots per block of the compaction
 constexpr int kMaxGridY = 65535;      // frontiers per launch
 
-struct TopKey {
+struct alignas(16) TopKey {
     uint32_t mk;    // order-preserving key of M_hat
     uint32_t idx;   // position of the entry in the ranked array (first pass)
     uint64_t code;  // mode code (tie break)
 };
+
+// Keys that the top-k passes over up to n keys write into top_a (pass 0, and
+// every other one) and top_b, for k up to k_max; callers copy k keys of either.
+inline int64_t top_a_keys(int64_t n, int k_max) {
+    return std::max<int64_t>((n + kRun - 1) / kRun * std::min(k_max, kRun), kTopMax);
+}
+inline int64_t top_b_keys(int64_t n, int k_max) {
+    const int64_t runs = (n + kRun - 1) / kRun;
+    return std::max<int64_t>((runs + kMerge - 1) / kMerge * std::min(k_max, kMerge * kRun), kTopMax);
+}
 
 struct FrontierDev {
     int instance, n_modes, lmax, slots;

@@ -66,7 +66,7 @@ comet_status comet_frontier_create_ex(comet_problem* p, int32_t instance, int64_
     if (!p || !out) return ffail(COMET_ERR_INVALID_ARG, "problem and out are required");
     *out = nullptr;
     if (instance < 0 || instance >= (int)p->inst.size()) return ffail(COMET_ERR_INVALID_ARG, "instance out of range");
-    if (capacity < 1 || batch < 1 || k_max < 1 || k_max > comet::kChunk || batch > capacity)
+    if (capacity < 1 || batch < 1 || k_max < 1 || k_max > comet::kTopMax || batch > capacity)
         return ffail(COMET_ERR_INVALID_ARG, "need 1 <= batch <= capacity and 1 <= k_max <= 4096");
     const comet_instance_desc& d = p->inst[instance];
     if (radius != 1 && radius != 2) return ffail(COMET_ERR_INVALID_ARG, "the edit radius is 1 or 2");
@@ -98,8 +98,6 @@ comet_status comet_frontier_create_ex(comet_problem* p, int32_t instance, int64_
     const uint64_t set_cap = pow2_at_least((uint64_t)capacity * 2);
     const int64_t total = (int64_t)k_max * F.slots;
     const uint64_t cand_cap = pow2_at_least((uint64_t)total * 2);
-    const int64_t chunks = (capacity + comet::kChunk - 1) / comet::kChunk;
-    const int64_t top_n = std::max<int64_t>(chunks * k_max, comet::kChunk);
     // carve one allocation
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -111,8 +109,8 @@ comet_status comet_frontier_create_ex(comet_problem* p, int32_t instance, int64_
     const size_t o_merit = take(sizeof(float) * capacity);
     const size_t o_nV = take(sizeof(unsigned long long));
     const size_t o_set = take(sizeof(unsigned long long) * set_cap);
-    const size_t o_ta = take(sizeof(comet::TopKey) * top_n);
-    const size_t o_tb = take(sizeof(comet::TopKey) * top_n);
+    const size_t o_ta = take(sizeof(comet::TopKey) * comet::top_a_keys(capacity, k_max));
+    const size_t o_tb = take(sizeof(comet::TopKey) * comet::top_b_keys(capacity, k_max));
     const size_t o_cc = take(sizeof(unsigned long long) * total);
     const size_t o_fl = take(sizeof(int) * total);
     const size_t o_ct = take(sizeof(int) * ((total + comet::kScan - 1) / comet::kScan));
@@ -448,7 +446,7 @@ comet_status plan_impl(comet_problem* p, int32_t instance, const comet_mode_seq*
         po = *po_in;
     else
         comet_default_plan_opts(&po);
-    if (po.k < 1 || po.batch < 1 || po.rounds < 0 || po.k_ref < 1 || po.k_ref > comet::kChunk)
+    if (po.k < 1 || po.batch < 1 || po.rounds < 0 || po.k_ref < 1 || po.k_ref > comet::kTopMax)
         return ffail(COMET_ERR_INVALID_ARG, "bad planner options");
     // a graph cannot be captured on the legacy default stream: the planner
     // runs on a private stream ordered after the problem's stream and the
@@ -484,7 +482,7 @@ comet_status plan_impl(comet_problem* p, int32_t instance, const comet_mode_seq*
     const int64_t capacity =
         po.budget > 0 ? std::max<int64_t>(po.budget, n0) : n0 + (int64_t)po.rounds * po.batch;
     const int32_t batch = (int32_t)std::min<int64_t>(po.batch, capacity);
-    if (q && batch > comet::kChunk) return ffail(COMET_ERR_INVALID_ARG, "a learned plan keeps at most 4096 per round");
+    if (q && batch > comet::kTopMax) return ffail(COMET_ERR_INVALID_ARG, "a learned plan keeps at most 4096 per round");
     // with a proposal the frontier's next batch holds the whole neighbourhood
     // of the beam, which the proposal then prunes to `batch`
     const comet_instance_desc& di = p->inst[instance];
@@ -740,9 +738,9 @@ comet_status plan_batch_impl(comet_problem* p, int32_t n_inst, const int32_t* in
         po = *po_in;
     else
         comet_default_plan_opts(&po);
-    if (po.k < 1 || po.batch < 1 || po.rounds < 0 || po.k_ref < 1 || po.k_ref > comet::kChunk)
+    if (po.k < 1 || po.batch < 1 || po.rounds < 0 || po.k_ref < 1 || po.k_ref > comet::kTopMax)
         return ffail(COMET_ERR_INVALID_ARG, "bad planner options");
-    if (q && po.batch > comet::kChunk) return ffail(COMET_ERR_INVALID_ARG, "a learned plan keeps at most 4096 per round");
+    if (q && po.batch > comet::kTopMax) return ffail(COMET_ERR_INVALID_ARG, "a learned plan keeps at most 4096 per round");
     for (int i = 0; i < n_inst; ++i) {
         if (instances[i] < 0 || instances[i] >= (int)p->inst.size())
             return ffail(COMET_ERR_INVALID_ARG, "instance out of range");

@@ -774,8 +774,6 @@ cudaError_t to_device(void* dst, const void* src, size_t bytes, cudaStream_t s) 
 }
 
 cudaError_t ensure_prune(comet_proposal* q, int64_t cap) {
-    // the top-k passes write at most chunks x keep <= chunks x kChunk keys
-    const int64_t chunks = (cap + comet::kChunk - 1) / comet::kChunk;
     if (cap <= q->pr_cap) return cudaSuccess;
     qfree(q, q->pr_seqs);
     qfree(q, q->pr_codes);
@@ -787,9 +785,8 @@ cudaError_t ensure_prune(comet_proposal* q, int64_t cap) {
     if ((e = qalloc(q, &q->pr_seqs, cap)) != cudaSuccess) return e;
     if ((e = qalloc(q, &q->pr_codes, cap)) != cudaSuccess) return e;
     if ((e = qalloc(q, &q->pr_merit, cap)) != cudaSuccess) return e;
-    const int64_t tn = std::max<int64_t>(chunks * comet::kChunk, comet::kChunk);
-    if ((e = qalloc(q, &q->pr_top_a, tn)) != cudaSuccess) return e;
-    if ((e = qalloc(q, &q->pr_top_b, tn)) != cudaSuccess) return e;
+    if ((e = qalloc(q, &q->pr_top_a, comet::top_a_keys(cap, comet::kTopMax))) != cudaSuccess) return e;
+    if ((e = qalloc(q, &q->pr_top_b, comet::top_b_keys(cap, comet::kTopMax))) != cudaSuccess) return e;
     q->pr_cap = cap;
     return cudaSuccess;
 }
@@ -833,7 +830,7 @@ comet_status proposal_prune_device(comet_proposal* q, comet_frontier* f, int kee
 }
 
 comet_status proposal_reserve_prune(comet_proposal* q, int64_t cap, int keep) {
-    if (keep < 1 || keep > kChunk) return qfail(COMET_ERR_INVALID_ARG, "keep must be in [1, 4096]");
+    if (keep < 1 || keep > kTopMax) return qfail(COMET_ERR_INVALID_ARG, "keep must be in [1, 4096]");
     QTRY(ensure_rows(q, cap), "proposal activations");
     QTRY(ensure_prune(q, cap), "prune buffers");
     return COMET_OK;
