@@ -247,14 +247,21 @@ namespace comet {
 // pays once the SMs are full and stay full.  A launch without a queue behind
 // it is bound by its slowest solves instead: there nobody waits for a CTA
 // mate, and while SMs have room, long TOs run one to a CTA, which spreads them
-// over all SMs.  Measured (ms; one to a CTA / four / four in step; N = 80 with
-// 1,824 resident, and mixed orders up to N = 145 with 1,216):
-//   N = 80:  624 TOs  7.2 /  7.3 /  8.8    mixed:  624   8.5 /  9.3 / 11.1
-//          1,400     10.6 / 11.3 / 11.1          1,000  11.5 / 11.4 / 13.1
-//          1,800     12.1 / 11.9 / 12.2          1,400  13.2 / 13.2 / 13.7
-//          2,600     14.5 / 14.9 / 13.7          2,200  16.3 / 15.7 / 15.0
-// and full launches of N = 80 64 / 64 / 54.  At N = 16 (one pass of the stage
-// loops) 144 TOs take 2.0 ms either way.
+// over all SMs.  Measured (ms; one to a CTA / four / four in step), random
+// orders of workloads.push_l4_instance(0) (N = 80, 1,824 resident; the last row
+// all of them) and of the 61 of push_mixed_instance(0..63) with N <= 145 (1,216
+// resident), drawn by numpy's default_rng(n):
+//   N = 80:  624 TOs  7.5 /  8.2 /  8.9    mixed:   624  10.1 / 11.4 / 12.4
+//          1,400     11.4 / 11.9 / 12.0          1,000  11.3 / 11.0 / 12.4
+//          1,800     13.2 / 13.1 / 12.5          1,400  11.7 / 11.7 / 11.5
+//          2,600     16.5 / 16.3 / 15.3          2,200  15.3 / 15.2 / 14.9
+//         20,736     94.7 / 94.1 / 79.4         16,384  60.3 / 60.2 / 55.6
+// At N = 16 (one pass of the stage loops) 150 TOs take 2.0 / 2.0 / 2.3 and
+// 20,000 34.0 / 31.2 / 30.0.  With FP64 refinement (N = 80) 2,600 take 14.5 /
+// 14.2 / 13.9 and 8,192 33.8 / 33.9 / 30.0.  Timing optimisation (N = 80)
+// follows the same rule: 624 TOs take 15.4 / 17.4 / 14.4, 8,192 155 / 155 / 97;
+// between 7/8 and 5/4 of the resident warps it would gain from warps in step
+// already (1,800 TOs 32.0 / 31.9 / 20.9).
 // A shape that the caller set, or that the autotuner is timing, is launched as
 // it is (`exact`): its CTAs hold warps_per_block TOs at any n.
 struct LaunchShape {

@@ -34,7 +34,8 @@
 // 1..6 segments took 213 -> 105 ms, the 507 one-segment orders 25 -> 15 ms.
 // Then the sequential parts: a lane per row and copies ahead in B and the
 // forward chain, two stages side by side and vector records in M: 105 -> 92
-// ms and 15 -> 12.4 ms.  Results are bit-identical throughout.
+// ms and 15 -> 12.4 ms.  Results stayed the same to rounding: most orders bit
+// for bit, isolated entries of mixed-length launches 1e-12 off.
 //
 // What bounds it (2,048 orders, cycles per TO-iteration with 4 CTAs on an
 // SM): M 126 k, B 70 k, A 28 k, C 27 k, trials 23 k.  Issue slots are 27 %
@@ -750,10 +751,10 @@ __device__ BMeasures bphase_a(BCtx& C, float beta, bool update, float beta_old) 
     return m;
 }
 
-// Phase M, a warp per stage: the AL model over (u, x_{k+1}, x_k) from the
+// Phase M, a warp per two stages: the AL model over (u, x_{k+1}, x_k) from the
 // stage's Jacobian record and the elimination of the 12 u columns, a model row
 // per lane in registers; records for the sweep, the gains and the controls.
-// The next stage's record is copied into shared memory meanwhile.
+// The next two records are copied into shared memory meanwhile.
 __device__ void bphase_m(BCtx& C, float beta, float rho) {
     BSmem& S = C.S;
     const BInst<float>& P = C.P;

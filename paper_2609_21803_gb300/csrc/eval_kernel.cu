@@ -63,18 +63,6 @@ __device__ __forceinline__ double warp_max_d(double v) {
     return v;
 }
 
-// The CTA's barrier if `on` (uniform over the launch), as one predicated
-// instruction.
-__device__ __forceinline__ void cta_in_step(int on) {
-    asm volatile(
-        "{\n"
-        ".reg .pred p;\n"
-        "setp.ne.s32 p, %0, 0;\n"
-        "@p bar.sync 0;\n"
-        "}\n" ::"r"(on)
-        : "memory");
-}
-
 // error-free sum a + b = s + e (Knuth two-sum)
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
     s = a + b;
@@ -391,8 +379,8 @@ struct Ctx {
 // a chunk as whole 128-byte lines, phases A and C (32 consecutive stages) as
 // `per` runs of a row, and the chunks of a record are constant offsets apart.
 // In stage order the lanes of phase B read 16 bytes of every per-th place, a
-// sector each: 20,736 orders of N = 80 took 67.0 ms against 64.6 now, 16,384
-// mixed ones (N up to 145) 64.4 against 59.1.
+// sector each: with the kernel otherwise as now, 20,736 orders of N = 80 took
+// 67.0 ms against 64.6, 16,384 mixed ones (N up to 145) 64.4 against 59.1.
 constexpr int kRecRow = 32 * (kRec / 4);  // float4s of one stage of every lane
 
 __device__ __forceinline__ float4* rec_chunk(const Ctx& C, int q, int at) {
@@ -409,9 +397,9 @@ __device__ __forceinline__ int rec_at(const Ctx& C, int k) {
 }
 
 // Record stores carry the persisting (evict-last) L2 priority: the records
-// of all resident warps (about 47 MB at N = 80) fit in L2 and are rewritten
-// every iteration, and with the normal priority they were written back to
-// DRAM at 1.1 GB per 4,096 TOs; with it, 46 MB, at the same speed.
+// of all resident warps (56 MB at N = 80, in rows of 96 stages) fit in L2 and
+// are rewritten every iteration.  With the normal priority a launch of 4,096
+// TOs writes 3.65 GB back to DRAM, with this one 135 MB, at the same speed.
 __device__ __forceinline__ void rec_st(const Ctx& C, int q, int at, float4 v) {
     cuda::annotated_ptr<float4, cuda::access_property::persisting> p(rec_chunk(C, q, at));
     *p = v;
@@ -1433,10 +1421,12 @@ __device__ void refine_step(Ctx& C, float beta, float rho, bool curvature) {
 // places of a 96-128 KB loop reach 0.33-0.38 issues per cycle and quarter,
 // 12 warps in step 0.91, as a fetched line then serves all of them).  In step
 // at the trip's start, the warps stay close enough to share most fetches:
-// 20,736 TOs at N = 80 took 76.6 ms without and 63.5 ms with the barrier, with
-// equal results (no_instruction stalls per issue 3.2 -> 0.75); a second
-// barrier before phase B gained nothing, and 2 or 12 warps per CTA took 12 %
-// longer than 4.  Launches that do not fill the SMs skip it (in_step = 0).
+// 20,736 TOs at N = 80 (all four-segment orders of one instance) take 94.2 ms
+// without and 79.5 ms with the barrier, with equal results (no_instruction
+// stalls per issue 3.2 -> 0.75 when it came); a second barrier before phase B
+// gained nothing, and 2 or 12 warps per CTA took 12 % longer than 4.  Launches
+// of at most 5/4 of the resident warps skip it (in_step = 0; launch_shape in
+// api.cu).
 // A warp that runs out of TOs leaves; a barrier waits only for warps that
 // have not left.
 // kUnr: stages per trip of the stage-parallel loops (phases A, C and D
@@ -1706,8 +1696,8 @@ int eval_blocks_per_sm(int warps_per_block, size_t smem_per_block) {
 
 cudaError_t launch_eval(const EvalArgs& a, int total_warps, int warps_per_block, cudaStream_t s) {
     const size_t smem = smem_per_warp_bytes(a.Nmax) * warps_per_block;
-    // not a stream operation, so raising it outside of a capture keeps
-    // launches capturable (problem creation raises it first)
+    // the shared-memory limit (problem creation raises it first; it is not a
+    // stream operation, so a launch that finds it too low can be captured)
     const cudaError_t e = g_smem_limit.raise(smem, set_smem_all);
     if (e != cudaSuccess) return e;
     const int blocks = (total_warps + warps_per_block - 1) / warps_per_block;

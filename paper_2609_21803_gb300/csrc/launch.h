@@ -44,13 +44,26 @@ cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t s
     return e;
 }
 
+// The CTA's barrier if `on` (uniform over the launch), as one predicated
+// instruction: the persistent evaluators' warps in step.
+__device__ __forceinline__ void cta_in_step(int on) {
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        "setp.ne.s32 p, %0, 0;\n"
+        "@p bar.sync 0;\n"
+        "}\n" ::"r"(on)
+        : "memory");
+}
+
 // Launch of a persistent evaluator, whose CTAs are all resident: the SM's
 // on-chip memory is split between shared memory and L1 by what this launch
 // puts on an SM, not by what the kernel's occupancy would allow (the default).
 // Stage records come back through L1, and a launch that leaves SMs partly idle
 // is bound by the latency of its slowest solves: 624 mixed pushing orders (N up
-// to 145, a warp per CTA) take 10.3 ms with the default split (28 KB of L1),
-// 8.4 with this one, 150 orders 9.6 and 7.9; full launches keep their split.
+// to 145, a warp per CTA; the orders of launch_shape's table in api.cu) take
+// 12.2 ms with the default split (28 KB of L1), 10.1 with this one, 150 orders
+// 9.3 and 7.6; full launches keep their split.
 // Shared memory keeps at least 44 % (100 KB), so that another stream's CTAs
 // still fit beside a small launch; without that floor the times are the same.
 template <class K, class A>

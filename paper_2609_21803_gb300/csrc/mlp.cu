@@ -381,8 +381,9 @@ int grid_for(int64_t work, int threads = 256) {
     return (int)std::max<int64_t>(1, std::min<int64_t>((work + threads - 1) / threads, 152 * 16));
 }
 
-// The same with an Euler rollout of the pusher-slider model from the start
-// pose (warm_mode 0, pushing; s_0 = 0, s reset to 0 after a face change): a
+// merit = exp(y_0) and the warm start of order i (as predict_post_kernel below)
+// with an Euler rollout of the pusher-slider model from the start pose for its
+// poses (warm_mode 0, pushing; s_0 = 0, s reset to 0 after a face change): a
 // chain over the knots, so a thread takes a whole order.
 __global__ void predict_rollout_kernel(const float* Y, int out_dim, const comet_mode_seq* seqs, const int* row_of,
                                        int64_t n_rows, const int64_t* d_n, const comet::DevInstance* inst, int n_inst,

@@ -88,18 +88,6 @@ __device__ __forceinline__ double twarp_max_d(double v) {
     return v;
 }
 
-// the CTA's barrier if `on` (uniform over the launch), as one predicated
-// instruction
-__device__ __forceinline__ void cta_in_step(int on) {
-    asm volatile(
-        "{\n"
-        ".reg .pred p;\n"
-        "setp.ne.s32 p, %0, 0;\n"
-        "@p bar.sync 0;\n"
-        "}\n" ::"r"(on)
-        : "memory");
-}
-
 // error-free sum a + b = s + e (Knuth two-sum)
 __device__ __forceinline__ void two_sum_t(float a, float b, float& s, float& e) {
     s = a + b;
@@ -707,7 +695,7 @@ __device__ __forceinline__ void tload_elem(const TCtx& C, int k, int at, float e
 
 // Eliminate the node shared by e (over (y = m, x = a)) and f (over (y = b,
 // x = m)); e becomes the element over (y = b, x = a).  Stores node m's
-// (L, Y) in record `km` when `store`; false on a non-positive pivot.
+// (L, Y) in the record at `at` when `store`; false on a non-positive pivot.
 __device__ __forceinline__ bool tcombine(const TCtx& C, float e[kTElem], const float f[kTElem], int at, bool store) {
     float L[15];
 #pragma unroll
