@@ -153,11 +153,13 @@ __global__ void add_many_kernel(const FrontierDev* Fs, const comet_mode_seq* seq
 // to 16,384; before that, chunks of 4,096 were sorted in a CTA each (78
 // barriers, 80 us however small the set).  A comet_frontier_best call, which
 // copies k keys back and waits (us: sorted chunks / counted chunks / now):
-//      n = 8,000  k = 64     249 /   65 /  46    k = 2,048   254 /   67 /  60
-//         20,736             249 /   69 /  55                480 /  127 /  83
-//        105,000             251 /  164 /  69                699 /  403 / 109
-//        420,000             357 /  537 / 108                921 / 1329 / 222
-//      1,048,576             454 / 1321 / 193               1131 / 3173 / 438
+//      n = 8,000  k = 64     249 /   65 /  45    k = 2,048   254 /   67 /  57
+//         20,736             249 /   69 /  55                480 /  127 /  76
+//        105,000             251 /  164 /  58                699 /  403 / 101
+//        420,000             357 /  537 /  86                921 / 1329 / 197
+//      1,048,576             454 / 1321 / 135               1131 / 3173 / 385
+// Runs of 128 keys and merges of 8 are as good; runs of 512 take 49 us at 8,000
+// keys and 108 at 420,000 (k = 64), merges of 16 more everywhere.
 struct Runs {
     int64_t n;      // sorted runs, one after the other
     int len, tail;  // length of every run but the last, and of the last
@@ -192,23 +194,35 @@ __device__ __forceinline__ int64_t keys_of(const FrontierDev& F) {
 __global__ void __launch_bounds__(kRun) topk_rank_kernel(FrontierDev F0, const FrontierDev* Fs, int k) {
     launch_next();
     await_previous();
-    __shared__ TopKey run[kRun];
+    // merit keys apart from the codes: four a load, and codes only for a tie
+    __shared__ __align__(16) uint32_t mk[kRun];
+    __shared__ unsigned long long code[kRun];
     const FrontierDev F = Fs ? Fs[blockIdx.y] : F0;
     const int64_t base = (int64_t)blockIdx.x * kRun;
     const int len = (int)min((int64_t)kRun, keys_of(F) - base), i = threadIdx.x;
     if (len <= 0) return;
     TopKey me;
+    me.mk = 0xffffffffu;  // past the end: before no key
+    me.idx = (uint32_t)(base + i);
+    me.code = ~0ull;
     if (i < len) {
         me.mk = float_key(F.merit[base + i]);
-        me.idx = (uint32_t)(base + i);
         me.code = F.codes[base + i];
-        run[i] = me;
     }
+    mk[i] = me.mk;
+    code[i] = me.code;
     __syncthreads();
     if (i >= len) return;
-    int rank = 0;
-#pragma unroll 4
-    for (int j = 0; j < len; ++j) rank += key_before(run[j], me, j < i);
+    int rank = 0, same = 0;
+#pragma unroll 8
+    for (int j = 0; j < kRun; j += 4) {
+        const uint4 o = *reinterpret_cast<const uint4*>(mk + j);
+        rank += (o.x < me.mk) + (o.y < me.mk) + (o.z < me.mk) + (o.w < me.mk);
+        same += (o.x == me.mk) + (o.y == me.mk) + (o.z == me.mk) + (o.w == me.mk);
+    }
+    if (same > 1)
+        for (int j = 0; j < len; ++j)
+            rank += mk[j] == me.mk && (code[j] < me.code || (code[j] == me.code && j < i));
     if (rank < k) F.top_a[blockIdx.x * (int64_t)min(k, kRun) + rank] = me;
 }
 
