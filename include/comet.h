@@ -395,7 +395,7 @@ comet_status comet_set_launch_config(comet_problem* p, const comet_launch_config
  * -- 1..4 TOs per CTA, each at its occupancy limit and at three quarters of
  * it, each with the stage loops unrolled 1 and 2 times -- and keeps the
  * fastest for p.  The sample should be as large as the launches to come: if it
- * exceeds 5/4 of the resident warps of every candidate (1,824 warps at N_max =
+ * exceeds twice the resident warps of every candidate (1,824 warps at N_max =
  * 80), the pick is for launches that fill the SMs (smaller ones follow the
  * rule above) and is cached per (device, N_max) for problems created later in
  * the process; a smaller sample's pick stays with p, as if it had been set.

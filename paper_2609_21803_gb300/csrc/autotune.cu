@@ -2,12 +2,14 @@
 // warp per TO, 1..4), resident CTAs per SM and the unrolling of the stage
 // loops (1 or 2 stages per trip).  comet_autotune times the evaluator on a
 // sample of the caller's orders under every candidate shape and keeps the
-// fastest.  A pick timed on more than 5/4 of the resident warps of every
+// fastest.  A pick timed on more than twice the resident warps of every
 // candidate holds for launches that fill the SMs, whose CTAs run in step (see
 // launch_shape in api.cu): it is cached per (device, N_max) for the process,
 // and problems created later with the same key start from it.  A pick timed on
-// fewer orders says nothing about those: it stays with its problem, whose
-// launches then run it at every size.
+// fewer orders says little about those (1,920 orders at N_max = 174, 1.4 to 2.1
+// times the candidates' resident warps: 3.20 ms with one TO per CTA and 3.23
+// with two, which rounds of 262,144 slots run 10 % faster): it stays with its
+// problem, whose launches then run it at every size.
 //
 // Every (TOs per CTA, CTAs per SM) shape solves each TO in one warp with the
 // same arithmetic, so the results do not depend on it, only the time does;
@@ -144,7 +146,7 @@ comet_status comet_autotune(comet_problem* p, const comet_mode_seq* sample, int6
     const bool x0 = p->shape_exact;
     p->shape_exact = true;  // time each candidate as it is
     bool full = true;
-    for (const Shape& c : cand) full = full && 4 * n > 5 * (int64_t)p->num_sms * c.bps * c.wpb;
+    for (const Shape& c : cand) full = full && n > 2 * (int64_t)p->num_sms * c.bps * c.wpb;
     float best_ms = 0.f;
     int best = -1;
     comet_status st = COMET_OK;
